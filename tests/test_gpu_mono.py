@@ -86,6 +86,25 @@ def test_m256_cluster_of_four_bands(scales, weights, k):
     check(B, scales, weights, k)
 
 
+@pytest.mark.parametrize("M,J", [(64, 1), (64, 12), (64, 20), (128, 1), (128, 40), (128, 64), (256, 3), (256, 21),
+                                 (256, 22), (256, 64)])
+def test_walk_groups_and_tables(M, J):
+    """The strip kernels (M = 64, 128, 256) on both sides of the spectrum sizes whose fraction tables fit in
+    shared memory, with scales at the edges of their sample groups: below 1 (samples leave the grid, rows
+    advance by more than one), exactly 1, just above 1 and about 2 (groups of 1 | 2 | 3 sources), 2.5."""
+    edges = [1.0, 0.35, 0.9995, 1.0005, 1.5, 1.9985, 2.0, 2.001, 2.5, 0.999, 4.0 / 3.0, 0.6]
+    rng = np.random.default_rng(1000 * M + J)
+    scales = [edges[j] if j < len(edges) else float(rng.uniform(0.5, 2.5)) for j in range(J)]
+    B = rng.uniform(0.0, 1e3, size=(2, M, M)).astype(np.float32).astype(np.float64)
+    weights = rng.uniform(0.1, 1.0, J)
+    Xg, Rg = run_gpu(B, scales, weights, 2)
+    Xo, Ro = mono.monochromatise(B, scales, weights, 2)
+    for n in range(B.shape[0]):
+        # residual norms against ||b||: with the one scale 1 the residual itself vanishes after one step
+        assert np.linalg.norm(Xg[n] - Xo[n]) <= TOL * np.linalg.norm(Xo[n]), n
+        assert np.max(np.abs(Rg[n] - Ro[n])) <= TOL * Ro[n][0], n
+
+
 def test_monochromatic_light_is_exact_and_clamp():
     rng = np.random.default_rng(3)
     B = rng.standard_normal((3, 32, 32)).astype(np.float32).astype(np.float64)
