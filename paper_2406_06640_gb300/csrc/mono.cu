@@ -385,7 +385,8 @@ struct WalkShape {
   static constexpr size_t TAB = AXES * TAB_S + (QUAD_ ? align16((size_t)TILE + 2) : 0);
   static constexpr size_t FIXED = P_BYTES + 2 * R_BYTES + RED_BYTES + SPEC_BYTES + HALO_BYTES;
   static constexpr size_t TAB_F = (size_t)AXES * TILE * 4;
-  static constexpr size_t bytes(int J, bool ft) { return FIXED + (size_t)J * (TAB + (ft ? TAB_F : 0)); }
+  // (16 bytes behind the tables: a walk loads one source ahead)
+  static constexpr size_t bytes(int J, bool ft) { return FIXED + (size_t)J * (TAB + (ft ? TAB_F : 0)) + 16; }
   static constexpr size_t LIMIT = MIN_BLOCKS == 1 ? 232448 : 233472 / MIN_BLOCKS - 1024;  // of one CTA
   static_assert(TILE % 64 == 0 && TPB % 32 == 0 && TPB > TILE, "strips, a thread per halo element");
   static_assert(bytes(kMonoMaxJ, false) <= 232448, "shared memory of one CTA");
@@ -401,21 +402,39 @@ struct WalkAxis {
   const float* f;  // fractions of the tile's samples (with tables)
 };
 
-// source k (tile frame) of the group of output u, for two lines: v += (1 - f) r, b += f r with f = its
-// position - u, from the table x.f (FT) or the running index kc = its index - c; then the next source
+// walks the sources of two lines in order, each loaded one step before it is used (the uniform branches
+// of a walk keep the compiler from moving a load ahead of the one that decides about it)
 template <int ES, int LINE2, bool FT>
-__device__ __forceinline__ void take_source(const unsigned char* line, const WalkAxis& x, float u, int& k, float& kc,
-                                            float (&v)[2], float (&b)[2]) {
-  const float f = FT ? x.f[k] : fmaf(kc, x.inv_a, x.c) - u, g = 1.f - f;
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const float r = *reinterpret_cast<const float*>(line + k * ES + h * LINE2);
-    v[h] = fmaf(g, r, v[h]);
-    b[h] = fmaf(f, r, b[h]);
+struct Sources {
+  const unsigned char* line;
+  const WalkAxis& x;
+  int k;       // the next source (tile frame)
+  float kc;    // its index - c
+  float f, r[2];
+  __device__ __forceinline__ Sources(const unsigned char* l, const WalkAxis& ax, int first)
+      : line(l), x(ax), k(first), kc((float)(ax.o + first) - ax.c) {
+    load();
   }
-  ++k;
-  kc += 1.f;
-}
+  // (the load after a line's last source reads the padding behind it and is not used)
+  __device__ __forceinline__ void load() {
+    if constexpr (FT) f = x.f[k];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) r[h] = *reinterpret_cast<const float*>(line + k * ES + h * LINE2);
+  }
+  // the next source, of the group of output u: v += (1 - f) r, b += f r with f = its position - u, from
+  // the table x.f (FT) or the running index
+  __device__ __forceinline__ void take(float u, float (&v)[2], float (&b)[2]) {
+    const float ft = FT ? f : fmaf(kc, x.inv_a, x.c) - u, g = 1.f - ft;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      v[h] = fmaf(g, r[h], v[h]);
+      b[h] = fmaf(ft, r[h], b[h]);
+    }
+    ++k;
+    kc += 1.f;
+    load();
+  }
+};
 
 // the transposed interpolation of one strip of two lines, outputs u0 .. (ES bytes between samples, the
 // second line LINE2 bytes after the first), groups of at most GM sources. st = (., ., first source of the
@@ -426,24 +445,23 @@ __device__ __forceinline__ void adjoint_walk(const unsigned char* line, const Wa
                                              float (&last)[2], Sink sink) {
   const int z = warp_uniform(st.z), w = warp_uniform(st.w);
   const int before = (z >> 8) & 3;
-  int k = z & 0xff;
-  float kc = (float)(x.o + k) - x.c;
+  Sources<ES, LINE2, FT> src(line, x, z & 0xff);
   const float uf = (float)(x.o + u0);
   float prev[2] = {0.f, 0.f};
   {
     float unused[2] = {0.f, 0.f};
 #pragma unroll
     for (int l = 0; l < GM; ++l)
-      if (before > l) take_source<ES, LINE2, FT>(line, x, uf - 1.f, k, kc, unused, prev);
+      if (before > l) src.take(uf - 1.f, unused, prev);
   }
 #pragma unroll
   for (int i = 0; i < STRIP; ++i) {
     float v[2] = {prev[0], prev[1]};
     prev[0] = prev[1] = 0.f;
     const float u = uf + (float)i;
-    if (w & (1 << i)) take_source<ES, LINE2, FT>(line, x, u, k, kc, v, prev);
-    if (GM > 1 && (w & (1 << (16 + i)))) take_source<ES, LINE2, FT>(line, x, u, k, kc, v, prev);
-    if (GM > 2 && (z & (1 << (16 + i)))) take_source<ES, LINE2, FT>(line, x, u, k, kc, v, prev);
+    if (w & (1 << i)) src.take(u, v, prev);
+    if (GM > 1 && (w & (1 << (16 + i)))) src.take(u, v, prev);
+    if (GM > 2 && (z & (1 << (16 + i)))) src.take(u, v, prev);
     sink(i, v);
   }
   last[0] = prev[0];
@@ -674,7 +692,7 @@ __global__ void __launch_bounds__(WalkShape<TILE, QUAD>::TPB, WalkShape<TILE, QU
       const int mask = warp_uniform(st.y), x = warp_uniform(st.x);
       int off = (x - 1) * (LDP * 4);  // of row i0 - 1, i0 the sample row
       float yc = (float)(oy + u0) - c, i0f = (float)(oy + x - 2);
-      float fx[2], gx[2], top[2] = {0.f, 0.f}, bot[2] = {0.f, 0.f};
+      float fx[2], gx[2], top[2] = {0.f, 0.f}, bot[2] = {0.f, 0.f}, nx[2][2] = {};
       const float4* f4 = reinterpret_cast<const float4*>(tab_f(j, 0) + (FT ? u0 : 0));
       float4 fr = make_float4(0.f, 0.f, 0.f, 0.f);
       // the two columns' samples; w_j goes into their weights
@@ -709,12 +727,18 @@ __global__ void __launch_bounds__(WalkShape<TILE, QUAD>::TPB, WalkShape<TILE, QU
             for (int h = 0; h < 2; ++h) {
               const float* p = reinterpret_cast<const float*>(q[h] + off);
               top[h] = fmaf(fx[h], p[1], gx[h] * p[0]);
+              nx[h][0] = p[LDP];
+              nx[h][1] = p[LDP + 1];
             }
           }
+          // the row after next is loaded one step ahead of its use (past the tile's last row it reads
+          // what lies behind p and is not used)
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
-            const float* p = reinterpret_cast<const float*>(q[h] + off) + LDP;
-            bot[h] = fmaf(fx[h], p[1], gx[h] * p[0]);
+            const float* p = reinterpret_cast<const float*>(q[h] + off) + 2 * LDP;
+            bot[h] = fmaf(fx[h], nx[h][1], gx[h] * nx[h][0]);
+            nx[h][0] = p[0];
+            nx[h][1] = p[1];
           }
         }
         if (FT && i % 4 == 0) fr = f4[i / 4];
