@@ -102,6 +102,10 @@ static std::vector<int> philox_permutation(int n, uint64_t seed, uint32_t stream
   return a;
 }
 
+// pc-DM: groups of positions the probe sums are split into. 32 groups of M^2 / 512 blocks fill the GPU at
+// M = 128 while their partials (32 K M^2 complex) stay small beside the state they are summed from
+constexpr int kDmParts = 32;
+
 struct ptycho_plan_s {
   ptycho_params p{};
   std::vector<int32_t> windows;
@@ -404,7 +408,7 @@ static ptycho_status build_plan(ptycho_plan_s* pl, const float* intensities, con
     int max_slots = 0;
     if (p.engine == PTYCHO_ENGINE_DM) {
       PT_CUDA(fused_dm_max_slots(M, K, &max_slots), "occupancy of the pc-DM kernel");
-      if (max_slots < 1) return fail(PTYCHO_EUNSUPPORTED, "a cluster of K CTAs does not fit on this device");
+      if (max_slots < 1) return fail(PTYCHO_EUNSUPPORTED, "the pc-DM kernel does not fit on this device");
     } else {
       PT_CUDA(fused_max_slots(M, K, &max_slots), "occupancy of the fused kernel");
       if (max_slots < 1) return fail(PTYCHO_EUNSUPPORTED, "the fused kernel does not fit on this device");
@@ -480,8 +484,11 @@ static ptycho_status build_plan(ptycho_plan_s* pl, const float* intensities, con
   float* d_dacc;
   double* d_errpart;
   PT_CUDA(pl->alloc(&d_cn, (size_t)N * MM), "alloc contributions");
-  PT_CUDA(pl->alloc(&d_pacc, (size_t)pl->slots * K * MM), "alloc probe partials");
-  PT_CUDA(pl->alloc(&d_dacc, (size_t)pl->slots * MM), "alloc probe partials");
+  // probe partials: one per slot, or (pc-DM, whose probe sums are a pass of their own over the state)
+  // one per group of positions
+  const int parts = p.engine == PTYCHO_ENGINE_DM ? std::min(N, kDmParts) : pl->slots;
+  PT_CUDA(pl->alloc(&d_pacc, (size_t)parts * K * MM), "alloc probe partials");
+  PT_CUDA(pl->alloc(&d_dacc, (size_t)parts * MM), "alloc probe partials");
   const size_t nerr = pl->big ? (size_t)N * big_row_blocks(M) : (size_t)pl->slots * K;
   PT_CUDA(pl->alloc(&d_errpart, nerr), "alloc error partials");
   float2* d_W = nullptr;
@@ -583,7 +590,7 @@ static ptycho_status build_plan(ptycho_plan_s* pl, const float* intensities, con
   ua.M = M;
   ua.obj_h = p.obj_h;
   ua.obj_w = p.obj_w;
-  ua.slots = pl->slots;
+  ua.slots = parts;
   ua.cn = d_cn;
   ua.pacc = d_pacc;
   ua.dacc = d_dacc;
@@ -668,7 +675,7 @@ static ptycho_status build_plan(ptycho_plan_s* pl, const float* intensities, con
     }
     pl->chunk = std::min(c, pl->chunk);  // a chunk holds at most N positions; buffers hold the largest
     pl->slots = pl->chunk;
-    pl->ua.slots = pl->chunk;
+    if (p.engine != PTYCHO_ENGINE_DM) pl->ua.slots = pl->chunk;
   }
   return PTYCHO_OK;
 }

@@ -14,7 +14,7 @@ constexpr int kMaxModes = 8;        // probe modes K handled (one cluster rank p
 constexpr int kObjSplit = 8;        // position groups per object tile (one cluster, fixed order)
 constexpr int kErrHistory = 4096;   // ring of per-iteration errors kept on the device
 
-// Arguments of the fused per-position kernel (one cluster of K CTAs per position).
+// Arguments of the fused per-position kernels.
 struct FusedArgs {
   const float2* O;      // object, obj_h x obj_w, row-major
   const float2* P;      // probe modes, K x M x M
@@ -46,7 +46,7 @@ struct FusedArgs {
   int dm_init;
 };
 
-// single-problem fused launch (pc_fused_seq.cu: one CTA per position, modes in sequence) over
+// single-problem fused launch (pc_fused_seq.cuh: one CTA per position, modes in sequence) over
 // `slots` persistent CTAs; fused_max_slots gives the co-resident CTAs of the GPU. Partials: pacc
 // slots x K x M x M, dacc slots x M x M, errpart slots x K (the slot's error in entry 0)
 cudaError_t launch_fused(int M, const FusedArgs& a, int slots, cudaStream_t s);
@@ -55,14 +55,14 @@ cudaError_t fused_max_slots(int M, int K, int* slots);
 // as launch_fused (errpart slots x K, one entry per rank)
 cudaError_t launch_fused_cluster(int M, const FusedArgs& a, int slots, cudaStream_t s);
 cudaError_t fused_cluster_max_slots(int M, int K, int* slots);
-// work-queue launch (M = 32, 64, 128): `slots` persistent clusters drain a.chunks through a.queue;
+// work-queue launch: `slots` persistent CTAs drain a.chunks through a.queue;
 // a.K, a.near_field, a.kh (kernel width class) and a.tw are those of every problem in a.probs
 cudaError_t launch_fused_queue(int M, const FusedArgs& a, int slots, cudaStream_t s);
 cudaError_t fused_queue_max_slots(int M, int K, int* slots);
-// pc-DM launch (single problem, M <= 128): as launch_fused with the exit-wave state a.psi
+// pc-DM launch (single problem, M <= 128): as launch_fused with the exit-wave state a.psi and no probe
+// partials
 cudaError_t launch_fused_dm(int M, const FusedArgs& a, int slots, cudaStream_t s);
 cudaError_t fused_dm_max_slots(int M, int K, int* slots);
-cudaError_t fused_dm_timed_out(bool* out);
 bool fused_queue_supported(int M);
 size_t fused_smem_bytes(int M);
 // true if a bounded device wait of the fused kernel gave up since the last call (clears the flag; synchronous)

@@ -1,7 +1,6 @@
-// Fused per-position pc-engine kernel in its cluster form, used by the work-queue launches of
-// batch plans and by mini-batches too small to fill the GPU with one CTA per position (the
-// single-problem launch runs the one-CTA-per-position kernel of pc_fused_seq.cu):
-// one cluster of K CTAs per scan position,
+// Fused per-position pc-engine kernel in its cluster form, used by mini-batches too small to fill the
+// GPU with one CTA per position (every other launch runs the one-CTA-per-position kernel of
+// pc_fused_seq.cuh): one cluster of K CTAs per scan position,
 // CTA rank k owns probe mode k and rows [k R, (k + 1) R) of the detector
 // (R = ceil(M / K)). Everything between the object gather and the per-position
 // contributions stays on chip:
@@ -60,10 +59,8 @@ cudaError_t fused_timed_out(bool* out) {
     e = cudaMemcpyToSymbol(g_fused_timeout, &z, sizeof(int));
     if (e != cudaSuccess) return e;
   }
-  bool dm = false;
-  e = fused_dm_timed_out(&dm);  // the pc-DM instantiations keep their own flag
-  *out = h != 0 || dm;
-  return e;
+  *out = h != 0;
+  return cudaSuccess;
 }
 
 size_t fused_smem_bytes(int M) {
@@ -77,12 +74,12 @@ size_t fused_smem_bytes(int M) {
   }
 }
 
-template <int M, int KH, bool QUEUED = false>
+template <int M, int KH>
 static cudaLaunchConfig_t fused_config(const FusedArgs& a, int slots, cudaStream_t s, cudaLaunchAttribute* attr) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(slots * a.K));
   cfg.blockDim = dim3(FusedShape<M>::TR);
-  cfg.dynamicSmemBytes = FusedSmem<M, KH>::BYTES + (QUEUED ? FusedSmem<M, KH>::DESC : 0);
+  cfg.dynamicSmemBytes = FusedSmem<M, KH>::BYTES;
   cfg.stream = s;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned)a.K;
@@ -93,14 +90,13 @@ static cudaLaunchConfig_t fused_config(const FusedArgs& a, int slots, cudaStream
   return cfg;
 }
 
-template <int M, bool NEAR, int KH, bool QUEUED = false>
+template <int M, bool NEAR, int KH>
 static cudaError_t launch_kh(const FusedArgs& a, int slots, cudaStream_t s) {
-  auto kern = pc_fused_kernel<M, NEAR, KH, QUEUED>;
-  const size_t bytes = FusedSmem<M, KH>::BYTES + (QUEUED ? FusedSmem<M, KH>::DESC : 0);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  auto kern = pc_fused_kernel<M, NEAR, KH>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FusedSmem<M, KH>::BYTES);
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = fused_config<M, KH, QUEUED>(a, slots, s, attr);
+  cudaLaunchConfig_t cfg = fused_config<M, KH>(a, slots, s, attr);
   return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
@@ -125,7 +121,7 @@ cudaError_t launch_fused_cluster(int M, const FusedArgs& a, int slots, cudaStrea
 
 template <int M>
 static cudaError_t cluster_slots_t(int K, int* slots) {
-  auto kern = pc_fused_kernel<M, false, 15, false>;
+  auto kern = pc_fused_kernel<M, false, 15>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FusedSmem<M, 15>::BYTES);
   if (e != cudaSuccess) return e;
   FusedArgs a = {};
@@ -145,54 +141,6 @@ cudaError_t fused_cluster_max_slots(int M, int K, int* slots) {
     case 32: return cluster_slots_t<32>(K, slots);
     case 64: return cluster_slots_t<64>(K, slots);
     case 128: return cluster_slots_t<128>(K, slots);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-// ---- work-queue launches (batches of problems sharing M, K, geometry and kernel width class)
-template <int M, bool NEAR>
-static cudaError_t launch_queue_t(const FusedArgs& a, int slots, cudaStream_t s) {
-  return a.kh == 5 ? launch_kh<M, NEAR, 5, true>(a, slots, s) : launch_kh<M, NEAR, 15, true>(a, slots, s);
-}
-
-bool fused_queue_supported(int M) { return M == 8 || M == 16 || M == 32 || M == 64 || M == 128; }
-
-cudaError_t launch_fused_queue(int M, const FusedArgs& a, int slots, cudaStream_t s) {
-  if (!a.probs || !a.chunks || !a.queue || a.nchunks < 0) return cudaErrorInvalidValue;
-  const bool nf = a.near_field != 0;
-  switch (M) {
-    case 8: return nf ? launch_queue_t<8, true>(a, slots, s) : launch_queue_t<8, false>(a, slots, s);
-    case 16: return nf ? launch_queue_t<16, true>(a, slots, s) : launch_queue_t<16, false>(a, slots, s);
-    case 32: return nf ? launch_queue_t<32, true>(a, slots, s) : launch_queue_t<32, false>(a, slots, s);
-    case 64: return nf ? launch_queue_t<64, true>(a, slots, s) : launch_queue_t<64, false>(a, slots, s);
-    case 128: return nf ? launch_queue_t<128, true>(a, slots, s) : launch_queue_t<128, false>(a, slots, s);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-template <int M>
-static cudaError_t queue_slots_t(int K, int* slots) {
-  auto kern = pc_fused_kernel<M, false, 15, true>;
-  const size_t bytes = FusedSmem<M, 15>::BYTES + FusedSmem<M, 15>::DESC;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e != cudaSuccess) return e;
-  FusedArgs a = {};
-  a.K = K;
-  cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = fused_config<M, 15, true>(a, 1, 0, attr);
-  int n = 0;
-  e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
-  *slots = n;
-  return e;
-}
-
-cudaError_t fused_queue_max_slots(int M, int K, int* slots) {
-  switch (M) {
-    case 8: return queue_slots_t<8>(K, slots);
-    case 16: return queue_slots_t<16>(K, slots);
-    case 32: return queue_slots_t<32>(K, slots);
-    case 64: return queue_slots_t<64>(K, slots);
-    case 128: return queue_slots_t<128>(K, slots);
     default: return cudaErrorInvalidValue;
   }
 }

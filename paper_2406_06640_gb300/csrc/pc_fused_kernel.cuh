@@ -1,6 +1,5 @@
-// Device code of the fused per-position kernel (see pc_fused.cu for what it computes); included by
-// the translation units that instantiate it (pc_fused.cu: single-problem and work-queue launches;
-// pc_fused_dm.cu: the pc-DM engine).
+// Device code of the cluster form of the fused per-position kernel (see pc_fused.cu for what it computes
+// and when it runs).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -21,8 +20,7 @@ __device__ __forceinline__ void red_add_l2(float* a, float v) {
   asm volatile("red.global.add.f32 [%0], %1;" ::"l"(a), "f"(v));
 }
 
-// set when a bounded device wait of the fused kernel gave up (one flag per translation unit that
-// instantiates the kernel; read and cleared by fused_timed_out)
+// set when a bounded device wait of the fused kernel gave up (read and cleared by fused_timed_out)
 static __device__ int g_fused_timeout;
 
 // ---- bounded mbarrier wait (global timer); false once `budget_ns` has passed without the phase
@@ -68,9 +66,7 @@ struct FusedSmem {
   static constexpr size_t HQ = (size_t)M * 8;                                             // Fresnel factors
   static constexpr size_t TAPS = 2 * kMaxTaps * 4 + 8 + 16;  // taps, TMEM address, mbarrier (16-byte aligned)
   static constexpr size_t BYTES = CBUF + IBUF + TWT + HQ + TAPS;
-  // queued launches: the current problem's arguments and the chunk index handed out by rank 0
-  static constexpr size_t DESC = (sizeof(FusedArgs) + 15) / 16 * 16 + 16;
-  static_assert(BYTES + DESC <= 232448, "shared memory budget of one CTA");
+  static_assert(BYTES <= 232448, "shared memory budget of one CTA");
 };
 
 // lines per thread: the 128 x 128 tile runs on 512 threads with two lines each
@@ -88,7 +84,7 @@ struct FusedShape {
                 "TMEM allocation must be a power of two in [32, 512] columns");
 };
 
-template <int M, bool NEAR, int KH, bool QUEUED, bool DM = false>
+template <int M, bool NEAR, int KH>
 __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const FusedArgs a_in) {
   using TL = Tile<M>;
   using SM = FusedSmem<M, KH>;
@@ -190,17 +186,12 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
   auto run_position = [&](const FusedArgs& a, int n, bool first, float2* pacc, float* dacc) {
     const float2* Pk = a.P + (size_t)rank * M * M;
     const float eps = a.eps;
-    // pc-DM: this position's exit-wave state of mode `rank` (P o_n itself when the state starts)
-    float2* Sn = DM ? a.psi + ((size_t)n * K + rank) * M * M : nullptr;
-    const bool dm_init = DM && a.dm_init;
     const int2 pn = a.pos[n];
     const float2* On = a.O + (size_t)pn.x * a.obj_w + pn.y;
     float2 v[V][E];
 
-    // ---- exit wave in ROW layout: P o_n, or (pc-DM, CHI) the reflected wave 2 P o_n - psi_n;
-    // far field: times (-1)^(y + x), which centres the transform
-    auto exit_wave = [&](auto chi_c) {
-      constexpr bool CHI = decltype(chi_c)::value != 0;
+    // ---- exit wave P o_n in ROW layout; far field: times (-1)^(y + x), which centres the transform
+    auto exit_wave = [&]() {
       if constexpr (TM) {
         // every object load of this thread in flight at once (the TMEM waits below are compiler
         // barriers: loads issued after them would expose one L2 round trip per group)
@@ -219,10 +210,6 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
             for (int jj = 0; jj < 4; ++jj) {
               const int x = tp[q] + G * (4 * h + jj);
               float2 psi = cmul(make_float2(pr[2 * jj], pr[2 * jj + 1]), v[q][4 * h + jj]);
-              if constexpr (CHI) {
-                const float2 st = dm_init ? psi : Sn[line[q] * M + x];
-                psi = make_float2(2.f * psi.x - st.x, 2.f * psi.y - st.y);
-              }
               if (!NEAR && ((line[q] + x) & 1)) psi = make_float2(-psi.x, -psi.y);
               v[q][4 * h + jj] = psi;
             }
@@ -234,21 +221,16 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
           for (int j = 0; j < E; ++j) {
             const int x = tp[q] + G * j;
             float2 psi = cmul(Pk[line[q] * M + x], On[(size_t)line[q] * a.obj_w + x]);
-            if constexpr (CHI) {
-              const float2 st = dm_init ? psi : Sn[line[q] * M + x];
-              psi = make_float2(2.f * psi.x - st.x, 2.f * psi.y - st.y);
-            }
             if (!NEAR && ((line[q] + x) & 1)) psi = make_float2(-psi.x, -psi.y);
             v[q][j] = psi;
           }
       }
     };
 
-    // ---- propagation to the detector and the pc intensity model of Fig. 1 box 1 on the own rows.
-    // PS bit 0: accumulate the error of the model intensity; bit 1: push the modulus ratio R to
-    // every rank (then Z holds R for the whole tile)
-    auto detector = [&](auto ps_c) {
-      constexpr int PS = decltype(ps_c)::value;
+    // ---- propagation to the detector and the pc intensity model of Fig. 1 box 1 on the own rows: the
+    // error of the model intensity, and the modulus ratio R pushed to every rank (Z holds R for the
+    // whole tile)
+    auto detector = [&]() {
       // ---- forward propagation
       fft2_forward<M, V>(v, cbuf, s_tw, tid);  // COL layout
       if constexpr (NEAR) {
@@ -344,7 +326,7 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
             if (lr >= nrow) break;
             const int gr = r0 + lr;
             const float acc = out[o];
-            if constexpr ((PS & 1) != 0) {
+            {
               const float im = pre ? s_meas[(nrow + lr) * M + col] : In[gr * M + col];
               const float ihat = a.blur_intensity ? acc : acc * acc;
               const float d = ihat - im;
@@ -353,7 +335,7 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
               err_c = (tt - err_s) - y;
               err_s = tt;
             }
-            if constexpr ((PS & 2) != 0) {
+            {
               const float sq = pre ? s_meas[lr * M + col] : Qn[gr * M + col];
               const float R = a.blur_intensity ? sq * rsqrtf(acc + eps * eps) : __fdividef(sq, acc + eps);
               const uint32_t zoff = z_s + (uint32_t)((gr * LD + col) * 4);
@@ -362,20 +344,11 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
           }
         }
       }
-      // R arrives from every rank; without R only this CTA's shared memory was read
-      if constexpr ((PS & 2) != 0) cluster_sync_all();
-      else __syncthreads();
+      cluster_sync_all();  // R arrives from every rank
     };
 
-    if constexpr (DM) {
-      exit_wave(IntC<0>{});  // the estimate P o_n: its model error is E
-      detector(IntC<1>{});
-      exit_wave(IntC<1>{});  // the reflected wave: its modulus ratio
-      detector(IntC<2>{});
-    } else {
-      exit_wave(IntC<0>{});
-      detector(IntC<3>{});
-    }
+    exit_wave();
+    detector();
     // ---- (5) Psi' = R Psi
 #pragma unroll
     for (int q = 0; q < V; ++q)
@@ -415,7 +388,7 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
         for (int h = 0; h < E / 4; ++h) {
           float pr[8], ac[8];
           tmem_ld8(t_lane + colP + 2 * (q * E + 4 * h), pr);
-          if (!DM && !first) tmem_ld8(t_lane + colA + 2 * (q * E + 4 * h), ac);
+          if (!first) tmem_ld8(t_lane + colA + 2 * (q * E + 4 * h), ac);
           tmem_wait_ld();
 #pragma unroll
           for (int jj = 0; jj < 4; ++jj) {
@@ -424,15 +397,9 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
             float2 psi_new = cscale(v[q][j], inv_m2);
             if (!NEAR && ((ln + x) & 1)) psi_new = make_float2(-psi_new.x, -psi_new.y);
             const float2 p = make_float2(pr[2 * jj], pr[2 * jj + 1]);
-            float2 dpsi = csub(psi_new, cmul(p, o[j]));
-            if constexpr (DM) {  // psi_n <- psi_n + Pi_F(chi) - P o_n; the overlap step takes psi_n - P o_n
-              const float2 ov = cmul(p, o[j]);
-              const float2 st = cadd(dm_init ? ov : Sn[ln * M + x], dpsi);
-              Sn[ln * M + x] = st;
-              dpsi = csub(st, ov);
-            }
+            const float2 dpsi = csub(psi_new, cmul(p, o[j]));
             st_cluster_f2(dst + 8u * x, cconjmul(p, dpsi));
-            if constexpr (!DM) {  // pc-DM takes its probe step after the object step, from its state
+            {
               const float2 pc = cconjmul(o[j], dpsi);
               ac[2 * jj] = first ? pc.x : ac[2 * jj] + pc.x;
               ac[2 * jj + 1] = first ? pc.y : ac[2 * jj + 1] + pc.y;
@@ -442,9 +409,9 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
               }
             }
           }
-          if constexpr (!DM) tmem_st8(t_lane + colA + 2 * (q * E + 4 * h), ac);
+          tmem_st8(t_lane + colA + 2 * (q * E + 4 * h), ac);
         }
-        if constexpr (!DM) tmem_wait_st();
+        tmem_wait_st();
       } else {
 #pragma unroll
         for (int j = 0; j < E; ++j) {
@@ -453,15 +420,9 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
           if (!NEAR && ((ln + x) & 1)) psi_new = make_float2(-psi_new.x, -psi_new.y);
           const float2 p = Pk[ln * M + x];
           const float2 o = On[(size_t)ln * a.obj_w + x];
-          float2 dpsi = csub(psi_new, cmul(p, o));
-          if constexpr (DM) {  // psi_n <- psi_n + Pi_F(chi) - P o_n; the overlap step takes psi_n - P o_n
-            const float2 ov = cmul(p, o);
-            const float2 st = cadd(dm_init ? ov : Sn[ln * M + x], dpsi);
-            Sn[ln * M + x] = st;
-            dpsi = csub(st, ov);
-          }
+          const float2 dpsi = csub(psi_new, cmul(p, o));
           st_cluster_f2(dst + 8u * x, cconjmul(p, dpsi));
-          if constexpr (!DM) {
+          {
             const int qi = ln * M + x;
             const float2 pc = cconjmul(o, dpsi);
             if (first) pacc[qi] = pc;
@@ -491,7 +452,7 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
   // ---- end of a unit: probe-numerator partial from TMEM to global; per-CTA FP64 error
   // numerator (the compensated FP32 thread sums, added in thread order) into partial `part`
   auto finish_unit = [&](const FusedArgs& a, float2* pacc, int part) {
-    if constexpr (TM && !DM) {
+    if constexpr (TM) {
 #pragma unroll
       for (int q = 0; q < V; ++q)
 #pragma unroll
@@ -517,39 +478,13 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
     __syncthreads();  // red aliases the exchange buffer
   };
 
-  if constexpr (!QUEUED) {
-    // one problem: cluster `slot` takes positions slot, slot + slots, ... and owns partial `slot`
-    setup_unit(a_in);
-    __syncthreads();
-    float2* pacc = a_in.pacc + ((size_t)slot * K + rank) * M * M;
-    float* dacc = a_in.dacc + (size_t)slot * M * M;
-    for (int n = slot; n < a_in.N; n += nslots) run_position(a_in, n, n == slot, pacc, dacc);
-    finish_unit(a_in, pacc, slot);
-  } else {
-    // work queue over every problem of this launch: chunk (problem, first position, end, partial);
-    // rank 0 takes the next chunk index and hands it to every rank of the cluster
-    FusedArgs* s_desc = reinterpret_cast<FusedArgs*>(smem + SM::BYTES);
-    int* s_item = reinterpret_cast<int*>(smem + SM::BYTES + SM::DESC - 16);
-    for (;;) {
-      if (rank == 0 && tid == 0) {
-        const int c = atomicAdd(a_in.queue, 1);
-        for (int q = 0; q < K; ++q) st_cluster_s32(map_rank(smem_addr(s_item), (unsigned)q), c);
-      }
-      cluster_sync_all();
-      const int c = *s_item;
-      if (c >= a_in.nchunks) break;
-      const int4 ch = a_in.chunks[c];
-      const int* src = reinterpret_cast<const int*>(a_in.probs + ch.x);
-      for (int i = tid; i < (int)(sizeof(FusedArgs) / 4); i += TR) reinterpret_cast<int*>(s_desc)[i] = src[i];
-      __syncthreads();
-      setup_unit(*s_desc);
-      __syncthreads();
-      float2* pacc = s_desc->pacc + ((size_t)ch.w * K + rank) * M * M;
-      float* dacc = s_desc->dacc + (size_t)ch.w * M * M;
-      for (int n = ch.y; n < ch.z; ++n) run_position(*s_desc, n, n == ch.y, pacc, dacc);
-      finish_unit(*s_desc, pacc, ch.w);
-    }
-  }
+  // cluster `slot` takes positions slot, slot + slots, ... and owns partial `slot`
+  setup_unit(a_in);
+  __syncthreads();
+  float2* pacc = a_in.pacc + ((size_t)slot * K + rank) * M * M;
+  float* dacc = a_in.dacc + (size_t)slot * M * M;
+  for (int n = slot; n < a_in.N; n += nslots) run_position(a_in, n, n == slot, pacc, dacc);
+  finish_unit(a_in, pacc, slot);
   if constexpr (TM) {
     tmem_fence_before();
     __syncthreads();

@@ -144,46 +144,70 @@ __global__ void __launch_bounds__(256 * kProbeGroups) k_probe_gather(const Updat
 // After the object step: slot s sums, over positions n = s, s + slots, ..., conj(o'_n)(psi_n,k - P_k o'_n)
 // into pacc[s][k] and |o'_n|^2 into dacc[s] (o'_n: the new object under position n). Inside a
 // complex-constraint window the states first move with their boxes, psi_n,k += P_k (o'_n - o''_n),
-// o''_n the object before the constraint. grid (ceil(M^2 / 256), slots); one thread per probe pixel
-// and every mode, so o'_n is read once
-__global__ void k_dm_probe_partials(const UpdateArgs u) {
+// o''_n the object before the constraint. grid (ceil(M^2 / 512), slots); one thread per two neighbouring
+// probe pixels and every mode (KT >= K), so o'_n is read once. Bound by reading the state (N K M^2 complex):
+// 16-byte loads, two positions in flight
+template <int KT>
+__global__ void __launch_bounds__(256) k_dm_probe_partials(const UpdateArgs u) {
   const int MM = u.M * u.M;
-  const int p = blockIdx.x * 256 + threadIdx.x;
+  const int p = (blockIdx.x * 256 + threadIdx.x) * 2;
   if (p >= MM) return;
-  const int s = blockIdx.y;
+  const int s = blockIdx.y, K = u.K;
   const int row = p / u.M, col = p % u.M;
-  float2 pk[kMaxModes], acc[kMaxModes];
+  float2 pk[KT][2], acc[KT][2];
 #pragma unroll
-  for (int k = 0; k < kMaxModes; ++k) {
-    pk[k] = k < u.K ? u.P[(size_t)k * MM + p] : make_float2(0.f, 0.f);
-    acc[k] = make_float2(0.f, 0.f);
-  }
-  float d = 0.f;
+  for (int k = 0; k < KT; ++k)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      pk[k][h] = k < K ? u.P[(size_t)k * MM + p + h] : make_float2(0.f, 0.f);
+      acc[k][h] = make_float2(0.f, 0.f);
+    }
+  float d[2] = {0.f, 0.f};
+#pragma unroll 2
   for (int n = s; n < u.N; n += u.slots) {
     const int2 r = u.pos[n];
     const size_t q = (size_t)(r.x + row) * u.obj_w + r.y + col;
-    const float2 o = u.O[q];
-    d += cabs2(o);
-    float2* ps = u.dm_psi + (size_t)n * u.K * MM + p;
+    float4* ps = reinterpret_cast<float4*>(u.dm_psi + (size_t)n * K * MM + p);
+    const float2 o[2] = {u.O[q], u.O[q + 1]};
+    float4 st[KT];
+#pragma unroll
+    for (int k = 0; k < KT; ++k)
+      if (k < K) st[k] = ps[(size_t)k * (MM / 2)];
+    float2 dlt[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
     if (u.dm_obj_prev) {
-      const float2 dlt = csub(o, u.dm_obj_prev[q]);
-#pragma unroll
-      for (int k = 0; k < kMaxModes; ++k)
-        if (k < u.K) {
-          const float2 st = cadd(ps[(size_t)k * MM], cmul(pk[k], dlt));
-          ps[(size_t)k * MM] = st;
-          acc[k] = cadd(acc[k], cconjmul(o, csub(st, cmul(pk[k], o))));
-        }
-    } else {
-#pragma unroll
-      for (int k = 0; k < kMaxModes; ++k)
-        if (k < u.K) acc[k] = cadd(acc[k], cconjmul(o, csub(ps[(size_t)k * MM], cmul(pk[k], o))));
+      dlt[0] = csub(o[0], u.dm_obj_prev[q]);
+      dlt[1] = csub(o[1], u.dm_obj_prev[q + 1]);
     }
+    d[0] += cabs2(o[0]);
+    d[1] += cabs2(o[1]);
+#pragma unroll
+    for (int k = 0; k < KT; ++k)
+      if (k < K) {
+        float2 w[2] = {make_float2(st[k].x, st[k].y), make_float2(st[k].z, st[k].w)};
+        if (u.dm_obj_prev) {
+          w[0] = cadd(w[0], cmul(pk[k][0], dlt[0]));
+          w[1] = cadd(w[1], cmul(pk[k][1], dlt[1]));
+          ps[(size_t)k * (MM / 2)] = make_float4(w[0].x, w[0].y, w[1].x, w[1].y);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          acc[k][h] = cadd(acc[k][h], cconjmul(o[h], csub(w[h], cmul(pk[k][h], o[h]))));
+      }
   }
 #pragma unroll
-  for (int k = 0; k < kMaxModes; ++k)
-    if (k < u.K) const_cast<float2*>(u.pacc)[((size_t)s * u.K + k) * MM + p] = acc[k];
-  const_cast<float*>(u.dacc)[(size_t)s * MM + p] = d;
+  for (int k = 0; k < KT; ++k)
+    if (k < K)
+      *reinterpret_cast<float4*>(const_cast<float2*>(u.pacc) + ((size_t)s * K + k) * MM + p) =
+          make_float4(acc[k][0].x, acc[k][0].y, acc[k][1].x, acc[k][1].y);
+  *reinterpret_cast<float2*>(const_cast<float*>(u.dacc) + (size_t)s * MM + p) = make_float2(d[0], d[1]);
+}
+
+static void launch_dm_probe_partials(const UpdateArgs& u, cudaStream_t s) {
+  const dim3 grid((unsigned)((u.M * u.M / 2 + 255) / 256), (unsigned)u.slots);
+  if (u.K == 1) k_dm_probe_partials<1><<<grid, 256, 0, s>>>(u);
+  else if (u.K == 2) k_dm_probe_partials<2><<<grid, 256, 0, s>>>(u);
+  else if (u.K <= 4) k_dm_probe_partials<4><<<grid, 256, 0, s>>>(u);
+  else k_dm_probe_partials<8><<<grid, 256, 0, s>>>(u);
 }
 
 // ------------------------------------------------------------------ object: per-tile gather of the contributions
@@ -397,7 +421,7 @@ cudaError_t launch_update_probe(const UpdateArgs& u, cudaStream_t s) {
   const int MM = u.M * u.M;
   const int pb = (MM + 255) / 256;
   if (u.dm_psi && (u.update_probe || u.dm_obj_prev)) {
-    k_dm_probe_partials<<<dim3(pb, u.slots), 256, 0, s>>>(u);
+    launch_dm_probe_partials(u, s);
     if (u.update_probe) k_probe_gather<<<dim3(pb, u.K + 1), 256 * kProbeGroups, 0, s>>>(u);
   }
   k_probe_apply<<<dim3(pb, u.K), 256, 0, s>>>(u);
