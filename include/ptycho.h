@@ -181,11 +181,12 @@ ptycho_status ptycho_plan_batch(int32_t B, const ptycho_params* const* params, c
 ptycho_status ptycho_iterate_batch(ptycho_plan_t plan, void* const* objects, void* const* probes, int32_t n_iter);
 ptycho_status ptycho_error_batch(ptycho_plan_t plan, double* nrmse_last);
 
-/* Work-queue batching: problems with M in {32, 64, 128} sharing K, geometry and
+/* Work-queue batching: problems with M in {8, 16, 32, 64, 128} sharing K, geometry and
  * kernel width class (11 x 11 or any other size) are drained by one persistent
- * launch per class; each chunk of L consecutive positions keeps its own probe and
- * error partials, summed in chunk order (results do not depend on which cluster
- * took a chunk). L is chosen per class by an autotuner the first time a batch
+ * launch per class. Each chunk of L consecutive positions is one work item, or, in a class
+ * with fewer chunks than the GPU has CTA slots, up to eight items of consecutive positions;
+ * every item keeps its own probe and error partials, summed in position order (results do not
+ * depend on which CTA took an item). L is chosen per class by an autotuner the first time a batch
  * plan of that class is built on a device in the process: it times the class's
  * launch for L = 8, 16, 32, 64 on the device and keeps the fastest (cached per
  * device, M, K, geometry and kernel width class).
@@ -205,7 +206,7 @@ ptycho_status ptycho_set_staged_chunk(int32_t chunk);
 int32_t ptycho_staged_chunk(ptycho_plan_t plan);
 /* Describe the work-queue classes of a batch plan: for each of the first
  * max_classes classes, 8 int32 (M, K, near field, kernel width class 5 or 15,
- * members, chunk length, chunks, persistent clusters) into out; *count = the
+ * members, chunk length, chunks, co-resident groups of CTAs that serve a chunk) into out; *count = the
  * number of classes. */
 ptycho_status ptycho_batch_classes(ptycho_plan_t plan, int32_t max_classes, int32_t* out, int32_t* count);
 

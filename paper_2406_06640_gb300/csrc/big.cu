@@ -3,11 +3,16 @@
 // Fig. 1 box 1), split into passes over an L2-sized scratch W that holds a
 // chunk of C positions x K modes:
 //
-//   far field:  rows(exit wave, DFT) -> cols(DFT) -> modulus (R) -> cols(R x, IDFT)
+//   far field:  rows(exit wave, DFT) -> cols(DFT: S) -> modulus (R) -> cols(DFT, R x, IDFT)
 //               -> rows(IDFT, dpsi, contributions)
-//   near field: rows(exit wave, DFT) -> cols(DFT, x H, IDFT) -> rows(IDFT)
-//               -> modulus (R) -> rows(R x, DFT) -> cols(DFT, x conj H, IDFT)
+//   near field: rows(exit wave, DFT) -> cols(DFT, x H, IDFT) -> rows(IDFT: S)
+//               -> modulus (R) -> rows(IDFT, R x, DFT) -> cols(DFT, x conj H, IDFT)
 //               -> rows(IDFT, dpsi, contributions)
+//
+// The pass that reaches the detector field walks the K modes in order and writes S = sum_k |Psi_k|^2 only; the
+// pass after the modulus repeats that line transform on its way back. So W is written once less (it
+// streams through HBM for large chunks, and the passes run at its rate), and the modulus pass reads one
+// float per pixel instead of K complex values (with halo rows).
 //
 // A length-256 line is transformed by 16 threads: a radix-16 pass in
 // registers over x = t + 16 j, the twiddle W_256^(t k2), a warp-local swap in
@@ -20,6 +25,7 @@
 #include "big_line.cuh"
 #include "engine.h"
 #include "fft.cuh"
+#include "fused_common.cuh"
 
 namespace ptycho {
 
@@ -39,8 +45,7 @@ __device__ __forceinline__ void load_tw(float2* s_tw, const float2* tw) {
 
 }  // namespace
 
-// ---- row passes. mode 0: exit wave + forward DFT; 1: R x (row) then forward DFT in place;
-// 2: inverse DFT in place, / M^2
+// ---- row passes. mode 0: exit wave + forward DFT; 1: inverse DFT, R x (row), forward DFT in place
 template <int BL, int MODE, bool NEAR>
 __global__ void __launch_bounds__(BigShape<BL>::LROW * BT) k_big_rows(const BigArgs b) {
   constexpr int E = BigShape<BL>::E, LROW = BigShape<BL>::LROW;
@@ -72,101 +77,153 @@ __global__ void __launch_bounds__(BigShape<BL>::LROW * BT) k_big_rows(const BigA
       if (!NEAR && ((y + x) & 1)) psi = make_float2(-psi.x, -psi.y);
       a[j] = psi;
     }
-  } else if constexpr (MODE == 1) {
-    // Psi' = R Psi (the modulus ratio of this position) on the way in
-    const float* Rr = b.R + (size_t)c * MM + (size_t)y * BL;
-#pragma unroll
-    for (int j = 0; j < E; ++j) a[j] = cscale(row[t + 16 * j], Rr[t + 16 * j]);
   } else {
+    // Psi' = R Psi (the modulus ratio of this position)
+    const float* Rr = b.R + (size_t)c * MM + (size_t)y * BL;
+    float R[E];
 #pragma unroll
     for (int r = 0; r < E; ++r) a[r] = row[line_freq<BL>(t, r)];
-  }
-  if constexpr (MODE == 2) {
+#pragma unroll
+    for (int j = 0; j < E; ++j) R[j] = Rr[t + 16 * j];
     line_fft<BL, true>(a, s_sw[li], s_tw, t);
     const float s = 1.0f / (float)(BL * BL);
 #pragma unroll
-    for (int j = 0; j < E; ++j) row[t + 16 * j] = cscale(a[j], s);
-  } else {
-    line_fft<BL, false>(a, s_sw[li], s_tw, t);
-#pragma unroll
-    for (int r = 0; r < E; ++r) row[line_freq<BL>(t, r)] = a[r];
+    for (int j = 0; j < E; ++j) a[j] = cscale(cscale(a[j], s), R[j]);
   }
+  line_fft<BL, false>(a, s_sw[li], s_tw, t);
+#pragma unroll
+  for (int r = 0; r < E; ++r) row[line_freq<BL>(t, r)] = a[r];
 }
 
-// ---- column passes on a BL x LINES tile staged through shared memory.
-// op 0: forward DFT; 1: R x (tile), inverse DFT (far backward); 2: DFT, x H, IDFT (near forward);
-// 3: DFT, x conj H, IDFT (near backward)
+// near field: S = sum_k |Psi_k|^2 of the inverse row DFTs / M^2
+template <int BL>
+__global__ void __launch_bounds__(BigShape<BL>::LROW * BT) k_big_rows_detector(const BigArgs b) {
+  constexpr int E = BigShape<BL>::E, LROW = BigShape<BL>::LROW;
+  __shared__ float2 s_tw[BigShape<BL>::TWN];
+  __shared__ float2 s_sw[LROW][BigShape<BL>::SWN];
+  load_tw<BL>(s_tw, b.tw);
+  __syncthreads();
+  const int li = threadIdx.x / BT, t = threadIdx.x % BT;
+  const int y = blockIdx.x * LROW + li, c = blockIdx.y;
+  const size_t MM = (size_t)BL * BL;
+  const float s = 1.0f / (float)(BL * BL);
+  float sum[E];
+#pragma unroll
+  for (int j = 0; j < E; ++j) sum[j] = 0.f;
+  for (int k = 0; k < b.K; ++k) {
+    const float2* row = b.W + ((size_t)c * b.K + k) * MM + (size_t)y * BL;
+    float2 a[E];
+#pragma unroll
+    for (int r = 0; r < E; ++r) a[r] = row[line_freq<BL>(t, r)];
+    line_fft<BL, true>(a, s_sw[li], s_tw, t);
+#pragma unroll
+    for (int j = 0; j < E; ++j) sum[j] += cabs2(cscale(a[j], s));
+  }
+  float* S = b.S + (size_t)c * MM + (size_t)y * BL;
+#pragma unroll
+  for (int j = 0; j < E; ++j) S[t + 16 * j] = sum[j];
+}
+
+// ---- column passes on a BL x LINES tile staged through shared memory; the line swaps use the tile's own
+// column (its values are in registers then), so a CTA takes half the shared memory of a separate swap
+// buffer and four to eight CTAs overlap their loads, transforms and stores on an SM (with one CTA of 32
+// lines per SM the three phases ran one after the other: 112 us for 32 positions x 8 modes of 256^2).
+// op 0: S of the forward DFTs of every mode (far forward); 1: DFT, R x, IDFT (far backward);
+// 2: DFT, x H, IDFT (near forward); 3: DFT, x conj H, IDFT (near backward)
 template <int BL, int OP>
-__global__ void __launch_bounds__(BigShape<BL>::LINES * BT) k_big_cols(const BigArgs b) {
+__global__ void __launch_bounds__(BigShape<BL>::LINES * BT, BL == 256 ? (OP < 2 ? 3 : 4) : 2) k_big_cols(const BigArgs b) {
   constexpr int E = BigShape<BL>::E, LINES = BigShape<BL>::LINES;
   constexpr int TP = LINES + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* tile = reinterpret_cast<float2*>(smem_raw);  // [BL][TP]
-  float2* s_tw = tile + BL * TP;
-  float2* s_sw = s_tw + BigShape<BL>::TWN;  // [LINES][SWN]
-  float2* s_h = s_sw + LINES * BigShape<BL>::SWN;
+  float2* tile = reinterpret_cast<float2*>(smem_raw);  // [SWN][TP], rows 0 .. BL - 1 staged
+  float2* s_tw = tile + BigShape<BL>::SWN * TP;
+  float2* s_h = s_tw + BigShape<BL>::TWN;                  // OP >= 2: BL
+  float* s_r = reinterpret_cast<float*>(s_h);              // OP == 1: BL x TP
   load_tw<BL>(s_tw, b.tw);
   if constexpr (OP >= 2)
     for (int i = threadIdx.x; i < BL; i += blockDim.x) s_h[i] = b.hq[i];
-  const int x0 = blockIdx.x * LINES, k = blockIdx.y, c = blockIdx.z;
+  const int x0 = blockIdx.x * LINES, c = OP == 0 ? blockIdx.y : blockIdx.z;
   const size_t MM = (size_t)BL * BL;
-  float2* Wk = b.W + ((size_t)c * b.K + k) * MM;
-  // coalesced tile load: LINES consecutive columns per row; the far-field inverse pass applies
-  // Psi' = R Psi (the modulus ratio of this position) on the way in
-  const float* Rc = b.R + (size_t)c * MM;
-  for (int i = threadIdx.x; i < BL * LINES; i += blockDim.x) {
-    const int yy = i / LINES, xx = i % LINES;
-    const float2 w = Wk[(size_t)yy * BL + x0 + xx];
-    tile[yy * TP + xx] = OP == 1 ? cscale(w, Rc[(size_t)yy * BL + x0 + xx]) : w;
-  }
-  __syncthreads();
   const int cl = threadIdx.x / BT, t = threadIdx.x % BT;
-  float2* sw = s_sw + cl * BigShape<BL>::SWN;
-  float2 a[E];
-  if constexpr (OP == 1) {
+  const ColumnSwap<BL, TP> sw{tile + cl};
+  float sum[OP == 0 ? E : 1];
+  if constexpr (OP == 0)
 #pragma unroll
-    for (int r = 0; r < E; ++r) a[r] = tile[line_freq<BL>(t, r) * TP + cl];
-    line_fft<BL, true>(a, sw, s_tw, t);
-  } else {
+    for (int r = 0; r < E; ++r) sum[r] = 0.f;
+  const int k_lo = OP == 0 ? 0 : blockIdx.y, k_hi = OP == 0 ? b.K : k_lo + 1;
+  for (int k = k_lo; k < k_hi; ++k) {
+    float2* Wk = b.W + ((size_t)c * b.K + k) * MM;
+    // coalesced tile load: LINES consecutive columns per row; the far-field backward pass stages the
+    // modulus ratio of this position beside it
+    const float* Rc = b.R + (size_t)c * MM;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < BL * LINES; i += LINES * BT) {
+      const int yy = i / LINES, xx = i % LINES;
+      tile[yy * TP + xx] = Wk[(size_t)yy * BL + x0 + xx];
+      if constexpr (OP == 1) s_r[yy * TP + xx] = Rc[(size_t)yy * BL + x0 + xx];
+    }
+    __syncthreads();
+    float2 a[E];
 #pragma unroll
     for (int j = 0; j < E; ++j) a[j] = tile[(t + 16 * j) * TP + cl];
-    line_fft<BL, false>(a, sw, s_tw, t);  // a[r] = column spectrum at u = line_freq(t, r)
-    if constexpr (OP >= 2) {
+    __syncwarp();  // the line's values are in registers: its column is the swap buffer now
+    line_fft_swap<BL, false>(a, sw, s_tw, t);  // a[r] = column spectrum at u = line_freq(t, r)
+    if constexpr (OP == 0) {
+#pragma unroll
+      for (int r = 0; r < E; ++r) sum[r] += cabs2(a[r]);
+      __syncthreads();  // the next mode's load, or S, rewrites the tile
+      continue;
+    } else if constexpr (OP == 1) {
+#pragma unroll
+      for (int r = 0; r < E; ++r) a[r] = cscale(a[r], s_r[line_freq<BL>(t, r) * TP + cl]);  // Psi' = R Psi
+    } else {
       const float2 hv = s_h[x0 + cl];  // H(u, v) = h[u] h[v], v = this column's frequency
 #pragma unroll
       for (int r = 0; r < E; ++r) {
         const float2 hh = cmul(s_h[line_freq<BL>(t, r)], hv);
         a[r] = OP == 2 ? cmul(a[r], hh) : cmulc(a[r], hh);
       }
-      line_fft<BL, true>(a, sw, s_tw, t);
     }
-  }
-  __syncthreads();
-  if constexpr (OP == 0) {
-#pragma unroll
-    for (int r = 0; r < E; ++r) tile[line_freq<BL>(t, r) * TP + cl] = a[r];
-  } else {
+    line_fft_swap<BL, true>(a, sw, s_tw, t);
+    // (a line's transform ends with a warp barrier after its last read of the swap)
 #pragma unroll
     for (int j = 0; j < E; ++j) tile[(t + 16 * j) * TP + cl] = a[j];
+    __syncthreads();
+#pragma unroll 4
+    for (int i = threadIdx.x; i < BL * LINES; i += LINES * BT) {
+      const int yy = i / LINES, xx = i % LINES;
+      Wk[(size_t)yy * BL + x0 + xx] = tile[yy * TP + xx];
+    }
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < BL * LINES; i += blockDim.x) {
-    const int yy = i / LINES, xx = i % LINES;
-    Wk[(size_t)yy * BL + x0 + xx] = tile[yy * TP + xx];
+  if constexpr (OP == 0) {
+#pragma unroll
+    for (int r = 0; r < E; ++r) tile[line_freq<BL>(t, r) * TP + cl].x = sum[r];
+    __syncthreads();
+    float* S = b.S + (size_t)c * MM;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < BL * LINES; i += LINES * BT) {
+      const int yy = i / LINES, xx = i % LINES;
+      S[(size_t)yy * BL + x0 + xx] = tile[yy * TP + xx].x;
+    }
   }
 }
 
-// ---- modulus: rows [y0, y0 + RB) of one position, with KH halo rows for the y blur.
-// Writes the ratio R to its own buffer (W is still read by the neighbouring
-// blocks' halos); the next pass applies Psi' = R Psi as it loads W.
+// ---- modulus: rows [y0, y0 + RB) of one position from S, with KH halo rows for the y blur. Writes the ratio
+// R to its own buffer; the next pass applies Psi' = R Psi as it loads W. Each blur keeps a window of samples
+// in registers for eight outputs (blur_strip), lanes along the other axis of an odd-stride buffer.
+template <int BL>
+constexpr int kModTpb = BL == 256 ? 256 : 512;  // two CTAs fit an SM at 512 columns, four at 256
+
 template <int BL, int KH>
-__global__ void __launch_bounds__(256) k_big_modulus(const BigArgs b) {
+__global__ void __launch_bounds__(kModTpb<BL>) k_big_modulus(const BigArgs b) {
+  constexpr int TPB = kModTpb<BL>;
   constexpr int HR = RB + 2 * KH;  // rows held
+  constexpr int LD = BL + 1, NB = 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float* sA = reinterpret_cast<float*>(smem_raw);  // HR x BL
-  float* sB = sA + HR * BL;                          // HR x BL
+  float* sA = reinterpret_cast<float*>(smem_raw);  // HR x LD
+  float* sB = sA + HR * LD;                        // HR x LD
   __shared__ float s_gx[2 * KH + 1], s_gy[2 * KH + 1];
-  __shared__ double s_red[256];
+  __shared__ double s_red[TPB];
   for (int i = threadIdx.x; i < 2 * KH + 1; i += blockDim.x) {
     const int d = i - KH;
     const bool in = d >= -b.kh && d <= b.kh;
@@ -176,58 +233,57 @@ __global__ void __launch_bounds__(256) k_big_modulus(const BigArgs b) {
   const int y0 = blockIdx.x * RB, c = blockIdx.y;
   const int n = b.n0 + c;
   const size_t MM = (size_t)BL * BL;
-  const float2* Wc = b.W + (size_t)c * b.K * MM;
-  // mode sum (rank order k = 0..K-1), amplitude or intensity
-  for (int i = threadIdx.x; i < HR * BL; i += blockDim.x) {
-    const int yy = y0 - KH + i / BL, x = i % BL;
-    float s = 0.f;
-    if (yy >= 0 && yy < BL)
-      for (int k = 0; k < b.K; ++k) s += cabs2(Wc[(size_t)k * MM + (size_t)yy * BL + x]);
-    sA[i] = b.blur_intensity ? s : sqrtf(s);
+  // amplitude or intensity of the mode sum; rows outside the pattern are zero
+  const float* Sc = b.S + (size_t)c * MM;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < HR * BL; i += TPB) {
+    const int r = i / BL, x = i % BL, yy = y0 - KH + r;
+    const float s = yy >= 0 && yy < BL ? Sc[(size_t)yy * BL + x] : 0.f;
+    sA[r * LD + x] = b.blur_intensity ? s : sqrtf(s);
   }
   __syncthreads();
   // blur along x (columns, sigma_1), zero padded
-  for (int i = threadIdx.x; i < HR * BL; i += blockDim.x) {
-    const int r = i / BL, x = i % BL;
-    float acc = 0.f;
+  for (int w = threadIdx.x; w < HR * (BL / NB); w += TPB) {
+    const int r = w % HR, c0 = (w / HR) * NB;
+    float out[NB];
+    blur_strip<NB, KH>(sA, r * LD, 1, c0, 0, BL, s_gx, out);
 #pragma unroll
-    for (int d = -KH; d <= KH; ++d) {
-      const int xx = x + d;
-      if (xx >= 0 && xx < BL) acc = fmaf(s_gx[d + KH], sA[r * BL + xx], acc);
-    }
-    sB[i] = acc;
+    for (int o = 0; o < NB; ++o) sB[r * LD + c0 + o] = out[o];
   }
   __syncthreads();
-  // blur along y (rows, sigma_2) for the own rows, ratio, error; Psi' = R Psi for every mode
+  // blur along y (rows, sigma_2) for the own rows, ratio, error
   const float eps = b.eps;
   float es = 0.f, ec = 0.f;
-  const float* In = b.I + (size_t)n * MM;
   const float* Sn = b.sqrtI + (size_t)n * MM;
-  for (int i = threadIdx.x; i < RB * BL; i += blockDim.x) {
-    const int r = i / BL, x = i % BL, y = y0 + r;
-    float acc = 0.f;
+  for (int w = threadIdx.x; w < BL * (RB / NB); w += TPB) {
+    const int x = w % BL, rs = (w / BL) * NB;
+    float sq[NB], out[NB];
 #pragma unroll
-    for (int d = -KH; d <= KH; ++d) acc = fmaf(s_gy[d + KH], sB[(r + KH + d) * BL + x], acc);
-    const float sq = Sn[(size_t)y * BL + x];
-    float ihat, R;
-    if (b.blur_intensity) {
-      ihat = acc;
-      R = sq * rsqrtf(acc + eps * eps);
-    } else {
-      ihat = acc * acc;
-      R = __fdividef(sq, acc + eps);
+    for (int o = 0; o < NB; ++o) sq[o] = __ldcs(&Sn[(size_t)(y0 + rs + o) * BL + x]);
+    blur_strip<NB, KH>(sB, x, LD, rs + KH, 0, HR, s_gy, out);
+#pragma unroll
+    for (int o = 0; o < NB; ++o) {
+      const float acc = out[o];
+      float ihat, R;
+      if (b.blur_intensity) {
+        ihat = acc;
+        R = sq[o] * rsqrtf(acc + eps * eps);
+      } else {
+        ihat = acc * acc;
+        R = __fdividef(sq[o], acc + eps);
+      }
+      const float dd = ihat - sq[o] * sq[o];
+      const float yv = fmaf(dd, dd, -ec);
+      const float tt = es + yv;
+      ec = (tt - es) - yv;
+      es = tt;
+      if (b.dm_pass != 1) b.R[(size_t)c * MM + (size_t)(y0 + rs + o) * BL + x] = R;  // pc-DM: R of chi only
     }
-    const float dd = ihat - In[(size_t)y * BL + x];
-    const float yv = fmaf(dd, dd, -ec);
-    const float tt = es + yv;
-    ec = (tt - es) - yv;
-    es = tt;
-    if (b.dm_pass != 1) b.R[(size_t)c * MM + (size_t)y * BL + x] = R;  // pc-DM: R of chi only
   }
   if (b.dm_pass == 2) return;  // pc-DM: the error is the estimate's (first sweep); uniform per block
   s_red[threadIdx.x] = (double)es - (double)ec;
   __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
+  for (int w = TPB / 2; w > 0; w >>= 1) {
     if (threadIdx.x < w) s_red[threadIdx.x] += s_red[threadIdx.x + w];
     __syncthreads();
   }
@@ -244,92 +300,192 @@ __device__ __forceinline__ void red_add(float* a, float v) {
   asm volatile("red.global.add.f32 [%0], %1;" ::"l"(a), "f"(v));
 }
 
-// ---- final inverse row DFT of every mode, dpsi, contributions
-template <int BL, bool NEAR>
-__global__ void __launch_bounds__(BigShape<BL>::LROW * BT) k_big_final(const BigArgs b) {
-  constexpr int E = BigShape<BL>::E, LROW = BigShape<BL>::LROW;
+// ---- final inverse row DFT of every mode, dpsi, contributions. A CTA owns FR rows of the tile and walks the
+// positions g, g + groups, ... of the chunk (g = blockIdx.y) and their modes.
+// ACC: the probe partial of (group, mode, rows) stays in shared memory, every element touched by one thread,
+// and is read and written once per launch. Otherwise (partials of K modes too large for three CTAs on an
+// SM) one group per position and L2 reductions into its partial. pc-DM (b.psi) has no probe partials here.
+template <int BL>
+struct FinalShape {
+  static constexpr int FR = 4, TPB = FR * BT;
+  static constexpr size_t ACC_MAX = 72 * 1024;  // three CTAs on an SM
+  static constexpr size_t acc_bytes(int K) { return (size_t)K * FR * BL * sizeof(float2); }
+  static constexpr bool accumulates(int K) { return acc_bytes(K) <= ACC_MAX; }
+};
+
+template <int BL, bool NEAR, bool ACC>
+__global__ void __launch_bounds__(FinalShape<BL>::TPB) k_big_final(const BigArgs b, int nc) {
+  constexpr int E = BigShape<BL>::E, FR = FinalShape<BL>::FR;
+  constexpr bool AHEAD = BL == 256;  // registers for the next mode's line and this one's probe values
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* s_p = reinterpret_cast<float2*>(smem_raw);  // ACC: K x FR x BL
   __shared__ float2 s_tw[BigShape<BL>::TWN];
-  __shared__ float2 s_sw[LROW][BigShape<BL>::SWN];
+  __shared__ float2 s_sw[FR][BigShape<BL>::SWN];
   load_tw<BL>(s_tw, b.tw);
   __syncthreads();
   const int li = threadIdx.x / BT, t = threadIdx.x % BT;
-  const int y = blockIdx.x * LROW + li;
-  const int c = blockIdx.y;
-  const int n = b.n0 + c;
-  const bool first = b.n0 == b.n_first;
-  const size_t MM = (size_t)BL * BL;
-  const int2 pn = b.pos[n];
-  const float2* On = b.O + (size_t)(pn.x + y) * b.obj_w + pn.y;
+  const int y = blockIdx.x * FR + li;
+  const int g = blockIdx.y, G = gridDim.y, K = b.K;
+  if (g >= nc) return;  // (a short last chunk: the group's partial stays as it is)
+  const bool start = b.n0 == b.n_first;  // this launch starts the partials
+  const size_t MM = (size_t)BL * BL, yo = (size_t)y * BL;
   const float s = 1.0f / (float)(BL * BL);
-  float2 cacc[E];
+  float2* pacc = b.pacc + (size_t)g * K * MM + yo;
+  float* dacc = b.dacc + (size_t)g * MM + yo;
+  if (ACC && !start)
+    for (int k = 0; k < K; ++k)
 #pragma unroll
-  for (int j = 0; j < E; ++j) cacc[j] = make_float2(0.f, 0.f);
-  for (int k = 0; k < b.K; ++k) {
-    const float2* row = b.W + ((size_t)c * b.K + k) * MM + (size_t)y * BL;
-    float2 a[E];
+      for (int j = 0; j < E; ++j) s_p[(k * FR + li) * BL + t + 16 * j] = pacc[(size_t)k * MM + t + 16 * j];
+  float dsum[E];
+#pragma unroll
+  for (int j = 0; j < E; ++j) dsum[j] = 0.f;
+  auto line = [&](int c, int k, float2 (&a)[E]) {
+    const float2* row = b.W + ((size_t)c * K + k) * MM + yo;
 #pragma unroll
     for (int r = 0; r < E; ++r) a[r] = row[line_freq<BL>(t, r)];
-    line_fft<BL, true>(a, s_sw[li], s_tw, t);
-    const float2* Pk = b.P + (size_t)k * MM + (size_t)y * BL;
-    float2* pacc = b.pacc + ((size_t)c * b.K + k) * MM + (size_t)y * BL;
-    // pc-DM: psi_n <- psi_n + Pi_F(chi) - P o_n, the overlap step takes psi_n - P o_n (its probe
-    // sums follow the object step)
-    float2* St = b.psi ? b.psi + ((size_t)n * b.K + k) * MM + (size_t)y * BL : nullptr;
+  };
+  float2 nx[AHEAD ? E : 1];
+  if constexpr (AHEAD) line(g, 0, nx);
+  for (int c = g; c < nc; c += G) {
+    const int n = b.n0 + c;
+    const bool first = start && c == g;
+    const int2 pn = b.pos[n];
+    const float2* On = b.O + (size_t)(pn.x + y) * b.obj_w + pn.y;
+    float2 cacc[E], ov[AHEAD ? E : 1];
 #pragma unroll
     for (int j = 0; j < E; ++j) {
-      const int x = t + 16 * j;
-      float2 psi_new = cscale(a[j], s);
-      if (!NEAR && ((y + x) & 1)) psi_new = make_float2(-psi_new.x, -psi_new.y);
-      const float2 p = Pk[x], o = On[x];
-      float2 dpsi = csub(psi_new, cmul(p, o));
-      if (St) {
-        const float2 ov = cmul(p, o);
-        const float2 st = cadd(b.dm_init ? ov : St[x], dpsi);
-        St[x] = st;
-        dpsi = csub(st, ov);
+      cacc[j] = make_float2(0.f, 0.f);
+      const float2 o = On[t + 16 * j];
+      dsum[j] += cabs2(o);
+      if constexpr (AHEAD) ov[j] = o;
+    }
+    for (int k = 0; k < K; ++k) {
+      const float2* Pk = b.P + (size_t)k * MM + yo;
+      float2 a[E], pv[AHEAD ? E : 1];
+      if constexpr (AHEAD) {
+#pragma unroll
+        for (int r = 0; r < E; ++r) a[r] = nx[r];
+#pragma unroll
+        for (int j = 0; j < E; ++j) pv[j] = Pk[t + 16 * j];
+        if (k + 1 < K) line(c, k + 1, nx);
+        else if (c + G < nc) line(c + G, 0, nx);
+      } else {
+        line(c, k, a);
       }
-      cacc[j] = cadd(cacc[j], cconjmul(p, dpsi));
-      if (!St) {
+      line_fft<BL, true>(a, s_sw[li], s_tw, t);
+      // pc-DM: psi_n <- psi_n + Pi_F(chi) - P o_n, the overlap step takes psi_n - P o_n (its probe
+      // sums follow the object step)
+      float2* St = b.psi ? b.psi + ((size_t)n * K + k) * MM + yo : nullptr;
+#pragma unroll
+      for (int j = 0; j < E; ++j) {
+        const int x = t + 16 * j;
+        float2 psi_new = cscale(a[j], s);
+        if (!NEAR && ((y + x) & 1)) psi_new = make_float2(-psi_new.x, -psi_new.y);
+        const float2 p = AHEAD ? pv[AHEAD ? j : 0] : Pk[x], o = AHEAD ? ov[AHEAD ? j : 0] : On[x];
+        const float2 po = cmul(p, o);
+        float2 dpsi = csub(psi_new, po);
+        if (St) {
+          const float2 st = cadd(b.dm_init ? po : St[x], dpsi);
+          St[x] = st;
+          dpsi = csub(st, po);
+        }
+        cacc[j] = cadd(cacc[j], cconjmul(p, dpsi));
         const float2 pc = cconjmul(o, dpsi);
-        if (first) pacc[x] = pc;
-        else red_add(&pacc[x], pc);
+        if constexpr (ACC) {
+          float2& q = s_p[(k * FR + li) * BL + x];
+          q = first ? pc : cadd(q, pc);
+        } else if (!St) {
+          if (first) pacc[(size_t)k * MM + x] = pc;
+          else red_add(&pacc[(size_t)k * MM + x], pc);
+        }
       }
     }
-  }
-  float2* cn = b.cn + (size_t)n * MM + (size_t)y * BL;
-  float* dacc = b.dacc + (size_t)c * MM + (size_t)y * BL;
+    float2* cn = b.cn + (size_t)n * MM + yo;
 #pragma unroll
-  for (int j = 0; j < E; ++j) {
-    const int x = t + 16 * j;
-    cn[x] = cacc[j];
-    const float o2 = cabs2(On[x]);
-    if (first) dacc[x] = o2;
-    else red_add(&dacc[x], o2);
+    for (int j = 0; j < E; ++j) cn[t + 16 * j] = cacc[j];
   }
+  if (b.psi) return;
+#pragma unroll
+  for (int j = 0; j < E; ++j) dacc[t + 16 * j] = start ? dsum[j] : dacc[t + 16 * j] + dsum[j];
+  if constexpr (ACC)
+    for (int k = 0; k < K; ++k)
+#pragma unroll
+      for (int j = 0; j < E; ++j) pacc[(size_t)k * MM + t + 16 * j] = s_p[(k * FR + li) * BL + t + 16 * j];
 }
 
-template <int BL>
-static size_t big_cols_smem() {
-  constexpr int LINES = BigShape<BL>::LINES;
-  return sizeof(float2) * ((size_t)BL * (LINES + 1) + BigShape<BL>::TWN + (size_t)LINES * BigShape<BL>::SWN + BL);
+template <int BL, int OP>
+constexpr size_t big_cols_smem() {
+  return sizeof(float2) * ((size_t)BigShape<BL>::SWN * (BigShape<BL>::LINES + 1) + BigShape<BL>::TWN) +
+         (OP >= 2 ? sizeof(float2) * BL : OP == 1 ? sizeof(float) * BL * (BigShape<BL>::LINES + 1) : 0);
 }
 
 int big_row_blocks(int M) { return M / RB; }
 
+// groups of the final pass (probe partials of an accumulation that starts with nc positions): as many as
+// are co-resident, so that no second wave is nearly empty; one per position without accumulators
+template <int BL>
+static cudaError_t final_groups(int K, int nc, int* out) {
+  using FS = FinalShape<BL>;
+  int dev = 0, sms = 0, most = 1 << 30;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  for (auto kern : {k_big_final<BL, false, true>, k_big_final<BL, true, true>}) {
+    int per_sm = 0;
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FS::ACC_MAX);
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, FS::TPB, FS::acc_bytes(K));
+    most = per_sm < most ? per_sm : most;
+  }
+  if (e != cudaSuccess) return e;
+  const int g = most * sms / (BL / FS::FR);
+  *out = g < 1 ? 1 : g < nc ? g : nc;
+  return cudaSuccess;
+}
+cudaError_t big_groups(int M, int K, bool dm, int nc, int* out) {
+  *out = nc;
+  if (dm) return cudaSuccess;
+  if (M == 256 && FinalShape<256>::accumulates(K)) return final_groups<256>(K, nc, out);
+  if (M == 512 && FinalShape<512>::accumulates(K)) return final_groups<512>(K, nc, out);
+  return cudaSuccess;
+}
+
 template <int BL, int KH>
-constexpr size_t big_mod_smem() { return sizeof(float) * 2 * (size_t)(RB + 2 * KH) * BL; }
+constexpr size_t big_mod_smem() { return sizeof(float) * 2 * (size_t)(RB + 2 * KH) * (BL + 1); }
+
+template <int BL, bool NEAR>
+static cudaError_t big_final(const BigArgs& b, int nc, cudaStream_t s) {
+  using FS = FinalShape<BL>;
+  if (FS::accumulates(b.K) && !b.psi) {
+    const dim3 grid(BL / FS::FR, b.groups);
+    const size_t bytes = FS::acc_bytes(b.K);
+    cudaError_t e = cudaFuncSetAttribute(k_big_final<BL, NEAR, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)FS::ACC_MAX);
+    if (e != cudaSuccess) return e;
+    k_big_final<BL, NEAR, true><<<grid, FS::TPB, bytes, s>>>(b, nc);
+  } else {
+    k_big_final<BL, NEAR, false><<<dim3(BL / FS::FR, nc), FS::TPB, 0, s>>>(b, nc);
+  }
+  return cudaGetLastError();
+}
 
 // the passes of one chunk; `full` false stops after the modulus pass (pc-DM first sweep)
 template <int BL>
 static cudaError_t big_passes(const BigArgs& b, int nc, bool full, cudaStream_t s) {
   constexpr int LINES = BigShape<BL>::LINES, LROW = BigShape<BL>::LROW;
   const dim3 blk(LINES * BT), rblk(LROW * BT);
-  const dim3 grow(BL / LROW, b.K, nc), gcol(BL / LINES, b.K, nc), gfin(BL / LROW, nc), gmod(BL / RB, nc);
-  const size_t cs = big_cols_smem<BL>();
+  const dim3 grow(BL / LROW, b.K, nc), gdet(BL / LROW, nc), gcol(BL / LINES, b.K, nc), gcol0(BL / LINES, nc);
+  const dim3 gmod(BL / RB, nc);
   cudaError_t e;
-  for (auto kern : {k_big_cols<BL, 0>, k_big_cols<BL, 1>, k_big_cols<BL, 2>, k_big_cols<BL, 3>})
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs)) != cudaSuccess)
-      return e;
+  if ((e = cudaFuncSetAttribute(k_big_cols<BL, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)big_cols_smem<BL, 0>())) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(k_big_cols<BL, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)big_cols_smem<BL, 1>())) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(k_big_cols<BL, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)big_cols_smem<BL, 2>())) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(k_big_cols<BL, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)big_cols_smem<BL, 3>())) != cudaSuccess)
+    return e;
   if ((e = cudaFuncSetAttribute(k_big_modulus<BL, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)big_mod_smem<BL, 5>())) != cudaSuccess)
     return e;
@@ -338,24 +494,22 @@ static cudaError_t big_passes(const BigArgs& b, int nc, bool full, cudaStream_t 
     return e;
   if (b.near_field) {
     k_big_rows<BL, 0, true><<<grow, rblk, 0, s>>>(b);
-    k_big_cols<BL, 2><<<gcol, blk, cs, s>>>(b);
-    k_big_rows<BL, 2, true><<<grow, rblk, 0, s>>>(b);
+    k_big_cols<BL, 2><<<gcol, blk, big_cols_smem<BL, 2>(), s>>>(b);
+    k_big_rows_detector<BL><<<gdet, rblk, 0, s>>>(b);
   } else {
     k_big_rows<BL, 0, false><<<grow, rblk, 0, s>>>(b);
-    k_big_cols<BL, 0><<<gcol, blk, cs, s>>>(b);
+    k_big_cols<BL, 0><<<gcol0, blk, big_cols_smem<BL, 0>(), s>>>(b);
   }
-  if (b.kh == 5) k_big_modulus<BL, 5><<<gmod, 256, big_mod_smem<BL, 5>(), s>>>(b);
-  else k_big_modulus<BL, 15><<<gmod, 256, big_mod_smem<BL, 15>(), s>>>(b);
+  if (b.kh == 5) k_big_modulus<BL, 5><<<gmod, kModTpb<BL>, big_mod_smem<BL, 5>(), s>>>(b);
+  else k_big_modulus<BL, 15><<<gmod, kModTpb<BL>, big_mod_smem<BL, 15>(), s>>>(b);
   if (!full) return cudaGetLastError();
   if (b.near_field) {
     k_big_rows<BL, 1, true><<<grow, rblk, 0, s>>>(b);
-    k_big_cols<BL, 3><<<gcol, blk, cs, s>>>(b);
-    k_big_final<BL, true><<<gfin, rblk, 0, s>>>(b);
-  } else {
-    k_big_cols<BL, 1><<<gcol, blk, cs, s>>>(b);
-    k_big_final<BL, false><<<gfin, rblk, 0, s>>>(b);
+    k_big_cols<BL, 3><<<gcol, blk, big_cols_smem<BL, 3>(), s>>>(b);
+    return big_final<BL, true>(b, nc, s);
   }
-  return cudaGetLastError();
+  k_big_cols<BL, 1><<<gcol, blk, big_cols_smem<BL, 1>(), s>>>(b);
+  return big_final<BL, false>(b, nc, s);
 }
 
 static cudaError_t big_dispatch(const BigArgs& b, int nc, bool full, cudaStream_t s) {

@@ -154,6 +154,11 @@ struct ptycho_plan_s {
     int* d_queue = nullptr;
     int slots = 0;
     int chunk_len = 0;
+    // CTAs per chunk: a class with fewer chunks than the GPU has CTA slots splits each of them into this many
+    // items of chunk_len / split positions, each with its own partials (22 chunks of 8 positions of 128^2, two
+    // modes, near field: 741 us on 22 CTAs)
+    int split = 1;
+    int nitems = 0;
   };
   std::vector<QueueClass> qclasses;
   std::vector<char> queued;  // per member: drained by its class's work-queue launch
@@ -325,6 +330,7 @@ static ptycho_status tune_staged_chunk(ptycho_plan_s* pl, int* best) {
     float t_best = 1e30f;
     for (int r = 0; r < 3 && ce == cudaSuccess; ++r) {
       ce = cudaEventRecord(e0, s);
+      ce = big_groups(p.M, p.K, p.engine == PTYCHO_ENGINE_DM, c, &ba.groups);
       for (int n0 = 0; n0 < p.N && ce == cudaSuccess; n0 += c) {
         ba.n0 = n0;
         ce = launch_big_chunk(ba, std::min(c, p.N - n0), s);
@@ -492,10 +498,11 @@ static ptycho_status build_plan(ptycho_plan_s* pl, const float* intensities, con
   const size_t nerr = pl->big ? (size_t)N * big_row_blocks(M) : (size_t)pl->slots * K;
   PT_CUDA(pl->alloc(&d_errpart, nerr), "alloc error partials");
   float2* d_W = nullptr;
-  float* d_R = nullptr;
+  float *d_R = nullptr, *d_S = nullptr;
   if (pl->big) {
     PT_CUDA(pl->alloc(&d_W, (size_t)pl->chunk * K * MM), "alloc staged scratch");
     PT_CUDA(pl->alloc(&d_R, (size_t)pl->chunk * MM), "alloc staged ratios");
+    PT_CUDA(pl->alloc(&d_S, (size_t)pl->chunk * MM), "alloc staged mode sums");
   }
 
   // object tiles and their position lists (increasing n)
@@ -653,6 +660,7 @@ static ptycho_status build_plan(ptycho_plan_s* pl, const float* intensities, con
   ba.hq = d_hq;
   ba.W = d_W;
   ba.R = d_R;
+  ba.S = d_S;
   ba.cn = d_cn;
   ba.pacc = d_pacc;
   ba.dacc = d_dacc;
@@ -675,7 +683,8 @@ static ptycho_status build_plan(ptycho_plan_s* pl, const float* intensities, con
     }
     pl->chunk = std::min(c, pl->chunk);  // a chunk holds at most N positions; buffers hold the largest
     pl->slots = pl->chunk;
-    if (p.engine != PTYCHO_ENGINE_DM) pl->ua.slots = pl->chunk;
+    PT_CUDA(big_groups(M, K, p.engine == PTYCHO_ENGINE_DM, pl->chunk, &pl->ba.groups), "occupancy of the final pass");
+    if (p.engine != PTYCHO_ENGINE_DM) pl->ua.slots = pl->ba.groups;
   }
   return PTYCHO_OK;
 }
@@ -727,11 +736,12 @@ static ptycho_status enqueue_batch(ptycho_plan_s* pl, const FusedArgs& fa, const
     ba.O = fa.O;
     ba.P = fa.P;
     ba.n_first = s0;
+    ba.groups = std::min(ba.groups, len);
     for (int n0 = s0; n0 < s0 + len; n0 += pl->chunk) {
       ba.n0 = n0;
       PT_CUDA(launch_big_chunk(ba, std::min(pl->chunk, s0 + len - n0), s), "staged pass launch");
     }
-    ub.slots = std::min(pl->chunk, len);
+    ub.slots = ba.groups;
     ub.errpart = ua.errpart + (size_t)s0 * big_row_blocks(pl->p.M);
     ub.nerr = len * big_row_blocks(pl->p.M);
   } else {
@@ -1035,14 +1045,14 @@ ptycho_status ptycho_iterate(ptycho_plan_t pl, void* object, void* probe, int32_
   return PTYCHO_OK;
 }
 
-// Chunk list of a class for chunk length L: (member position in the class, first position, end,
-// partial index), members in order; sets each member's partial count (<= what its buffers hold).
+// Work items of a class for chunk length L: (member position in the class, first position, end,
+// partial index), members in order, qc.split items per chunk.
 static std::vector<int4> chunk_list(ptycho_plan_s* pl, ptycho_plan_s::QueueClass& qc, int L) {
   std::vector<int4> chunks;
   for (size_t j = 0; j < qc.members.size(); ++j) {
     const ptycho_plan_s* m = pl->members[qc.members[j]];
-    const int parts = (m->p.N + L - 1) / L;
-    for (int c = 0; c < parts; ++c) chunks.push_back(make_int4((int)j, c * L, std::min(m->p.N, (c + 1) * L), c));
+    const int len = L / qc.split, parts = (m->p.N + len - 1) / len;
+    for (int c = 0; c < parts; ++c) chunks.push_back(make_int4((int)j, c * len, std::min(m->p.N, (c + 1) * len), c));
   }
   return chunks;
 }
@@ -1050,12 +1060,14 @@ static std::vector<int4> chunk_list(ptycho_plan_s* pl, ptycho_plan_s::QueueClass
 static cudaError_t st_apply_chunk_length(ptycho_plan_s* pl, ptycho_plan_s::QueueClass& qc, int L, int max_slots) {
   const std::vector<int4> chunks = chunk_list(pl, qc, L);
   qc.chunk_len = L;
-  qc.nchunks = (int)chunks.size();
-  qc.slots = std::min(max_slots, qc.nchunks);
+  qc.nitems = (int)chunks.size();
+  qc.slots = std::min(max_slots, qc.nitems);
+  qc.nchunks = 0;
   const cudaError_t e = h2d(pl->stream, qc.d_chunks, chunks.data(), sizeof(int4) * chunks.size());
   for (int b : qc.members) {
     ptycho_plan_s* m = pl->members[b];
-    m->parts = (m->p.N + L - 1) / L;
+    qc.nchunks += (m->p.N + L - 1) / L;
+    m->parts = (m->p.N + L / qc.split - 1) / (L / qc.split);
     m->slots = m->parts;
     m->ua.slots = m->parts;
     m->ua.nerr = m->parts * m->p.K;
@@ -1187,6 +1199,16 @@ ptycho_status ptycho_plan_batch(int32_t B, const ptycho_params* const* params, c
     pl->qclasses[ci].members.push_back(b);
     member_class[b] = ci;
   }
+  for (auto& qc : pl->qclasses) {
+    int max_slots = 0, chunks = 0;
+    const cudaError_t oe = fused_queue_max_slots(qc.M, qc.K, &max_slots);
+    if (oe != cudaSuccess) {
+      delete pl;
+      return cuda_fail(oe, "occupancy of the work-queue kernel");
+    }
+    for (int b : qc.members) chunks += (params[b]->N + kQueueChunkMin - 1) / kQueueChunkMin;
+    while (qc.split < kQueueChunkMin && chunks * qc.split < max_slots) qc.split *= 2;
+  }
   pl->queued.assign(B, 0);
   for (int b = 0; b < B; ++b) {
     ptycho_status st = PTYCHO_OK;
@@ -1201,8 +1223,9 @@ ptycho_status ptycho_plan_batch(int32_t B, const ptycho_params* const* params, c
       m->iter = params[b]->start_iteration;
       m->device = pl->device;
       if (member_class[b] >= 0) {
-        const int L = pl->qclasses[member_class[b]].chunk_len;
-        m->parts = (m->p.N + L - 1) / L;
+        const auto& qc = pl->qclasses[member_class[b]];
+        const int len = qc.chunk_len / qc.split;
+        m->parts = (m->p.N + len - 1) / len;
         pl->queued[b] = 1;
       }
       st = build_plan(m, intensities[b], positions[b]);
@@ -1308,7 +1331,7 @@ ptycho_status ptycho_iterate_batch(ptycho_plan_t pl, void* const* objects, void*
         FusedArgs fa = pl->members[qc.members[0]]->fa;
         fa.probs = descs[c];
         fa.chunks = qc.d_chunks;
-        fa.nchunks = qc.nchunks;
+        fa.nchunks = qc.nitems;
         fa.queue = qc.d_queue;
         fa.kh = qc.kh;
         if (ce == cudaSuccess) ce = launch_fused_queue(qc.M, fa, qc.slots, bs);
@@ -1402,7 +1425,8 @@ ptycho_status ptycho_batch_classes(ptycho_plan_t pl, int32_t max_classes, int32_
   *count = (int32_t)pl->qclasses.size();
   for (int c = 0; c < std::min<int>(max_classes, *count); ++c) {
     const auto& qc = pl->qclasses[c];
-    const int32_t v[8] = {qc.M, qc.K, qc.near, qc.kh, (int32_t)qc.members.size(), qc.chunk_len, qc.nchunks, qc.slots};
+    const int32_t v[8] = {qc.M, qc.K, qc.near, qc.kh, (int32_t)qc.members.size(), qc.chunk_len, qc.nchunks,
+                          (qc.slots + qc.split - 1) / qc.split};
     std::memcpy(out + 8 * c, v, sizeof(v));
   }
   return PTYCHO_OK;

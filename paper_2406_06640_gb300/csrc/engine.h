@@ -83,11 +83,13 @@ struct BigArgs {
   const float2* hq;   // near field: h[u]
   float2* W;          // C x K x M x M scratch
   float* R;           // C x M x M modulus ratios
+  float* S;           // C x M x M mode sums of the detector intensity
   int n0;             // first position of the chunk
   int n_first;        // first position of the current accumulation (its chunk restarts the partials)
   float2* cn;         // N x M x M contributions
-  float2* pacc;       // C x K x M x M probe partials (slot = position within the chunk)
-  float* dacc;        // C x M x M
+  float2* pacc;       // groups x K x M x M probe partials (big_groups)
+  float* dacc;        // groups x M x M
+  int groups;         // groups of positions the partials of this accumulation are split into
   double* errpart;    // N x big_row_blocks(M) error partials
   // pc-DM: exit-wave state (N x K x M x M) or null; dm_init: the state starts at P o_n this pass
   float2* psi;
@@ -97,6 +99,8 @@ struct BigArgs {
 // the staged passes of one chunk; launch_big_chunk_dm: the two pc-DM sweeps (b.psi set)
 cudaError_t launch_big_chunk(const BigArgs& b, int nc, cudaStream_t s);
 cudaError_t launch_big_chunk_dm(const BigArgs& b, int nc, cudaStream_t s);
+// groups (probe partials) of an accumulation whose first chunk holds nc positions
+cudaError_t big_groups(int M, int K, bool dm, int nc, int* out);
 int big_row_blocks(int M);  // error partials per position (row blocks of the modulus pass)
 
 // tcgen05 BF16 GEMM (unet_gemm.cu): D[M x Ntot] (+)= A[M x K] . B[Ntot x K]^T, bf16 operands

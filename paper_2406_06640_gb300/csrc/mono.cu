@@ -880,7 +880,8 @@ cudaError_t launch_walk_t(const MonoArgs& a, cudaStream_t s) {
   using SH = WalkShape<TILE, QUAD>;
   auto kern = k_mono_walk<TILE, QUAD, FT>;
   const size_t bytes = SH::bytes(a.J, FT);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  // (the largest any call takes, so that calls of several threads never lower it under one another)
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::LIMIT);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(QUAD ? a.N * 4 : a.N));
