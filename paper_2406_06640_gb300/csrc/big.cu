@@ -150,13 +150,14 @@ __global__ void __launch_bounds__(BigShape<BL>::LINES * BT, BL == 256 ? (OP < 2 
   if constexpr (OP == 0)
 #pragma unroll
     for (int r = 0; r < E; ++r) sum[r] = 0.f;
+  constexpr int UL = OP == 0 ? 4 : BL / BT;  // tile loads in flight per thread (the sums take registers)
   const int k_lo = OP == 0 ? 0 : blockIdx.y, k_hi = OP == 0 ? b.K : k_lo + 1;
   for (int k = k_lo; k < k_hi; ++k) {
     float2* Wk = b.W + ((size_t)c * b.K + k) * MM;
     // coalesced tile load: LINES consecutive columns per row; the far-field backward pass stages the
     // modulus ratio of this position beside it
     const float* Rc = b.R + (size_t)c * MM;
-#pragma unroll 4
+#pragma unroll UL
     for (int i = threadIdx.x; i < BL * LINES; i += LINES * BT) {
       const int yy = i / LINES, xx = i % LINES;
       tile[yy * TP + xx] = Wk[(size_t)yy * BL + x0 + xx];
