@@ -150,46 +150,84 @@ __global__ void k_up2_concat(const bf16* a, const bf16* skip, bf16* q, int n, in
   }
 }
 
-// out (n, h, w, Ca) = bf16( (sum of the 2x2 children of dq[..., :Ca]) + extra[b][c] ) * (act > 0);
-// skip (n, 2h, 2w, Cq - Ca) = dq[..., Ca:]  (FP32 copy, if skip != nullptr)
-__global__ void k_up2_bwd_mask(const float* dq, int Cq, int Ca, const float* extra, const bf16* act, bf16* out,
-                               float* skip, int n, int h, int w) {
-  const size_t total = (size_t)n * h * w * Ca;
+// Backward elementwise kernels: 8 channels (16 bytes of bf16) per thread, so that each runs at the memory
+// rate (one element per thread spent its time on index divisions and 2- and 4-byte accesses: 100, 80
+// and 62 us for the three at S = 128, C = 32, 64 patterns).
+__device__ __forceinline__ void load8(const float* p, float (&f)[8]) {
+  const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
+  f[0] = a.x, f[1] = a.y, f[2] = a.z, f[3] = a.w;
+  f[4] = b.x, f[5] = b.y, f[6] = b.z, f[7] = b.w;
+}
+// bf16(s) where the activation is positive, else 0
+__device__ __forceinline__ uint4 relu_mask8(const float (&s)[8], const uint4& act) {
+  float a[8], r[8];
+  bf8_to_f(act, a);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) r[k] = a[k] > 0.f ? s[k] : 0.f;
+  return f_to_bf8(r);
+}
+
+// out (n, h, w, Ca) = bf16( (sum of the 2x2 children of dq[..., :Ca]) + extra[b][c] ) * (act > 0), dq (n, 2h,
+// 2w, Cq). The skip part dq[..., Ca:] stays where it is (k_pool_bwd_mask reads it there)
+__global__ void k_up2_bwd_mask(const float* dq, int Cq, int Ca, const float* extra, const bf16* act, bf16* out, int n,
+                               int h, int w) {
+  const int A8 = Ca / 8;
+  const size_t total = (size_t)n * h * w * A8;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    const int c = i % Ca;
-    const size_t p = i / Ca;
-    const int x = p % w, y = (p / w) % h, b = p / ((size_t)w * h);
+    const int c = (int)(i % A8) * 8;
+    const int p = (int)(i / A8);
+    const int x = p % w, y = (p / w) % h, b = p / (w * h);
     const size_t f = (((size_t)b * 2 * h + 2 * y) * 2 * w + 2 * x) * Cq + c;
-    float s = dq[f] + dq[f + Cq] + dq[f + (size_t)2 * w * Cq] + dq[f + (size_t)2 * w * Cq + Cq];
-    if (extra) s += extra[(size_t)b * Ca + c];
-    out[i] = __float2bfloat16(__bfloat162float(act[i]) > 0.f ? s : 0.f);
-  }
-  const int Cs = Cq - Ca;
-  if (skip) {
-    const size_t ts = (size_t)n * 2 * h * 2 * w * Cs;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < ts; i += (size_t)gridDim.x * blockDim.x)
-      skip[i] = dq[(i / Cs) * Cq + Ca + i % Cs];
+    float s[8], t[8];
+    load8(dq + f, s);
+    load8(dq + f + Cq, t);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s[k] += t[k];
+    load8(dq + f + (size_t)2 * w * Cq, t);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s[k] += t[k];
+    load8(dq + f + (size_t)2 * w * Cq + Cq, t);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s[k] += t[k];
+    if (extra) {
+      load8(extra + (size_t)b * Ca + c, t);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) s[k] += t[k];
+    }
+    reinterpret_cast<uint4*>(out)[i] = relu_mask8(s, reinterpret_cast<const uint4*>(act)[i]);
   }
 }
 
-// out (n, H, W, C) = bf16( (dp[b][y/2][x/2][c] / 4 + skip) * (act > 0) )
-__global__ void k_pool_bwd_mask(const float* dp, const float* skip, const bf16* act, bf16* out, int n, int H, int W,
-                                int C) {
-  const size_t total = (size_t)n * H * W * C;
+// out (n, H, W, C) = bf16( (dp[b][y/2][x/2][c] / 4 + skip) * (act > 0) ), skip = dq[..., Ca:] of a (n, H, W, Cq)
+// gradient, or none
+__global__ void k_pool_bwd_mask(const float* dp, const float* dq, int Cq, int Ca, const bf16* act, bf16* out, int n,
+                                int H, int W, int C) {
+  const int C8 = C / 8;
+  const size_t total = (size_t)n * H * W * C8;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    const int c = i % C;
-    const size_t p = i / C;
-    const int x = p % W, y = (p / W) % H, b = p / ((size_t)W * H);
-    float s = 0.25f * dp[(((size_t)b * (H / 2) + y / 2) * (W / 2) + x / 2) * C + c];
-    if (skip) s += skip[i];
-    out[i] = __float2bfloat16(__bfloat162float(act[i]) > 0.f ? s : 0.f);
+    const int c = (int)(i % C8) * 8;
+    const int p = (int)(i / C8);
+    const int x = p % W, y = (p / W) % H, b = p / (W * H);
+    float s[8], t[8];
+    load8(dp + (((size_t)b * (H / 2) + y / 2) * (W / 2) + x / 2) * C + c, s);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s[k] *= 0.25f;
+    if (dq) {
+      load8(dq + (size_t)p * Cq + Ca + c, t);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) s[k] += t[k];
+    }
+    reinterpret_cast<uint4*>(out)[i] = relu_mask8(s, reinterpret_cast<const uint4*>(act)[i]);
   }
 }
 
-// out = bf16(d * (act > 0)), d with row stride ld (first C channels)
-__global__ void k_mask(const float* d, const bf16* act, bf16* out, size_t npix, int C) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < npix * C; i += (size_t)gridDim.x * blockDim.x)
-    out[i] = __float2bfloat16(__bfloat162float(act[i]) > 0.f ? d[i] : 0.f);
+// out = bf16(d * (act > 0)), `total` groups of 8 channels
+__global__ void k_mask(const float* d, const bf16* act, bf16* out, size_t total) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+    float s[8];
+    load8(d + 8 * i, s);
+    reinterpret_cast<uint4*>(out)[i] = relu_mask8(s, reinterpret_cast<const uint4*>(act)[i]);
+  }
 }
 
 // colT[k][p] of the zero-padded 3x3 neighbourhoods of X (n, H, W, Cin): k = tap * Cin + c < 9 Cin,
@@ -222,56 +260,116 @@ __global__ void k_im2colT(const bf16* X, bf16* colT, int n, int H, int W, int Ci
   }
 }
 
-// XT3[d][c][p] = X[p + d - 1][c] when pixel x + d - 1 lies in [0, W), else 0 (d = 0, 1, 2);
-// X (Mpix, Cin) NHWC; 32 pixels x 32 channels per block through shared memory
-__global__ void k_shift3T(const bf16* X, bf16* XT3, int Mpix, int W, int Cin) {
-  __shared__ bf16 tile[34][33];
-  const int p0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
-  for (int i = threadIdx.y * 32 + threadIdx.x; i < 34 * 32; i += 256) {
-    const int j = i / 32, c = c0 + i % 32, p = p0 - 1 + j;
-    tile[j][i % 32] = (p >= 0 && p < Mpix && c < Cin) ? X[(size_t)p * Cin + c] : __float2bfloat16(0.f);
+// Channel-major copies for the weight gradients: tiles of 128 pixels x CT channels through shared memory,
+// 16-byte loads (8 channels of a pixel) and stores (8 pixels of a channel); 2-byte stores of 32-pixel tiles
+// took 57 and 28 us on average over the seven layers at S = 128, C = 32, 64 patterns.
+constexpr int kTilePix = 128;
+
+// XT3[d][c][p] = X[p + d - 1][c] when pixel x + d - 1 lies in [0, W), else 0 (d = 0, 1, 2); X (Mpix, Cin) NHWC,
+// Mpix a multiple of 128, W of 8 (the 8 pixels of a store share an image row). grid (Mpix / 128, Cin / CT)
+template <int CT>
+__global__ void __launch_bounds__(128) k_shift3T(const bf16* X, bf16* XT3, int Mpix, int W, int Cin) {
+  constexpr int LD = kTilePix + 6;  // pixels p0 - 1 .. p0 + 128 of a channel
+  __shared__ bf16 tile[CT][LD];
+  const int p0 = blockIdx.x * kTilePix, c0 = blockIdx.y * CT;
+  for (int i = threadIdx.x; i < (kTilePix + 2) * (CT / 8); i += 128) {
+    const int j = i / (CT / 8), g = i % (CT / 8), p = p0 - 1 + j;
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (p >= 0 && p < Mpix) v = *reinterpret_cast<const uint4*>(X + (size_t)p * Cin + c0 + 8 * g);
+    const bf16* h = reinterpret_cast<const bf16*>(&v);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) tile[8 * g + k][j] = h[k];
   }
   __syncthreads();
-  const int j = threadIdx.x, p = p0 + j, x = p % W;
-  for (int cc = threadIdx.y; cc < 32; cc += 8) {
-    const int c = c0 + cc;
-    if (c >= Cin || p >= Mpix) continue;
+  for (int i = threadIdx.x; i < CT * (kTilePix / 8); i += 128) {
+    const int cc = i / (kTilePix / 8), q = (i % (kTilePix / 8)) * 8;  // pixels p0 + q ..
+    const int p = p0 + q, x = p % W;
+    bf16 v[10];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const int xx = x + d - 1;
-      XT3[((size_t)d * Cin + c) * Mpix + p] = (xx >= 0 && xx < W) ? tile[j + d][cc] : __float2bfloat16(0.f);
+    for (int k = 0; k < 10; ++k) v[k] = tile[cc][q + k];
+    if (x == 0) v[0] = __float2bfloat16(0.f);
+    if (x + 8 == W) v[9] = __float2bfloat16(0.f);
+#pragma unroll
+    for (int dd = 0; dd < 3; ++dd) {
+      __align__(16) bf16 o[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) o[k] = v[k + dd];
+      *reinterpret_cast<uint4*>(XT3 + ((size_t)dd * Cin + c0 + cc) * Mpix + p) = *reinterpret_cast<const uint4*>(o);
     }
   }
 }
 
-// out[o] = sum over p of dYT[o][p] in a fixed order (one block per output channel)
-__global__ void k_bias_grad(const bf16* dYT, int M, float* out) {
-  __shared__ float red[256];
-  const int o = blockIdx.x;
-  float s = 0.f;
-  for (int p = threadIdx.x; p < M; p += 256) s += __bfloat162float(dYT[(size_t)o * M + p]);
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
+// dst[c][p] = src[p][c], bf16, Mpix x C, Mpix a multiple of 128, C of 16. grid (Mpix / 128, C / 16)
+__global__ void __launch_bounds__(128) k_transpose(const bf16* src, bf16* dst, int Mpix, int C) {
+  constexpr int CT = 16, LD = kTilePix + 2;
+  __shared__ bf16 tile[CT][LD];
+  const int p0 = blockIdx.x * kTilePix, c0 = blockIdx.y * CT;
+  for (int i = threadIdx.x; i < kTilePix * 2; i += 128) {
+    const int j = i / 2, g = i % 2;
+    const uint4 v = *reinterpret_cast<const uint4*>(src + (size_t)(p0 + j) * C + c0 + 8 * g);
+    const bf16* h = reinterpret_cast<const bf16*>(&v);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) tile[8 * g + k][j] = h[k];
   }
-  if (threadIdx.x == 0) out[(size_t)o] = red[0];
+  __syncthreads();
+  for (int i = threadIdx.x; i < CT * (kTilePix / 8); i += 128) {
+    const int cc = i / (kTilePix / 8), q = (i % (kTilePix / 8)) * 8;
+    __align__(16) bf16 o[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) o[k] = tile[cc][q + k];
+    *reinterpret_cast<uint4*>(dst + (size_t)(c0 + cc) * Mpix + p0 + q) = *reinterpret_cast<const uint4*>(o);
+  }
 }
 
-// dst[c][r] = src[r][c], bf16, R x C
-__global__ void k_transpose(const bf16* src, bf16* dst, int R, int C) {
-  __shared__ bf16 tile[32][33];
-  const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
-  for (int r = threadIdx.y; r < 32; r += 8) {
-    const int rr = r0 + r, cc = c0 + threadIdx.x;
-    tile[r][threadIdx.x] = (rr < R && cc < C) ? src[(size_t)rr * C + cc] : __float2bfloat16(0.f);
+// out[o] = sum over p of dYT[o][p] in a fixed order (one block per output channel, thread t the pixels t,
+// t + 256, ..., then a tree). The order leaves 256 chains per channel, so the loads have to run far ahead of
+// the sums: the channel's pixels pass through two shared-memory buffers of 32768 (16-byte asynchronous
+// copies; 2-byte loads in the chain took 47 us on average over the layers). M a multiple of 8
+constexpr int kBiasChunk = 32768;
+__global__ void __launch_bounds__(256) k_bias_grad(const bf16* dYT, int M, float* out) {
+  extern __shared__ __align__(16) unsigned char smem_bias[];
+  bf16* buf = reinterpret_cast<bf16*>(smem_bias);  // 2 x kBiasChunk
+  __shared__ float red[256];
+  const int o = blockIdx.x, t = threadIdx.x;
+  const bf16* row = dYT + (size_t)o * M;
+  const int chunks = (M + kBiasChunk - 1) / kBiasChunk;
+  auto fetch = [&](int ch) {
+    const int base = ch * kBiasChunk, len = min(kBiasChunk, M - base);
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(buf + (ch & 1) * kBiasChunk);
+    for (int i = t * 8; i < len; i += 256 * 8)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 2u * i), "l"(row + base + i) : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  fetch(0);
+  float s = 0.f;
+  for (int ch = 0; ch < chunks; ++ch) {
+    if (ch + 1 < chunks) {
+      fetch(ch + 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();  // every thread's copies of this chunk have landed
+    const bf16* b = buf + (ch & 1) * kBiasChunk;
+    const int len = min(kBiasChunk, M - ch * kBiasChunk);
+    int p = t;
+    for (; p + 15 * 256 < len; p += 16 * 256) {
+      float v[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = __bfloat162float(b[p + 256 * k]);
+#pragma unroll
+      for (int k = 0; k < 16; ++k) s += v[k];
+    }
+    for (; p < len; p += 256) s += __bfloat162float(b[p]);
+    __syncthreads();  // the buffer is refilled by the next but one chunk
   }
+  red[t] = s;
   __syncthreads();
-  for (int c = threadIdx.y; c < 32; c += 8) {
-    const int cc = c0 + c, rr = r0 + threadIdx.x;
-    if (rr < R && cc < C) dst[(size_t)cc * R + rr] = tile[threadIdx.x][c];
+  for (int w = 128; w > 0; w >>= 1) {
+    if (t < w) red[t] += red[t + w];
+    __syncthreads();
   }
+  if (t == 0) out[(size_t)o] = red[0];
 }
 
 // master weights -> forward operand wb [Cp][Kf] and data-gradient operand wr [Cin][Kd]:
@@ -295,20 +393,41 @@ __global__ void k_weights_bf16(const float* w, bf16* wb, bf16* wr, int Cp, int C
   }
 }
 
-// out (Mo, 16) fp32, first 2 channels used; target (Mo, 2). d_out bf16 (Mo, 16); per-block loss partials
-__global__ void k_loss(const float* out, const float* target, bf16* d_out, float* partial, int Mo) {
+// out (Mo, 16) fp32, first 2 channels used; target (Mo, 2). d_out bf16 (Mo, 16), one pixel per thread
+__global__ void k_loss_grad(const float* out, const float* target, bf16* d_out, int Mo) {
+  const float inv = 1.0f / (2.0f * Mo);
+  uint4* d4 = reinterpret_cast<uint4*>(d_out);
+  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < Mo; p += gridDim.x * blockDim.x) {
+    const float2 o = *reinterpret_cast<const float2*>(out + (size_t)p * 16);
+    const float2 t = reinterpret_cast<const float2*>(target)[p];
+    const float d0 = o.x - t.x, d1 = o.y - t.y;
+    float g[8] = {2.f * d0 * inv, 2.f * d1 * inv, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    d4[2 * (size_t)p] = f_to_bf8(g);
+    d4[2 * (size_t)p + 1] = make_uint4(0u, 0u, 0u, 0u);
+  }
+}
+
+// per-block loss partials (64 blocks of 256): thread i sums the elements i, i + 16384, ... of (Mo, 16), of
+// which channels 0 and 1 count; the loads run eight ahead of the chain of sums
+__global__ void __launch_bounds__(256) k_loss(const float* out, const float* target, float* partial, int Mo) {
   __shared__ float red[256];
   float s = 0.f;
   const float inv = 1.0f / (2.0f * Mo);
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Mo * 16; i += gridDim.x * blockDim.x) {
-    const int p = i / 16, c = i % 16;
-    float g = 0.f;
-    if (c < 2) {
-      const float d = out[i] - target[p * 2 + c];
-      s += d * d;
-      g = 2.f * d * inv;
+  const int first = blockIdx.x * 256 + threadIdx.x, c = first % 16;
+  const int stride = gridDim.x * 256;  // a multiple of 16
+  if (c < 2) {
+    int i = first;
+    for (; i + 7 * stride < Mo * 16; i += 8 * stride) {
+      float d[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) d[k] = out[i + k * stride] - target[(i + k * stride) / 16 * 2 + c];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) s += d[k] * d[k];
     }
-    d_out[i] = __float2bfloat16(g);
+    for (; i < Mo * 16; i += stride) {
+      const float d = out[i] - target[i / 16 * 2 + c];
+      s += d * d;
+    }
   }
   red[threadIdx.x] = s;
   __syncthreads();
@@ -420,7 +539,15 @@ __global__ void k_extract2(const float* out, float* dst, int Mo) {
 __global__ void k_sum_splits(const float* part, int ks, size_t count, float* out) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x) {
     float s = 0.f;
-    for (int z = 0; z < ks; ++z) s += part[(size_t)z * count + i];
+    int z = 0;
+    for (; z + 16 <= ks; z += 16) {  // the loads ahead of the chain of sums
+      float v[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = part[(size_t)(z + k) * count + i];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) s += v[k];
+    }
+    for (; z < ks; ++z) s += part[(size_t)z * count + i];
     out[i] = s;
   }
 }
@@ -476,7 +603,7 @@ struct ptycho_unet_s {
   bf16 *xn, *w0n, *w0np;
   float *out, *g, *sigma, *extra, *loss_part, *loss_s;
   bf16 *d_out, *dY, *dYT, *colT, *xt3;
-  float *dX, *skip1, *skip2;
+  float *dX, *dq1, *dq2;  // data gradients; of the two concatenations (their skip parts are read later)
   float* wpart;  // split-K partial weight gradients
   int* status;
   bool wb_fresh = false;  // the bf16 weight copies match the FP32 masters
@@ -590,12 +717,14 @@ cudaError_t conv_forward(ptycho_unet_s* u, Conv& L, const bf16* in, bf16* out_bf
 cudaError_t conv_backward(ptycho_unet_s* u, Conv& L, const bf16* in, const bf16* dY, float* dX) {
   const int M = u->nrun * L.H * L.W;
   cudaStream_t s = u->stream;
-  k_transpose<<<dim3((M + 31) / 32, (L.Cp + 31) / 32), dim3(32, 8), 0, s>>>(dY, u->dYT, M, L.Cp);
+  k_transpose<<<dim3(M / kTilePix, L.Cp / 16), 128, 0, s>>>(dY, u->dYT, M, L.Cp);
   const Split sp = wgrad_split(L.Kw, L.Cp, M);
   const bool shifted = L.W % 8 == 0;  // transposed shifted copies (else the explicit neighbourhood matrix)
   cudaError_t e;
-  if (shifted)
-    k_shift3T<<<dim3(M / 32, (L.Cin + 31) / 32), dim3(32, 8), 0, s>>>(in, u->xt3, M, L.W, L.Cin);
+  if (shifted && L.Cin % 16 == 0)
+    k_shift3T<16><<<dim3(M / kTilePix, L.Cin / 16), 128, 0, s>>>(in, u->xt3, M, L.W, L.Cin);
+  else if (shifted)
+    k_shift3T<8><<<dim3(M / kTilePix, L.Cin / 8), 128, 0, s>>>(in, u->xt3, M, L.W, L.Cin);
   else
     k_im2colT<<<dim3((M + 31) / 32, L.Kw / 32), dim3(32, 8), 0, s>>>(in, u->colT, u->nrun, L.H, L.W, L.Cin, L.Kw);
   float* D = sp.ks > 1 ? u->wpart : L.gT;
@@ -604,7 +733,12 @@ cudaError_t conv_backward(ptycho_unet_s* u, Conv& L, const bf16* in, const bf16*
   if (e != cudaSuccess) return e;
   if (sp.ks > 1) k_sum_splits<<<grid_for((size_t)L.Kw * L.Cp), 256, 0, s>>>(u->wpart, sp.ks, (size_t)L.Kw * L.Cp, L.gT);
   // bias gradient (row 9 Cin of gT); the explicit matrix's row of ones already produced it
-  if (shifted) k_bias_grad<<<L.Cp, 256, 0, s>>>(u->dYT, M, L.gT + (size_t)9 * L.Cin * L.Cp);
+  if (shifted) {
+    constexpr int bytes = 2 * kBiasChunk * (int)sizeof(bf16);
+    if ((e = cudaFuncSetAttribute(k_bias_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess)
+      return e;
+    k_bias_grad<<<L.Cp, 256, bytes, s>>>(u->dYT, M, L.gT + (size_t)9 * L.Cin * L.Cp);
+  }
   if (e != cudaSuccess || !dX) return e;
   Conv R = L;  // the data gradient gathers dY with Cp channels
   R.Cin = L.Cp;
@@ -681,28 +815,29 @@ static cudaError_t unet_backward(ptycho_unet_s* u, const float* target, const fl
   cudaStream_t s = u->stream;
   const int n = u->nrun, S = u->S, C = u->C;
   const int Mo = n * (S / 2) * (S / 2);
-  k_loss<<<64, 256, 0, s>>>(u->out, target, u->d_out, u->loss_part, Mo);
+  k_loss_grad<<<grid_for(Mo), 256, 0, s>>>(u->out, target, u->d_out, Mo);
+  k_loss<<<64, 256, 0, s>>>(u->out, target, u->loss_part, Mo);
   k_sigma_pool<<<n, 1024, 0, s>>>(u->a3, u->g, (S / 8) * (S / 8), 8 * C);
   k_sigma_head<<<1, kMaxBatch, 0, s>>>(u->w7, u->b7, sigma_t, lam, u->sigma, u->g, u->extra, u->gw7, u->gb7,
                                   u->loss_s, n, (S / 8) * (S / 8), 8 * C, 1);
   cudaError_t e;
   // head and a5
   if ((e = conv_backward(u, u->L[6], u->a5, u->d_out, u->dX)) != cudaSuccess) return e;
-  k_mask<<<grid_for((size_t)Mo * 2 * C), 256, 0, s>>>(u->dX, u->a5, u->dY, (size_t)Mo, 2 * C);
-  if ((e = conv_backward(u, u->L[5], u->q1, u->dY, u->dX)) != cudaSuccess) return e;  // dX = d q1 (6C)
-  k_up2_bwd_mask<<<grid_for((size_t)n * (S / 4) * (S / 4) * 4 * C), 256, 0, s>>>(
-      u->dX, 6 * C, 4 * C, nullptr, u->a4, u->dY, u->skip1, n, S / 4, S / 4);
-  if ((e = conv_backward(u, u->L[4], u->q2, u->dY, u->dX)) != cudaSuccess) return e;  // dX = d q2 (12C)
-  k_up2_bwd_mask<<<grid_for((size_t)n * (S / 8) * (S / 8) * 8 * C), 256, 0, s>>>(
-      u->dX, 12 * C, 8 * C, u->extra, u->a3, u->dY, u->skip2, n, S / 8, S / 8);
+  k_mask<<<grid_for((size_t)Mo * 2 * C / 8), 256, 0, s>>>(u->dX, u->a5, u->dY, (size_t)Mo * 2 * C / 8);
+  if ((e = conv_backward(u, u->L[5], u->q1, u->dY, u->dq1)) != cudaSuccess) return e;  // d q1 (6C)
+  k_up2_bwd_mask<<<grid_for((size_t)n * (S / 4) * (S / 4) * 4 * C / 8), 256, 0, s>>>(u->dq1, 6 * C, 4 * C, nullptr,
+                                                                                     u->a4, u->dY, n, S / 4, S / 4);
+  if ((e = conv_backward(u, u->L[4], u->q2, u->dY, u->dq2)) != cudaSuccess) return e;  // d q2 (12C)
+  k_up2_bwd_mask<<<grid_for((size_t)n * (S / 8) * (S / 8) * 8 * C / 8), 256, 0, s>>>(
+      u->dq2, 12 * C, 8 * C, u->extra, u->a3, u->dY, n, S / 8, S / 8);
   if ((e = conv_backward(u, u->L[3], u->p2, u->dY, u->dX)) != cudaSuccess) return e;  // d p2 (4C)
-  k_pool_bwd_mask<<<grid_for((size_t)n * (S / 4) * (S / 4) * 4 * C), 256, 0, s>>>(u->dX, u->skip2, u->a2, u->dY, n,
-                                                                                   S / 4, S / 4, 4 * C);
+  k_pool_bwd_mask<<<grid_for((size_t)n * (S / 4) * (S / 4) * 4 * C / 8), 256, 0, s>>>(
+      u->dX, u->dq2, 12 * C, 8 * C, u->a2, u->dY, n, S / 4, S / 4, 4 * C);
   if ((e = conv_backward(u, u->L[2], u->p1, u->dY, u->dX)) != cudaSuccess) return e;  // d p1 (2C)
-  k_pool_bwd_mask<<<grid_for((size_t)n * (S / 2) * (S / 2) * 2 * C), 256, 0, s>>>(u->dX, u->skip1, u->a1, u->dY, n,
-                                                                                   S / 2, S / 2, 2 * C);
+  k_pool_bwd_mask<<<grid_for((size_t)n * (S / 2) * (S / 2) * 2 * C / 8), 256, 0, s>>>(
+      u->dX, u->dq1, 6 * C, 4 * C, u->a1, u->dY, n, S / 2, S / 2, 2 * C);
   if ((e = conv_backward(u, u->L[1], u->p0, u->dY, u->dX)) != cudaSuccess) return e;  // d p0 (C)
-  k_pool_bwd_mask<<<grid_for((size_t)n * S * S * C), 256, 0, s>>>(u->dX, nullptr, u->a0, u->dY, n, S, S, C);
+  k_pool_bwd_mask<<<grid_for((size_t)n * S * S * C / 8), 256, 0, s>>>(u->dX, nullptr, 0, 0, u->a0, u->dY, n, S, S, C);
   if ((e = conv_backward(u, u->L[0], u->x, u->dY, nullptr)) != cudaSuccess) return e;
   return cudaGetLastError();
 }
@@ -849,9 +984,9 @@ ptycho_status ptycho_unet_create(int32_t S, int32_t C, int32_t batch, uint64_t s
   UA(dYT, px * C);
   UA(colT, colT_max);
   UA(xt3, xt3_max);
-  UA(dX, std::max(px * C, px * 6 * C / 4));
-  UA(skip1, px * 2 * C / 4);
-  UA(skip2, px * 4 * C / 16);
+  UA(dX, px * 2 * C / 4);  // the largest of a5, p2, p1 and p0
+  UA(dq1, px * 6 * C / 4);
+  UA(dq2, px * 12 * C / 16);
   UA(wpart, wpart_max);
   UA(status, 1);
 #undef UA
