@@ -183,7 +183,8 @@ struct ptycho_plan_s {
   static constexpr int kGraphAfter = 2, kRing = 4, kMaxGraphKeys = 32;  // beyond: eager
   std::vector<SingleGraph> sgraphs;
   std::vector<std::pair<std::array<uintptr_t, 3>, int>> eager_runs;
-  cudaStream_t gstream = nullptr;
+  cudaStream_t gstream = nullptr, gside = nullptr;  // capture streams: the iteration, and its side branch
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int ring = 0;
   // mini-batch plans: one graph per batch (its fused launch or staged passes and its update), keyed
   // by (batch, probe step on, object, probe) and replayed in each iteration's visiting order
@@ -210,6 +211,9 @@ struct ptycho_plan_s {
       if (g.e1) cudaEventDestroy(g.e1);
     }
     if (gstream) cudaStreamDestroy(gstream);
+    if (gside) cudaStreamDestroy(gside);
+    if (ev_fork) cudaEventDestroy(ev_fork);
+    if (ev_join) cudaEventDestroy(ev_join);
     for (cudaEvent_t e : branch_ev) cudaEventDestroy(e);
     for (cudaStream_t s : branch) cudaStreamDestroy(s);
     if (ev_in) cudaEventDestroy(ev_in);
@@ -368,6 +372,14 @@ static void append_tile_lists(const std::vector<int2>& pos, int n0, int n1, int 
     for (int n : l) flat.push_back(make_int4(n, pos[n].x, pos[n].y, 0));
   }
   start.push_back((int)flat.size());
+}
+
+// average length of the non-empty lists of one or more CSR offset arrays (batches follow one another, so
+// offsets only grow) against the line between the two forms of the gather (k_gather)
+static bool long_lists(const std::vector<int>& start) {
+  long long used = 0;
+  for (size_t i = 0; i + 1 < start.size(); ++i) used += start[i + 1] > start[i] ? 1 : 0;
+  return used > 0 && (long long)start.back() >= 24 * used;
 }
 
 static ptycho_status build_plan(ptycho_plan_s* pl, const float* intensities, const int32_t* positions) {
@@ -532,17 +544,17 @@ static ptycho_status build_plan(ptycho_plan_s* pl, const float* intensities, con
 
   const size_t plane = (size_t)p.obj_h * p.obj_w;
   float2* d_no;
-  float *d_do, *d_bmo;
+  float* d_do;
+  int* d_dmax;
   PT_CUDA(pl->alloc(&d_no, plane), "alloc object sums");
   PT_CUDA(pl->alloc(&d_do, plane), "alloc object sums");
-  PT_CUDA(pl->alloc(&d_bmo, (size_t)tx * ty), "alloc tile maxima");
+  PT_CUDA(pl->alloc(&d_dmax, 2), "alloc maxima");
   const int pb = (int)((MM + 255) / 256);
   float2* d_np;
-  float *d_dp, *d_p2, *d_bmp, *d_cbar;
+  float *d_dp, *d_p2, *d_cbar;
   PT_CUDA(pl->alloc(&d_np, (size_t)K * MM), "alloc probe sums");
   PT_CUDA(pl->alloc(&d_dp, MM), "alloc probe sums");
   PT_CUDA(pl->alloc(&d_p2, MM), "alloc probe sums");
-  PT_CUDA(pl->alloc(&d_bmp, (size_t)pb), "alloc probe maxima");
   PT_CUDA(pl->alloc(&d_cbar, (size_t)N), "alloc cbar");
   long long *d_lna, *d_phi, *d_cbar_q;
   PT_CUDA(pl->alloc(&d_lna, (size_t)p.obj_h * (p.obj_w + 1)), "alloc constraint maps");
@@ -609,11 +621,11 @@ static ptycho_status build_plan(ptycho_plan_s* pl, const float* intensities, con
   ua.tiles_y = ty;
   ua.no_part = d_no;
   ua.do_part = d_do;
-  ua.blk_max_o = d_bmo;
+  ua.dmax = d_dmax;
+  ua.split_lists = long_lists(start) ? 1 : 0;
   ua.np_sum = d_np;
   ua.dp_sum = d_dp;
   ua.p2 = d_p2;
-  ua.blk_max_p = d_bmp;
   ua.probe_blocks = pb;
   ua.errhist = pl->d_errhist;
   ua.run_counter = d_runs;
@@ -761,7 +773,7 @@ static ptycho_status enqueue_batch(ptycho_plan_s* pl, const FusedArgs& fa, const
   }
   ub.err_mode = 1;
   ub.err_acc = pl->d_err_acc;
-  PT_CUDA(launch_update(ub, s), "update launch");
+  PT_CUDA(launch_update(ub, nullptr, true, true, s), "update launch");
   return PTYCHO_OK;
 }
 
@@ -825,6 +837,15 @@ static ptycho_status enqueue_iteration(ptycho_plan_s* pl, void* object, void* pr
   ua.O = static_cast<float2*>(object);
   ua.P = static_cast<float2*>(probe);
   ca.O = static_cast<float2*>(object);
+  // in a graph of a single plan the |P|^2 map runs beside the fused kernel (a branch from here to the update)
+  bool p2_done = false;
+  if (pe0 && pl->mb == 0 && !pl->d_psi) {
+    PT_CUDA(cudaEventRecord(pl->ev_fork, s), "fork event");
+    PT_CUDA(cudaStreamWaitEvent(pl->gside, pl->ev_fork, 0), "fork");
+    PT_CUDA(launch_p2(ua, pl->gside), "update launch");
+    PT_CUDA(cudaEventRecord(pl->ev_join, pl->gside), "join event");
+    p2_done = true;
+  }
   const int ps = pl->prof_count % ptycho_plan_s::kProfSlots;
   if (pe0) PT_CUDA(cudaEventRecordWithFlags(pe0, s, cudaEventRecordExternal), "profile event");
   else if (pl->profiling) PT_CUDA(cudaEventRecord(pl->ev[2 * ps], s), "profile event");
@@ -849,7 +870,7 @@ static ptycho_status enqueue_iteration(ptycho_plan_s* pl, void* object, void* pr
       PT_CUDA(cudaEventRecord(pl->ev[2 * ps + 1], s), "profile event");
       pl->prof_count++;
     }
-    if (pl->in_window(t)) PT_CUDA(launch_constraint(ca, s), "constraint launch");
+    if (pl->in_window(t)) PT_CUDA(launch_constraint(ca, true, s), "constraint launch");
     return PTYCHO_OK;
   } else if (pl->big && pl->d_psi) {
     // pc-DM on the staged path: per chunk, the estimate sweep (error) and the chi sweep
@@ -888,23 +909,26 @@ static ptycho_status enqueue_iteration(ptycho_plan_s* pl, void* object, void* pr
     pl->prof_count++;
   }
   ua.update_probe = t >= pl->p.probe_update_start;
+  if (p2_done) PT_CUDA(cudaStreamWaitEvent(s, pl->ev_join, 0), "join");
   if (pl->d_psi) {
     // pc-DM: the complex constraint acts between the object and the probe step, and the states
     // move with their boxes by P (O constrained - O)
-    PT_CUDA(launch_update_object(ua, s), "update launch");
+    const bool win = pl->in_window(t);
+    PT_CUDA(launch_update_object(ua, win ? &ca : nullptr, s), "update launch");
     ua.dm_obj_prev = nullptr;
-    if (pl->in_window(t)) {
+    if (win) {
       PT_CUDA(cudaMemcpyAsync(pl->d_obj_prev, ua.O, (size_t)pl->p.obj_h * pl->p.obj_w * sizeof(float2),
                               cudaMemcpyDeviceToDevice, s),
               "object copy");
-      PT_CUDA(launch_constraint(ca, s), "constraint launch");
+      PT_CUDA(launch_constraint(ca, false, s), "constraint launch");
       ua.dm_obj_prev = pl->d_obj_prev;
     }
-    PT_CUDA(launch_update_probe(ua, s), "update launch");
+    PT_CUDA(launch_update_probe_dm(ua, s), "update launch");
     return PTYCHO_OK;
   }
-  PT_CUDA(launch_update(ua, s), "update launch");
-  if (pl->in_window(t)) PT_CUDA(launch_constraint(ca, s), "constraint launch");
+  const bool win = pl->in_window(t);
+  PT_CUDA(launch_update(ua, win ? &ca : nullptr, !p2_done, true, s), "update launch");
+  if (win) PT_CUDA(launch_constraint(ca, false, s), "constraint launch");
   return PTYCHO_OK;
 }
 
@@ -920,20 +944,22 @@ static ptycho_status enqueue_update(ptycho_plan_s* pl, void* object, void* probe
   if (pl->d_psi) {
     // pc-DM: the complex constraint acts between the object and the probe step, and the states
     // move with their boxes by P (O constrained - O)
-    PT_CUDA(launch_update_object(ua, s), "update launch");
+    const bool win = pl->in_window(t);
+    PT_CUDA(launch_update_object(ua, win ? &ca : nullptr, s), "update launch");
     ua.dm_obj_prev = nullptr;
-    if (pl->in_window(t)) {
+    if (win) {
       PT_CUDA(cudaMemcpyAsync(pl->d_obj_prev, ua.O, (size_t)pl->p.obj_h * pl->p.obj_w * sizeof(float2),
                               cudaMemcpyDeviceToDevice, s),
               "object copy");
-      PT_CUDA(launch_constraint(ca, s), "constraint launch");
+      PT_CUDA(launch_constraint(ca, false, s), "constraint launch");
       ua.dm_obj_prev = pl->d_obj_prev;
     }
-    PT_CUDA(launch_update_probe(ua, s), "update launch");
+    PT_CUDA(launch_update_probe_dm(ua, s), "update launch");
     return PTYCHO_OK;
   }
-  PT_CUDA(launch_update(ua, s), "update launch");
-  if (pl->in_window(t)) PT_CUDA(launch_constraint(ca, s), "constraint launch");
+  const bool win = pl->in_window(t);
+  PT_CUDA(launch_update(ua, win ? &ca : nullptr, true, false, s), "update launch");
+  if (win) PT_CUDA(launch_constraint(ca, false, s), "constraint launch");
   return PTYCHO_OK;
 }
 
@@ -979,6 +1005,9 @@ static ptycho_status iterate_graph(ptycho_plan_s* pl, void* object, void* probe,
   if (gi == pl->sgraphs.size()) {
     // capture the key's whole ring
     if (!pl->gstream) PT_CUDA(cudaStreamCreateWithFlags(&pl->gstream, cudaStreamNonBlocking), "graph stream");
+    if (!pl->gside) PT_CUDA(cudaStreamCreateWithFlags(&pl->gside, cudaStreamNonBlocking), "graph stream");
+    for (cudaEvent_t* ev : {&pl->ev_fork, &pl->ev_join})
+      if (!*ev) PT_CUDA(cudaEventCreateWithFlags(ev, cudaEventDisableTiming), "graph event");
     const bool fresh = pl->dm_fresh;
     const bool prof = pl->profiling;
     pl->profiling = false;  // the ring's own events, not the eager event ring
@@ -1534,17 +1563,18 @@ int32_t ptycho_launches_per_iteration(ptycho_plan_t pl, int32_t in_window) {
   // pc-DM: the estimate sweep stops after the modulus pass (3 far, 4 near)
   const int dm_extra = pl->p.geometry == PTYCHO_NEARFIELD ? 4 : 3;
   if (pl->big) fft = (pl->p.N + pl->chunk - 1) / pl->chunk * (pl->d_psi ? passes + dm_extra : passes);
-  if (pl->mb > 0) {  // per batch: its fused launch or staged passes, and the 4 update kernels; the error
-    fft = -4 + 1;    // finish after the batches
+  // update: |P|^2 map, gather, steps; pc-DM: the gather and the steps once per side, and the probe
+  // partials between them. Constraint: box sums, tile apply (the object step makes the row sums)
+  int update = pl->d_psi ? 6 : 3;
+  if (pl->mb > 0) {  // per batch: its fused launch or staged passes and its update; the error finish after them
+    fft = 1;
     for (int b = 0; b < pl->nb; ++b) {
       const int len = std::min(pl->mb, pl->p.N - b * pl->mb);
-      fft += (pl->big ? (len + pl->chunk - 1) / pl->chunk * passes : 1) + 4;
+      fft += (pl->big ? (len + pl->chunk - 1) / pl->chunk * passes : 1) + update;
     }
+    update = in_window ? 1 : 0;  // the constraint's row sums are a launch of their own
   }
-  if (pl->d_psi) fft += 2;                // pc-DM probe partials and their gather (probe step on)
-  // update: probe gather, object gather (one clustered launch), object step, probe step;
-  // constraint: row prefix sums, box sums, tile apply
-  return fft + 4 + (in_window ? 3 : 0);
+  return fft + update + (in_window ? 2 : 0);
 }
 
 ptycho_status ptycho_permutation(int32_t n, uint64_t seed, int32_t stream, int32_t t, int32_t* out) {
@@ -1620,5 +1650,6 @@ void capi_tile_lists(const std::vector<int2>& pos, int M, int tx, int ty, std::v
 ptycho_status capi_cuda_fail(cudaError_t e, const char* what) { return cuda_fail(e, what); }
 std::vector<double> capi_taps(double sigma, int h) { return taps_1d(sigma, h); }
 bool capi_is_device_pointer(const void* ptr) { return is_device_pointer(ptr); }
+bool capi_long_lists(const std::vector<int>& start) { return long_lists(start); }
 void capi_clear_error() { g_last_error.clear(); }
 }  // namespace ptycho

@@ -30,6 +30,7 @@ std::vector<double> capi_taps(double sigma, int h);
 void capi_tile_lists(const std::vector<int2>& pos, int M, int tx, int ty, std::vector<int>& start,
                      std::vector<int4>& flat);
 bool capi_is_device_pointer(const void* ptr);
+bool capi_long_lists(const std::vector<int>& start);
 void capi_clear_error();
 }  // namespace ptycho
 
@@ -150,11 +151,10 @@ extern "C" ptycho_status ptycho_iterate_static(const ptycho_params* p, const flo
     ua.tile_pos = cv.take<int4>(flat.size());
     ua.no_part = cv.take<float2>(plane);
     ua.do_part = cv.take<float>(plane);
-    ua.blk_max_o = cv.take<float>((size_t)tx * ty);
+    ua.dmax = cv.take<int>(2);
     ua.np_sum = cv.take<float2>((size_t)K * MM);
     ua.dp_sum = cv.take<float>(MM);
     ua.p2 = cv.take<float>(MM);
-    ua.blk_max_p = cv.take<float>((size_t)pb);
     ua.errhist = cv.take<double>((size_t)kErrHistory);
     ua.run_counter = cv.take<unsigned long long>(1);
     ca.cbar = cv.take<float>((size_t)N);
@@ -247,6 +247,7 @@ extern "C" ptycho_status ptycho_iterate_static(const ptycho_params* p, const flo
   ua.tiles_x = tx;
   ua.tiles_y = ty;
   ua.probe_blocks = pb;
+  ua.split_lists = capi_long_lists(start) ? 1 : 0;
   ua.errden = h_sums[1];
   ua.beta_obj = (float)p->beta_obj;
   ua.beta_probe = (float)p->beta_probe;
@@ -270,11 +271,11 @@ extern "C" ptycho_status ptycho_iterate_static(const ptycho_params* p, const flo
     const long long t = (long long)p->start_iteration + i;
     PS_CUDA(launch_fused(M, fa, slots, s), "fused kernel launch");
     ua.update_probe = t >= p->probe_update_start;
-    PS_CUDA(launch_update(ua, s), "update launch");
     bool win = false;
     for (int w = 0; w < p->n_windows; ++w)
       if (t >= p->windows[2 * w] && t <= p->windows[2 * w + 1]) win = true;
-    if (win) PS_CUDA(launch_constraint(ca, s), "constraint launch");
+    PS_CUDA(launch_update(ua, win ? &ca : nullptr, true, true, s), "update launch");
+    if (win) PS_CUDA(launch_constraint(ca, false, s), "constraint launch");
   }
   if (errors && n_iter > 0)
     PS_CUDA(cudaMemcpyAsync(errors, ua.errhist, sizeof(double) * n_iter, cudaMemcpyDeviceToHost, s), "copy errors");

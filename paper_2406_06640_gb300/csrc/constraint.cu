@@ -14,7 +14,7 @@
 // All box sums are exact: values are held in 32.32 fixed point (int64) and
 // summed with integer arithmetic, so the results do not depend on order.
 //   (1) |ln a| and |phi| of every object pixel in 32.32 fixed point, as prefix sums along the
-//       object rows;
+//       object rows (constraint.cuh; after an object step the step's own kernel does it);
 //   (2) one warp per box: each box sum is M differences of two row prefix sums -> C_n, and C_n
 //       in fixed point;
 //   (3) one block per 32 x 32 object tile: the boxes of the tile's position list, clipped to the
@@ -25,6 +25,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "constraint.cuh"
 #include "engine.h"
 #include "fft.cuh"
 
@@ -32,67 +33,10 @@ namespace ptycho {
 
 constexpr double kFix = 4294967296.0;  // 2^32
 
-// Row prefix sums of |ln a| and |phi| in 32.32 fixed point: P(y, x) = sum over x' < x of the value at
-// (y, x'), obj_h x (obj_w + 1) each. v * 2^32 is exact in FP32, so llrintf of it is the nearest
-// 32.32 value of v.
-__device__ __forceinline__ void cc_values(float2 o, long long& l, long long& p) {
-  const float f = 4294967296.0f;
-  l = llrintf(fabsf(logf(fmaxf(sqrtf(cabs2(o)), 1e-6f))) * f);
-  p = llrintf(fabsf(atan2f(o.y, o.x)) * f);
-}
-
+// one block per object row (constraint.cuh)
 __global__ void __launch_bounds__(256) k_cc_rows(const ConstraintArgs c) {
-  // one block per object row, warp w scanning segment w of SEG pixels (32 per step, a carry
-  // between steps), then every segment adds the totals of the segments before it
-  __shared__ long long s_tl[8], s_tp[8];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int y = blockIdx.x;
-  const int W1 = c.obj_w + 1;
-  const int SEG = ((c.obj_w + 7) / 8 + 31) / 32 * 32;
-  const int x_lo = min(c.obj_w, w * SEG), x_hi = min(c.obj_w, x_lo + SEG);
-  long long* pl = c.map_lna + (size_t)y * W1;
-  long long* pp = c.map_phi + (size_t)y * W1;
-  const float2* Oy = c.O + (size_t)y * c.obj_w;
-  if (threadIdx.x == 0) {
-    pl[0] = 0;
-    pp[0] = 0;
-  }
-  long long cl = 0, cp = 0;  // this segment's sums so far
-  for (int x0 = x_lo; x0 < x_hi; x0 += 32) {
-    const int x = x0 + lane;
-    long long vl = 0, vp = 0;
-    if (x < x_hi) cc_values(Oy[x], vl, vp);
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const long long ul = __shfl_up_sync(0xffffffffu, vl, d);
-      const long long up = __shfl_up_sync(0xffffffffu, vp, d);
-      if (lane >= d) {
-        vl += ul;
-        vp += up;
-      }
-    }
-    if (x < x_hi) {
-      pl[x + 1] = cl + vl;
-      pp[x + 1] = cp + vp;
-    }
-    cl += __shfl_sync(0xffffffffu, vl, 31);
-    cp += __shfl_sync(0xffffffffu, vp, 31);
-  }
-  if (lane == 0) {
-    s_tl[w] = cl;
-    s_tp[w] = cp;
-  }
-  __syncthreads();
-  long long ol = 0, op = 0;
-  for (int q = 0; q < w; ++q) {
-    ol += s_tl[q];
-    op += s_tp[q];
-  }
-  if (w > 0)
-    for (int x = x_lo + lane; x < x_hi; x += 32) {
-      pl[x + 1] += ol;
-      pp[x + 1] += op;
-    }
+  const float2* Oy = c.O + (size_t)blockIdx.x * c.obj_w;
+  constraint_row(c, (int)blockIdx.x, [&](int x) { return Oy[x]; });
 }
 
 // one warp per box: the two box sums (exact) from M row differences each, C_n clamped, C_n in fixed
@@ -239,9 +183,9 @@ __global__ void __launch_bounds__(256) k_cc_apply(const ConstraintArgs c) {
   }
 }
 
-cudaError_t launch_constraint(const ConstraintArgs& c, cudaStream_t s) {
+cudaError_t launch_constraint(const ConstraintArgs& c, bool with_rows, cudaStream_t s) {
   if (c.N == 0) return cudaSuccess;
-  k_cc_rows<<<c.obj_h, 256, 0, s>>>(c);
+  if (with_rows) k_cc_rows<<<c.obj_h, 256, 0, s>>>(c);
   k_cc_cbar<<<(c.N + 7) / 8, 256, 0, s>>>(c);
   k_cc_apply<<<dim3(c.tiles_x, c.tiles_y), dim3(32, 8), 0, s>>>(c);
   return cudaGetLastError();

@@ -149,11 +149,11 @@ struct UpdateArgs {
   const int4* tile_pos;   // per tile, (n, row, col, 0) of each overlapping position, increasing n
   int tiles_x, tiles_y;
   float2* no_part; float* do_part;  // N_O and D_O, obj_h x obj_w each
-  float* blk_max_o;                  // per object tile
+  int split_lists;                   // the lists are long: a cluster of eight blocks shares each (k_gather)
+  int* dmax;                         // maxima of D_O and D_P as float bits
   // probe gather
   float2* np_sum; float* dp_sum; float* p2;  // K x M x M, M x M, M x M
-  float* blk_max_p;
-  int probe_blocks;
+  int probe_blocks;                  // ceil(M^2 / 256)
   double* errhist; double errden;
   unsigned long long* run_counter;  // device: iterations finished; E goes to errhist[counter % kErrHistory]
   // error of a launch: 0 finishes E from this launch's partials; 1 adds them to *err_acc (a batch
@@ -170,11 +170,6 @@ struct UpdateArgs {
   // P (O - dm_obj_prev) under their boxes); null otherwise
   const float2* dm_obj_prev;
 };
-// launch_update = launch_update_object then launch_update_probe (pc-DM runs the complex constraint
-// between the two)
-cudaError_t launch_update(const UpdateArgs& u, cudaStream_t s);
-cudaError_t launch_update_object(const UpdateArgs& u, cudaStream_t s);
-cudaError_t launch_update_probe(const UpdateArgs& u, cudaStream_t s);
 // finishes E of a mini-batch iteration from *err_acc (every batch ran with err_mode 1)
 cudaError_t launch_err_finish(const UpdateArgs& u, cudaStream_t s);
 
@@ -200,7 +195,18 @@ struct ConstraintArgs {
   const int4* tile_pos;   // per tile, (n, row, col, 0) of every position whose box overlaps it
   int tiles_x, tiles_y;
 };
-cudaError_t launch_constraint(const ConstraintArgs& c, cudaStream_t s);
+// the row sums (unless the object step before it made them), the box sums and the constraint itself
+cudaError_t launch_constraint(const ConstraintArgs& c, bool with_rows, cudaStream_t s);
+
+// the update of one iteration or batch (update.cu): the |P|^2 map, the gather of both sides, the steps.
+// c: the object step also makes the row sums of the complex constraint that follows. with_p2 false: launch_p2
+// ran beside the fused kernel already. one_apply: object and probe step in one launch
+cudaError_t launch_p2(const UpdateArgs& u, cudaStream_t s);
+cudaError_t launch_update(const UpdateArgs& u, const ConstraintArgs* c, bool with_p2, bool one_apply,
+                          cudaStream_t s);
+// pc-DM: the object side, and (after the complex constraint) the probe side from the state
+cudaError_t launch_update_object(const UpdateArgs& u, const ConstraintArgs* c, cudaStream_t s);
+cudaError_t launch_update_probe_dm(const UpdateArgs& u, cudaStream_t s);
 
 // plan-time helpers (update.cu)
 cudaError_t launch_intensity_sums(const float* I, size_t count, double* partials, int nblocks, cudaStream_t s);

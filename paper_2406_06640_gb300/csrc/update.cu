@@ -19,6 +19,7 @@
 
 #include <algorithm>
 
+#include "constraint.cuh"
 #include "engine.h"
 #include "cluster.cuh"
 #include "fft.cuh"
@@ -91,53 +92,17 @@ cudaError_t launch_finish_sums(const double* partials, int nblocks, double* out,
   return cudaGetLastError();
 }
 
-// ------------------------------------------------------------------ probe: sum the per-slot partials
-// grid (ceil(M^2 / 256), K + 1): y < K sums N_P for mode y; y == K sums D_P, |P|^2 map and block max
-// thread (pixel p, group g) sums the slots g, g + 4, g + 8, ..., and the four group sums are added
-// in group order (a fixed summation order; four loads in flight per pixel instead of one)
-constexpr int kProbeGroups = 4;
-__global__ void __launch_bounds__(256 * kProbeGroups) k_probe_gather(const UpdateArgs u) {
+// ------------------------------------------------------------------ |P|^2 map
+// sum_k |P_k|^2 per probe pixel, and the maxima of D_O and D_P cleared for this update's gather. It depends
+// on the probe alone, so a single plan's graph runs it beside the fused kernel
+__global__ void __launch_bounds__(256) k_p2(const UpdateArgs u) {
   const int MM = u.M * u.M;
-  const int tx = threadIdx.x % 256, g = threadIdx.x / 256;
-  const int p = blockIdx.x * 256 + tx;
-  __shared__ float2 part[kProbeGroups][256];
-  __shared__ float smax[256];
-  if ((int)blockIdx.y < u.K) {
-    const int k = blockIdx.y;
-    float2 acc = make_float2(0.f, 0.f);
-    if (p < MM) {
-#pragma unroll 4
-      for (int s = g; s < u.slots; s += kProbeGroups) acc = cadd(acc, u.pacc[((size_t)s * u.K + k) * MM + p]);
-    }
-    part[g][tx] = acc;
-    __syncthreads();
-    if (g == 0 && p < MM)
-      u.np_sum[(size_t)k * MM + p] = cadd(cadd(cadd(part[0][tx], part[1][tx]), part[2][tx]), part[3][tx]);
-    return;
-  }
-  float dp = 0.f;
-  if (p < MM) {
-#pragma unroll 4
-    for (int s = g; s < u.slots; s += kProbeGroups) dp += u.dacc[(size_t)s * MM + p];
-  }
-  part[g][tx].x = dp;
-  __syncthreads();
-  if (g != 0) return;
-  dp = ((part[0][tx].x + part[1][tx].x) + part[2][tx].x) + part[3][tx].x;
-  if (p < MM) {
-    float p2 = 0.f;
-    for (int k = 0; k < u.K; ++k) p2 += cabs2(u.P[(size_t)k * MM + p]);
-    u.dp_sum[p] = dp;
-    u.p2[p] = p2;
-  }
-  smax[tx] = dp;
-  // the first 256 threads (whole warps) finish the block maximum
-  asm volatile("bar.sync 1, 256;" ::: "memory");
-  for (int w = 128; w > 0; w >>= 1) {
-    if (tx < w) smax[tx] = fmaxf(smax[tx], smax[tx + w]);
-    asm volatile("bar.sync 1, 256;" ::: "memory");
-  }
-  if (tx == 0) u.blk_max_p[blockIdx.x] = smax[0];
+  const int p = blockIdx.x * 256 + threadIdx.x;
+  if (p < 2) u.dmax[p] = 0;
+  if (p >= MM) return;
+  float s = 0.f;
+  for (int k = 0; k < u.K; ++k) s += cabs2(u.P[(size_t)k * MM + p]);
+  u.p2[p] = s;
 }
 
 // ------------------------------------------------------------------ pc-DM probe partials
@@ -210,146 +175,174 @@ static void launch_dm_probe_partials(const UpdateArgs& u, cudaStream_t s) {
   else k_dm_probe_partials<8><<<grid, 256, 0, s>>>(u);
 }
 
-// ------------------------------------------------------------------ object: per-tile gather of the contributions
-// grid (tiles_x, tiles_y, kObjSplit) in clusters of the kObjSplit blocks of one tile, block 32 x 8;
-// thread (tx, ty) owns pixels (Y0 + ty + 8 i, X0 + tx). Block `split` sums positions split,
-// split + kObjSplit, ... of the tile's list; the partial tiles meet in distributed shared memory,
-// where rank r adds up rows 4r .. 4r + 3 over the ranks in order and writes N_O, D_O; rank 0 also
-// takes the tile maximum of D_O.
-__global__ void __launch_bounds__(256, 3) k_obj_gather(const UpdateArgs u) {
-  constexpr int TT = kObjTile * kObjTile, RPR = TT / kObjSplit;  // pixels finished per rank
-  static_assert(RPR <= 256 && RPR % 32 == 0 && kObjTile == 32, "tile split");
-  __shared__ float2 s_acc[TT];
-  __shared__ float s_den[TT];
-  __shared__ float s_max[kObjSplit * (RPR / 32)];
-  const int tile = blockIdx.y * u.tiles_x + blockIdx.x;
-  const int split = blockIdx.z;
-  const unsigned rank = cluster_ctarank();
-  const int tx0 = blockIdx.x * kObjTile, ty0 = blockIdx.y * kObjTile;
-  const int X = tx0 + threadIdx.x;
-  const int Y0 = ty0 + threadIdx.y;
-  const int lt = threadIdx.y * 32 + threadIdx.x;
-  const int M = u.M;
-  const size_t MM = (size_t)M * M;
-  float2 acc[4];
-  float den[4];
+// ------------------------------------------------------------------ gather: N_O, D_O and N_P, D_P
+// One launch sums both sides. A unit of work is 256 PX values, PX per thread: part of a 32 x 32 object tile
+// (its positions' contributions and |P|^2 under their boxes), or probe pixels of one mode or of D_P (their
+// per-slot partials). Every sum has a fixed order.
+//   SPLIT = 8: a unit is a whole tile (PX = 4) shared by a cluster of eight blocks. Block `rank` takes terms
+//     rank, rank + 8, ..., and the ranks' sums are added in rank order through distributed shared memory. For
+//     long lists: a tile in the middle of a dense scan holds hundreds of positions.
+//   SPLIT = 1: a unit is 8 rows of a tile (PX = 1) and one block. For short lists (mini-batches, small scans),
+//     where the blocks of a cluster would mostly start, meet and end.
+// Bound by the latency of the term loads: 4 / PX positions of PX pixels and their |P|^2 in flight per thread. The
+// line between the forms is 24 terms on average. (Clusters of 8-row bands: 104 us against 77 us for 900
+// positions of 128^2 on 640^2, most blocks of the border tiles being overhead.)
+// The maxima of D_O and D_P are integer atomics on the float bits (non-negative: the order of the bits),
+// so they do not depend on the order either.
+template <int SPLIT>
+__global__ void __launch_bounds__(256, SPLIT == 8 ? 3 : 4) k_gather(const UpdateArgs u, int units_o) {
+  static_assert(SPLIT == 1 || SPLIT == 8, "cluster size");
+  constexpr int PX = SPLIT == 8 ? 4 : 1, VALUES = 256 * PX, BANDS = 4 / PX;  // units per tile
+  constexpr int U = SPLIT == 8 ? 4 : 8;                                      // positions in flight
+  __shared__ float2 s_acc[SPLIT > 1 ? VALUES : 1];
+  __shared__ float s_den[SPLIT > 1 ? VALUES : 1];
+  const int unit = blockIdx.x / SPLIT, rank = SPLIT > 1 ? (int)cluster_ctarank() : 0;
+  const int tid = threadIdx.x;
+  const int M = u.M, MM = M * M;
+  const bool obj = unit < units_o;
+  const int tile = unit / BANDS, X0 = tile % u.tiles_x * kObjTile;
+  const int Y0 = tile / u.tiles_x * kObjTile + unit % BANDS * (kObjTile / BANDS);
+  const int pu = (MM + VALUES - 1) / VALUES, k = obj ? 0 : (unit - units_o) / pu;  // k == K: D_P
+  const int P0 = obj ? 0 : (unit - units_o) % pu * VALUES;
+  // output of value t of the unit (object: row-major in the tile part), -1: outside
+  auto output = [&](int t) {
+    if (!obj) return P0 + t < MM ? P0 + t : -1;
+    const int X = X0 + t % kObjTile, Y = Y0 + t / kObjTile;
+    return X < u.obj_w && Y < u.obj_h ? Y * u.obj_w + X : -1;
+  };
+  float m = 0.f;
+  auto store = [&](int t, float2 a, float d) {
+    const int at = output(t);
+    if (at < 0) return;
+    if (obj) {
+      u.no_part[at] = a;
+      u.do_part[at] = d;
+      m = fmaxf(m, d);
+    } else if (k < u.K) {
+      u.np_sum[(size_t)k * MM + at] = a;
+    } else {
+      u.dp_sum[at] = d;
+      m = fmaxf(m, d);
+    }
+  };
+  constexpr int RPR = VALUES / SPLIT;  // values a rank finishes
+  float2 acc[PX];
+  float den[PX];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < PX; ++i) {
     acc[i] = make_float2(0.f, 0.f);
     den[i] = 0.f;
   }
-  const int s0 = u.tile_start[tile], s1 = u.tile_start[tile + 1];
-  // four positions per round: every load of the round is in flight before the sums, which run in
-  // list order (a tile in the middle of a dense scan holds hundreds of positions); three blocks
-  // per SM
-  constexpr int kU = 4;
-  for (int base = s0 + split; base < s1; base += kU * kObjSplit) {
-    float2 cv[kU][4];
-    float dv[kU][4];
+  if (obj) {
+    const int s0 = u.tile_start[tile], s1 = u.tile_start[tile + 1];
+    if (s0 == s1) {  // no position (the same in every rank)
+      for (int t = tid; t < RPR; t += 256) store(rank * RPR + t, make_float2(0.f, 0.f), 0.f);
+      return;
+    }
+    const int X = X0 + (tid & 31), Y = Y0 + (tid >> 5);
+    for (int base = s0 + rank; base < s1; base += U * SPLIT) {
+      float2 cv[U][PX];
+      float dv[U][PX];
 #pragma unroll
-    for (int r = 0; r < kU; ++r) {
-      const int idx = base + r * kObjSplit;
-      const int4 ent = idx < s1 ? u.tile_pos[idx] : make_int4(0, 0, -(1 << 20), 0);  // (n, row, col)
-      const int cx = X - ent.z;
-      const bool inx = cx >= 0 && cx < M;
-      const float2* cn = u.cn + (size_t)ent.x * MM;
+      for (int r = 0; r < U; ++r) {
+        const int idx = base + r * SPLIT;
+        const int4 ent = idx < s1 ? u.tile_pos[idx] : make_int4(0, 0, -(1 << 20), 0);  // (n, row, col)
+        const int cx = X - ent.z;
+        const bool inx = cx >= 0 && cx < M;
+        const float2* cn = u.cn + (size_t)ent.x * MM;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int cy = Y0 + 8 * i - ent.y;
-        const bool in = inx && cy >= 0 && cy < M;
-        cv[r][i] = in ? cn[(size_t)cy * M + cx] : make_float2(0.f, 0.f);
-        dv[r][i] = in ? u.p2[cy * M + cx] : 0.f;
+        for (int i = 0; i < PX; ++i) {
+          const int cy = Y + 8 * i - ent.y;
+          const bool in = inx && cy >= 0 && cy < M;
+          cv[r][i] = in ? cn[cy * M + cx] : make_float2(0.f, 0.f);
+          dv[r][i] = in ? u.p2[cy * M + cx] : 0.f;
+        }
       }
+#pragma unroll
+      for (int r = 0; r < U; ++r)
+#pragma unroll
+        for (int i = 0; i < PX; ++i) {
+          acc[i] = cadd(acc[i], cv[r][i]);
+          den[i] += dv[r][i];
+        }
     }
+  } else if (k < u.K) {
+#pragma unroll 4
+    for (int s = rank; s < u.slots; s += SPLIT)
 #pragma unroll
-    for (int r = 0; r < kU; ++r)
+      for (int i = 0; i < PX; ++i)
+        if (P0 + tid + 256 * i < MM)
+          acc[i] = cadd(acc[i], u.pacc[((size_t)s * u.K + k) * MM + P0 + tid + 256 * i]);
+  } else {
+#pragma unroll 4
+    for (int s = rank; s < u.slots; s += SPLIT)
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        acc[i] = cadd(acc[i], cv[r][i]);
-        den[i] += dv[r][i];
+      for (int i = 0; i < PX; ++i)
+        if (P0 + tid + 256 * i < MM) den[i] += u.dacc[(size_t)s * MM + P0 + tid + 256 * i];
+  }
+  // (thread tid's values are tid, tid + 256, ...: rows tid / 32 + 8 i of a tile)
+  if constexpr (SPLIT == 1) {
+    store(tid, acc[0], den[0]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < PX; ++i) {
+      s_acc[tid + 256 * i] = acc[i];
+      s_den[tid + 256 * i] = den[i];
+    }
+    cluster_sync_all();  // every rank's sums are complete
+    if (tid < RPR) {
+      const int t = rank * RPR + tid;
+      const uint32_t oa = smem_addr(&s_acc[t]), od = smem_addr(&s_den[t]);
+      float2 a = make_float2(0.f, 0.f);
+      float d = 0.f;
+#pragma unroll
+      for (int q = 0; q < SPLIT; ++q) {
+        a = cadd(a, ld_cluster_f2(map_rank(oa, (unsigned)q)));
+        d += ld_cluster_f32(map_rank(od, (unsigned)q));
       }
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    s_acc[(threadIdx.y + 8 * i) * kObjTile + threadIdx.x] = acc[i];
-    s_den[(threadIdx.y + 8 * i) * kObjTile + threadIdx.x] = den[i];
-  }
-  cluster_sync_all();  // every rank's partial tile is complete
-  float m = 0.f;
-  if (lt < RPR) {
-    const int lp = (int)rank * RPR + lt;
-    const uint32_t oa = smem_addr(&s_acc[lp]), od = smem_addr(&s_den[lp]);
-    float2 a = ld_cluster_f2(map_rank(oa, 0));
-    float d = ld_cluster_f32(map_rank(od, 0));
-    for (int q = 1; q < kObjSplit; ++q) {
-      a = cadd(a, ld_cluster_f2(map_rank(oa, (unsigned)q)));
-      d += ld_cluster_f32(map_rank(od, (unsigned)q));
+      store(t, a, d);
     }
-    const int Y = ty0 + lp / kObjTile, Xp = tx0 + lp % kObjTile;
-    if (Y < u.obj_h && Xp < u.obj_w) {
-      const size_t q = (size_t)Y * u.obj_w + Xp;
-      u.no_part[q] = a;
-      u.do_part[q] = d;
-      m = d;  // D_O >= 0
-    }
-    const int wm = __reduce_max_sync(0xffffffffu, __float_as_int(m));  // non-negative floats order as ints
-    if ((lt & 31) == 0) st_cluster_f32(map_rank(smem_addr(&s_max[rank * (RPR / 32) + lt / 32]), 0), __int_as_float(wm));
+    cluster_sync_all();  // no rank exits while another may still read its sums
   }
-  cluster_sync_all();  // remote reads and the maxima are done
-  if (rank == 0 && lt == 0) {
-    float mm = 0.f;
-    for (int i = 0; i < kObjSplit * (RPR / 32); ++i) mm = fmaxf(mm, s_max[i]);
-    u.blk_max_o[tile] = mm;
-  }
+  const int wm = __reduce_max_sync(0xffffffffu, __float_as_int(m));
+  if ((tid & 31) == 0 && wm > 0) atomicMax(&u.dmax[obj ? 0 : 1], wm);
 }
 
-__device__ float block_max_of(const float* vals, int n) {
-  __shared__ float smax[256];
-  float m = 0.f;
-  const int lt = threadIdx.y * blockDim.x + threadIdx.x;
-  const int nt = blockDim.x * blockDim.y;
-  for (int i = lt; i < n; i += nt) m = fmaxf(m, vals[i]);
-  smax[lt] = m;
-  __syncthreads();
-  for (int w = nt / 2; w > 0; w >>= 1) {
-    if (lt < w) smax[lt] = fmaxf(smax[lt], smax[lt + w]);
-    __syncthreads();
-  }
-  const float r = smax[0];
-  __syncthreads();
-  return r;
-}
-
-__global__ void __launch_bounds__(256) k_obj_apply(const UpdateArgs u) {
-  const float maxd = block_max_of(u.blk_max_o, u.tiles_x * u.tiles_y);
-  const int X = blockIdx.x * kObjTile + threadIdx.x;
-  const int Y0 = blockIdx.y * kObjTile + threadIdx.y;
-  if (X >= u.obj_w) return;
-  const float floor_d = u.cmax_obj * maxd;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int Y = Y0 + 8 * i;
-    if (Y >= u.obj_h) break;
-    const size_t q = (size_t)Y * u.obj_w + X;
-    const float d = u.do_part[q];
-    if (d > 0.f) {
-      const float w = u.beta_obj / fmaf(u.cd_obj, d, floor_d);
-      const float2 num = u.no_part[q];
+// ------------------------------------------------------------------ apply
+// Blocks 0 .. rows - 1 (rows = obj_h or 0) take one object row each: O += beta N_O / (c_d D_O + c_max max
+// D_O). CC: inside a complex-constraint window the row's prefix sums of the new object follow at once
+// (constraint.cu's row pass, without another launch and read of O). The next pblocks blocks take 256 probe
+// pixels of a mode each; the first of them also finishes the FP64 error.
+template <bool CC>
+__global__ void __launch_bounds__(256) k_apply(const UpdateArgs u, const ConstraintArgs c, int rows) {
+  if ((int)blockIdx.x < rows) {
+    const float floor_d = u.cmax_obj * __int_as_float(u.dmax[0]);
+    const size_t row = (size_t)blockIdx.x * u.obj_w;
+    auto step = [&](int x) {
+      const size_t q = row + x;
+      const float d = u.do_part[q];
       float2 o = u.O[q];
-      o.x = fmaf(w, num.x, o.x);
-      o.y = fmaf(w, num.y, o.y);
-      u.O[q] = o;
+      if (d > 0.f) {
+        const float w = u.beta_obj / fmaf(u.cd_obj, d, floor_d);
+        const float2 num = u.no_part[q];
+        o.x = fmaf(w, num.x, o.x);
+        o.y = fmaf(w, num.y, o.y);
+        u.O[q] = o;
+      }
+      return o;
+    };
+    if constexpr (CC) {
+      constraint_row(c, (int)blockIdx.x, step);
+    } else {
+      for (int x = threadIdx.x; x < u.obj_w; x += 256) step(x);
     }
+    return;
   }
-}
-
-// grid (ceil(M^2 / 256), K): apply the probe step; block (0, 0) also finishes the FP64 error
-__global__ void k_probe_apply(const UpdateArgs u) {
-  const float maxd = block_max_of(u.blk_max_p, u.probe_blocks);
-  double e = 0.0;
-  if (blockIdx.x == 0 && blockIdx.y == 0) {
+  const int b = (int)blockIdx.x - rows, pb = u.probe_blocks;
+  if (b == 0) {
     // error numerator: strided partial sums, then a fixed tree (every load in flight at once)
     __shared__ double s_e[256];
+    double e = 0.0;
     for (int s = threadIdx.x; s < u.nerr; s += 256) e += u.errpart[s];
     s_e[threadIdx.x] = e;
     __syncthreads();
@@ -357,27 +350,27 @@ __global__ void k_probe_apply(const UpdateArgs u) {
       if ((int)threadIdx.x < w) s_e[threadIdx.x] += s_e[threadIdx.x + w];
       __syncthreads();
     }
-    e = s_e[0];
-  }
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
-    if (u.err_mode != 0) e += *u.err_acc;
-    if (u.err_mode == 1) {
-      *u.err_acc = e;
-    } else {
-      const unsigned long long r = *u.run_counter;
-      u.errhist[r % kErrHistory] = sqrt(e / u.errden);
-      *u.run_counter = r + 1;
-      if (u.err_mode == 2) *u.err_acc = 0.0;
+    if (threadIdx.x == 0) {
+      e = s_e[0];
+      if (u.err_mode != 0) e += *u.err_acc;
+      if (u.err_mode == 1) {
+        *u.err_acc = e;
+      } else {
+        const unsigned long long r = *u.run_counter;
+        u.errhist[r % kErrHistory] = sqrt(e / u.errden);
+        *u.run_counter = r + 1;
+        if (u.err_mode == 2) *u.err_acc = 0.0;
+      }
     }
   }
   if (!u.update_probe) return;
   const int MM = u.M * u.M;
-  const int p = blockIdx.x * 256 + threadIdx.x;
+  const int k = b / pb, p = (b % pb) * 256 + threadIdx.x;
   if (p >= MM) return;
   const float d = u.dp_sum[p];
   if (d > 0.f) {
-    const float w = u.beta_probe / fmaf(u.cd_probe, d, u.cmax_probe * maxd);
-    const size_t q = (size_t)blockIdx.y * MM + p;
+    const float w = u.beta_probe / fmaf(u.cd_probe, d, u.cmax_probe * __int_as_float(u.dmax[1]));
+    const size_t q = (size_t)k * MM + p;
     const float2 num = u.np_sum[q];
     float2 pr = u.P[q];
     pr.x = fmaf(w, num.x, pr.x);
@@ -386,51 +379,67 @@ __global__ void k_probe_apply(const UpdateArgs u) {
   }
 }
 
-cudaError_t launch_update_object(const UpdateArgs& u, cudaStream_t s) {
-  const int MM = u.M * u.M;
-  const int pb = (MM + 255) / 256;
-  if (u.dm_psi) {
-    // the |P|^2 map for the object step only (no partials: the probe sums follow the object step)
-    UpdateArgs u0 = u;
-    u0.slots = 0;
-    k_probe_gather<<<dim3(pb, u.K + 1), 256 * kProbeGroups, 0, s>>>(u0);
-  } else {
-    k_probe_gather<<<dim3(pb, u.K + 1), 256 * kProbeGroups, 0, s>>>(u);
-  }
-  const dim3 tb(32, 8);
-  {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)u.tiles_x, (unsigned)u.tiles_y, kObjSplit);
-    cfg.blockDim = tb;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 1;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = kObjSplit;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_obj_gather, u);
-    if (e != cudaSuccess) return e;
-  }
-  k_obj_apply<<<dim3(u.tiles_x, u.tiles_y), tb, 0, s>>>(u);
+cudaError_t launch_p2(const UpdateArgs& u, cudaStream_t s) {
+  k_p2<<<u.probe_blocks, 256, 0, s>>>(u);
   return cudaGetLastError();
 }
 
-cudaError_t launch_update_probe(const UpdateArgs& u, cudaStream_t s) {
-  const int MM = u.M * u.M;
-  const int pb = (MM + 255) / 256;
-  if (u.dm_psi && (u.update_probe || u.dm_obj_prev)) {
+// object and / or probe side of the gather
+static cudaError_t launch_gather(const UpdateArgs& u, bool obj, bool probe, cudaStream_t s) {
+  const int px = u.split_lists ? 4 : 1, MM = u.M * u.M;
+  const int units_o = obj ? u.tiles_x * u.tiles_y * (4 / px) : 0;
+  const int units = units_o + (probe ? (MM + 256 * px - 1) / (256 * px) * (u.K + 1) : 0);
+  if (!u.split_lists) {
+    k_gather<1><<<units, 256, 0, s>>>(u, units_o);
+    return cudaGetLastError();
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)units * 8);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 8;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_gather<8>, u, units_o);
+}
+
+// object and / or probe side of the apply; c: the row pass of the complex constraint with the object side
+static cudaError_t launch_apply(const UpdateArgs& u, const ConstraintArgs* c, bool obj, bool probe, cudaStream_t s) {
+  const int rows = obj ? u.obj_h : 0;
+  const int blocks = rows + (probe ? u.probe_blocks * u.K : 0);
+  if (c && obj) k_apply<true><<<blocks, 256, 0, s>>>(u, *c, rows);
+  else k_apply<false><<<blocks, 256, 0, s>>>(u, ConstraintArgs{}, rows);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_update_object(const UpdateArgs& u, const ConstraintArgs* c, cudaStream_t s) {
+  cudaError_t e = launch_p2(u, s);
+  if (e == cudaSuccess) e = launch_gather(u, true, false, s);
+  if (e == cudaSuccess) e = launch_apply(u, c, true, false, s);
+  return e;
+}
+
+cudaError_t launch_update_probe_dm(const UpdateArgs& u, cudaStream_t s) {
+  cudaError_t e = cudaSuccess;
+  if (u.update_probe || u.dm_obj_prev) {
     launch_dm_probe_partials(u, s);
-    if (u.update_probe) k_probe_gather<<<dim3(pb, u.K + 1), 256 * kProbeGroups, 0, s>>>(u);
+    e = cudaGetLastError();
+    if (e == cudaSuccess && u.update_probe) e = launch_gather(u, false, true, s);
   }
-  k_probe_apply<<<dim3(pb, u.K), 256, 0, s>>>(u);
-  return cudaGetLastError();
+  return e == cudaSuccess ? launch_apply(u, nullptr, false, true, s) : e;
 }
 
-cudaError_t launch_update(const UpdateArgs& u, cudaStream_t s) {
-  cudaError_t e = launch_update_object(u, s);
-  return e != cudaSuccess ? e : launch_update_probe(u, s);
+cudaError_t launch_update(const UpdateArgs& u, const ConstraintArgs* c, bool with_p2, bool one_apply,
+                          cudaStream_t s) {
+  cudaError_t e = with_p2 ? launch_p2(u, s) : cudaSuccess;
+  if (e == cudaSuccess) e = launch_gather(u, true, true, s);
+  if (e == cudaSuccess) e = launch_apply(u, c, true, one_apply, s);
+  if (e == cudaSuccess && !one_apply) e = launch_apply(u, nullptr, false, true, s);
+  return e;
 }
 
 // E of a mini-batch iteration whose batches all added their partials to *err_acc (err_mode 1): the
