@@ -267,18 +267,21 @@ __global__ void __launch_bounds__(256, SPLIT == 8 ? 3 : 4) k_gather(const Update
         }
     }
   } else if (k < u.K) {
-#pragma unroll 4
+    const float2* part[PX];  // (past the last pixel: that pixel again, not stored)
+#pragma unroll
+    for (int i = 0; i < PX; ++i) part[i] = u.pacc + (size_t)k * MM + min(P0 + tid + 256 * i, MM - 1);
+#pragma unroll 8 / PX * 2
     for (int s = rank; s < u.slots; s += SPLIT)
 #pragma unroll
-      for (int i = 0; i < PX; ++i)
-        if (P0 + tid + 256 * i < MM)
-          acc[i] = cadd(acc[i], u.pacc[((size_t)s * u.K + k) * MM + P0 + tid + 256 * i]);
+      for (int i = 0; i < PX; ++i) acc[i] = cadd(acc[i], part[i][(size_t)s * u.K * MM]);
   } else {
-#pragma unroll 4
+    const float* part[PX];
+#pragma unroll
+    for (int i = 0; i < PX; ++i) part[i] = u.dacc + min(P0 + tid + 256 * i, MM - 1);
+#pragma unroll 8 / PX * 2
     for (int s = rank; s < u.slots; s += SPLIT)
 #pragma unroll
-      for (int i = 0; i < PX; ++i)
-        if (P0 + tid + 256 * i < MM) den[i] += u.dacc[(size_t)s * MM + P0 + tid + 256 * i];
+      for (int i = 0; i < PX; ++i) den[i] += part[i][(size_t)s * MM];
   }
   // (thread tid's values are tid, tid + 256, ...: rows tid / 32 + 8 i of a tile)
   if constexpr (SPLIT == 1) {
