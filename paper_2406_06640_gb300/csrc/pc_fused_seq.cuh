@@ -37,6 +37,7 @@
 #include "cluster.cuh"
 #include "engine.h"
 #include "fft.cuh"
+#include "fft3.cuh"
 #include "fused_common.cuh"
 
 namespace ptycho {
@@ -91,17 +92,28 @@ struct SeqShape {
   static constexpr int MIN_BLOCKS = M == 64 ? 2 : 1;
 };
 
+// exchange buffer of the 2-D transform: fft3.cuh for M = 64 and 128, fft.cuh below
+template <int M, bool F3 = (M >= 64)>
+struct SeqExchange {
+  static constexpr size_t BYTES = (size_t)Tile<M>::SMEM * 8;
+};
+template <int M>
+struct SeqExchange<M, true> {
+  static constexpr size_t BYTES = (size_t)Tile3<M>::SMEM * 8;
+};
+
 template <int M>
 struct SeqSmem {
   static constexpr int LD = M + 1;  // padded row stride of the f32 detector buffers
-  static constexpr size_t kX = (size_t)Tile<M>::SMEM * 8;  // FFT exchange buffer
+  static constexpr size_t kX = SeqExchange<M>::BYTES;
   static constexpr size_t kB = (size_t)M * LD * 4;         // one f32 detector buffer
   static constexpr size_t CBUF = ((kX > kB ? kX : kB) + 15) / 16 * 16;
   static constexpr size_t ZBUF = (kB + 15) / 16 * 16;      // S, then R
   static constexpr size_t TWT = ((size_t)Tile<M>::G * Tile<M>::LDW * 8 + 15) / 16 * 16;
+  static constexpr size_t TW2 = 64 * 8;  // second twiddles of fft3.cuh
   static constexpr size_t HQ = (size_t)M * 8;
   static constexpr size_t TAPS = 2 * kMaxTaps * 4 + 8;  // taps, TMEM address
-  static constexpr size_t BYTES = CBUF + ZBUF + TWT + HQ + TAPS;
+  static constexpr size_t BYTES = CBUF + ZBUF + TWT + TW2 + HQ + TAPS;
   // queued launches: the current problem's arguments and the chunk index
   static constexpr size_t DESC = (sizeof(FusedArgs) + 15) / 16 * 16 + 16;
   static constexpr size_t bytes(int mode) { return BYTES + (mode == 1 ? DESC : 0); }
@@ -126,8 +138,9 @@ __global__ void __launch_bounds__(SeqShape<M>::TR, SeqShape<M>::MIN_BLOCKS) pc_s
   float* X = reinterpret_cast<float*>(smem);               // x-blurred S (aliases the exchange buffer)
   float* Z = reinterpret_cast<float*>(smem + SM::CBUF);    // S during pass 1, then R
   float2* s_tw = reinterpret_cast<float2*>(smem + SM::CBUF + SM::ZBUF);
-  float2* s_h = reinterpret_cast<float2*>(smem + SM::CBUF + SM::ZBUF + SM::TWT);
-  float* s_gx = reinterpret_cast<float*>(smem + SM::CBUF + SM::ZBUF + SM::TWT + SM::HQ);
+  float2* s_tw2 = reinterpret_cast<float2*>(smem + SM::CBUF + SM::ZBUF + SM::TWT);
+  float2* s_h = s_tw2 + 64;
+  float* s_gx = reinterpret_cast<float*>(s_h + M);
   float* s_gy = s_gx + kMaxTaps;
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(s_gy + kMaxTaps);
 
@@ -138,6 +151,13 @@ __global__ void __launch_bounds__(SeqShape<M>::TR, SeqShape<M>::MIN_BLOCKS) pc_s
   for (int i = tid; i < G * TL::LDW; i += TR) {
     const int t = i / TL::LDW, k2 = i % TL::LDW;
     s_tw[i] = k2 < E ? a_in.tw[(t * k2) % M] : make_float2(0.f, 0.f);
+  }
+  // M >= 64: the three-pass transform (fft3.cuh), W_64^(yb ka) and this thread's W_M^yl
+  constexpr bool F3 = M >= 64;
+  float2 wy = make_float2(1.f, 0.f);
+  if constexpr (F3) {
+    for (int i = tid; i < 64; i += TR) s_tw2[i] = a_in.tw[(M / 64 * (i / 4) * (i % 4)) % M];
+    wy = a_in.tw[tid / G];
   }
   // per problem: Fresnel factors and taps (between CTA barriers)
   auto setup = [&](const FusedArgs& a) {
@@ -254,18 +274,43 @@ __global__ void __launch_bounds__(SeqShape<M>::TR, SeqShape<M>::MIN_BLOCKS) pc_s
     };
     using EstC = IntC<0>;
     using WaveC = IntC<MODE == DM ? 1 : 0>;  // the wave that carries the modulus step
-    // ---- forward propagation to the detector (far: COL layout; near: ROW layout, scaled)
+    // ---- 2-D transforms between the ROW layout and the frequency layout (row, col) = freq(q, r)
+    auto transform = [&](auto inv_c) {
+      constexpr bool INV = decltype(inv_c)::value != 0;
+      if constexpr (F3) {
+        if constexpr (INV) fft3_inverse<M>(v, cbuf, s_tw, s_tw2, wy, tid);
+        else fft3_forward<M>(v, cbuf, s_tw, s_tw2, wy, tid);
+      } else {
+        if constexpr (INV) fft2_inverse<M, V>(v, cbuf, s_tw, tid);
+        else fft2_forward<M, V>(v, cbuf, s_tw, tid);
+      }
+    };
+    auto freq = [&](int q, int r, int& row, int& col) {
+      if constexpr (F3) {
+        row = Tile3<M>::freq_row(tid, q, r);
+        col = Tile3<M>::freq_col(tid);
+      } else {
+        det_coords<M, false>(tid + q * TR, r, row, col);
+      }
+    };
+    // detector pixel of a register: the near field ends in the ROW layout, the far field in frequencies
+    auto pixel = [&](int q, int r, int& row, int& col) {
+      if constexpr (NEAR) det_coords<M, true>(tid + q * TR, r, row, col);
+      else freq(q, r, row, col);
+    };
+    // ---- forward propagation to the detector (far: frequency layout; near: ROW layout, scaled)
     auto forward = [&]() {
-      fft2_forward<M, V>(v, cbuf, s_tw, tid);
+      transform(IntC<0>{});
       if constexpr (NEAR) {
 #pragma unroll
         for (int q = 0; q < V; ++q)
 #pragma unroll
           for (int r = 0; r < E; ++r) {
-            const int vt = tid + q * TR;
-            v[q][r] = cmul(v[q][r], cmul(s_h[col_freq<M>(vt % G, r)], s_h[vt / G]));
+            int fu, fv;
+            freq(q, r, fu, fv);
+            v[q][r] = cmul(v[q][r], cmul(s_h[fu], s_h[fv]));
           }
-        fft2_inverse<M, V>(v, cbuf, s_tw, tid);
+        transform(IntC<1>{});
 #pragma unroll
         for (int q = 0; q < V; ++q)
 #pragma unroll
@@ -288,7 +333,7 @@ __global__ void __launch_bounds__(SeqShape<M>::TR, SeqShape<M>::MIN_BLOCKS) pc_s
 #pragma unroll
           for (int r = 0; r < E; ++r) {
             int row, col;
-            det_coords<M, NEAR>(tid + q * TR, r, row, col);
+            pixel(q, r, row, col);
             float s = cabs2(v[q][r]);
             if (k > 0) s += Z[row * LD + col];
             if (last && !a.blur_intensity) s = sqrtf(s);
@@ -394,25 +439,31 @@ __global__ void __launch_bounds__(SeqShape<M>::TR, SeqShape<M>::MIN_BLOCKS) pc_s
 #pragma unroll
         for (int r = 0; r < E; ++r) {
           int row, col;
-          det_coords<M, NEAR>(tid + q * TR, r, row, col);
+          pixel(q, r, row, col);
           v[q][r] = cscale(v[q][r], Z[row * LD + col]);
         }
       // back-propagation to ROW layout (times M^2)
       if constexpr (NEAR) {
-        fft2_forward<M, V>(v, cbuf, s_tw, tid);
+        transform(IntC<0>{});
 #pragma unroll
         for (int q = 0; q < V; ++q)
 #pragma unroll
           for (int r = 0; r < E; ++r) {
-            const int vt = tid + q * TR;
-            v[q][r] = cmulc(v[q][r], cmul(s_h[col_freq<M>(vt % G, r)], s_h[vt / G]));
+            int fu, fv;
+            freq(q, r, fu, fv);
+            v[q][r] = cmulc(v[q][r], cmul(s_h[fu], s_h[fv]));
           }
       }
-      fft2_inverse<M, V>(v, cbuf, s_tw, tid);
+      transform(IntC<1>{});
       // dpsi = psi' - P_k o_n; contributions, probe partials
       const float2* Pk = a.P + (size_t)k * M * M;
       float2* pk = MODE == DM ? Sn + (size_t)k * M * M : pacc + (size_t)k * M * M;  // (pc-DM: the mode's state)
       float* dk = dacc;
+      // groups of four values; the next group's probe values are loaded before this group's work (the
+      // tensor-memory waits are compiler barriers: loads behind them would each expose an L2 round trip)
+      float2 pn[4];
+#pragma unroll
+      for (int jj = 0; jj < 4; ++jj) pn[jj] = __ldg(&Pk[line[0] * M + tp[0] + G * jj]);
 #pragma unroll
       for (int q = 0; q < V; ++q) {
         const int ln = line[q];
@@ -420,7 +471,12 @@ __global__ void __launch_bounds__(SeqShape<M>::TR, SeqShape<M>::MIN_BLOCKS) pc_s
         for (int h = 0; h < E / 4; ++h) {
           float2 p[4];
 #pragma unroll
-          for (int jj = 0; jj < 4; ++jj) p[jj] = __ldg(&Pk[ln * M + tp[q] + G * (4 * h + jj)]);
+          for (int jj = 0; jj < 4; ++jj) p[jj] = pn[jj];
+          if (h + 1 < E / 4 || q + 1 < V) {
+            const int q2 = h + 1 < E / 4 ? q : q + 1 < V ? q + 1 : q, h2 = h + 1 < E / 4 ? h + 1 : 0;
+#pragma unroll
+            for (int jj = 0; jj < 4; ++jj) pn[jj] = __ldg(&Pk[line[q2] * M + tp[q2] + G * (4 * h2 + jj)]);
+          }
           float2 st[4];
           if constexpr (MODE == DM) {
 #pragma unroll
