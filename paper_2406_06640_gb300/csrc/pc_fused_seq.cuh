@@ -110,7 +110,7 @@ struct SeqSmem {
   static constexpr size_t CBUF = ((kX > kB ? kX : kB) + 15) / 16 * 16;
   static constexpr size_t ZBUF = (kB + 15) / 16 * 16;      // S, then R
   static constexpr size_t TWT = ((size_t)Tile<M>::G * Tile<M>::LDW * 8 + 15) / 16 * 16;
-  static constexpr size_t TW2 = 64 * 8;  // second twiddles of fft3.cuh
+  static constexpr size_t TW2 = (M >= 64 ? M : 0) * 8;  // second twiddles of fft3.cuh (Tile3::TW2)
   static constexpr size_t HQ = (size_t)M * 8;
   static constexpr size_t TAPS = 2 * kMaxTaps * 4 + 8;  // taps, TMEM address
   static constexpr size_t BYTES = CBUF + ZBUF + TWT + TW2 + HQ + TAPS;
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(SeqShape<M>::TR, SeqShape<M>::MIN_BLOCKS) pc_s
   float* Z = reinterpret_cast<float*>(smem + SM::CBUF);    // S during pass 1, then R
   float2* s_tw = reinterpret_cast<float2*>(smem + SM::CBUF + SM::ZBUF);
   float2* s_tw2 = reinterpret_cast<float2*>(smem + SM::CBUF + SM::ZBUF + SM::TWT);
-  float2* s_h = s_tw2 + 64;
+  float2* s_h = s_tw2 + SM::TW2 / 8;
   float* s_gx = reinterpret_cast<float*>(s_h + M);
   float* s_gy = s_gx + kMaxTaps;
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(s_gy + kMaxTaps);
@@ -152,13 +152,10 @@ __global__ void __launch_bounds__(SeqShape<M>::TR, SeqShape<M>::MIN_BLOCKS) pc_s
     const int t = i / TL::LDW, k2 = i % TL::LDW;
     s_tw[i] = k2 < E ? a_in.tw[(t * k2) % M] : make_float2(0.f, 0.f);
   }
-  // M >= 64: the three-pass transform (fft3.cuh), W_64^(yb ka) and this thread's W_M^yl
+  // M >= 64: the three-pass transform (fft3.cuh)
   constexpr bool F3 = M >= 64;
-  float2 wy = make_float2(1.f, 0.f);
-  if constexpr (F3) {
-    for (int i = tid; i < 64; i += TR) s_tw2[i] = a_in.tw[(M / 64 * (i / 4) * (i % 4)) % M];
-    wy = a_in.tw[tid / G];
-  }
+  if constexpr (F3)
+    for (int i = tid; i < Tile3<M>::TW2; i += TR) s_tw2[i] = a_in.tw[Tile3<M>::tw2_exp(i)];
   // per problem: Fresnel factors and taps (between CTA barriers)
   auto setup = [&](const FusedArgs& a) {
     if constexpr (NEAR)
@@ -278,8 +275,8 @@ __global__ void __launch_bounds__(SeqShape<M>::TR, SeqShape<M>::MIN_BLOCKS) pc_s
     auto transform = [&](auto inv_c) {
       constexpr bool INV = decltype(inv_c)::value != 0;
       if constexpr (F3) {
-        if constexpr (INV) fft3_inverse<M>(v, cbuf, s_tw, s_tw2, wy, tid);
-        else fft3_forward<M>(v, cbuf, s_tw, s_tw2, wy, tid);
+        if constexpr (INV) fft3_inverse<M>(v, cbuf, s_tw, s_tw2, tid);
+        else fft3_forward<M>(v, cbuf, s_tw, s_tw2, tid);
       } else {
         if constexpr (INV) fft2_inverse<M, V>(v, cbuf, s_tw, tid);
         else fft2_forward<M, V>(v, cbuf, s_tw, tid);

@@ -39,8 +39,7 @@ static int run() {
   std::vector<float2> tw(NT * 17), tw2(T::TW2);
   for (int t = 0; t < NT; ++t)
     for (int k = 0; k < 16; ++k) tw[t * 17 + k] = f2(W((long)t * k));
-  for (int yb = 0; yb < 16; ++yb)
-    for (int ka = 0; ka < 4; ++ka) tw2[yb * 4 + ka] = f2(W((long)S * yb * ka));
+  for (int i = 0; i < T::TW2; ++i) tw2[i] = f2(W(T::tw2_exp(i)));
   std::vector<cd> F(M * M), B(M * M);
   std::barrier<> bar(TR);
   g_bar = &bar;
@@ -49,13 +48,12 @@ static int run() {
     th.emplace_back([&, tid] {
       float2 a[S][16];
       const int yl = tid / NT, t = tid % NT;
-      const float2 wy = f2(W(yl));
       for (int s = 0; s < S; ++s)
         for (int j = 0; j < 16; ++j) a[s][j] = f2(A[(yl + 64 * s) * M + t + NT * j]);
-      fft3_forward<M>(a, sm, tw.data(), tw2.data(), wy, tid);
+      fft3_forward<M>(a, sm, tw.data(), tw2.data(), tid);
       for (int s = 0; s < S; ++s)
         for (int r = 0; r < 16; ++r) F[T::freq_row(tid, s, r) * M + T::freq_col(tid)] = cd(a[s][r].x, a[s][r].y);
-      fft3_inverse<M>(a, sm, tw.data(), tw2.data(), wy, tid);
+      fft3_inverse<M>(a, sm, tw.data(), tw2.data(), tid);
       for (int s = 0; s < S; ++s)
         for (int j = 0; j < 16; ++j) B[(yl + 64 * s) * M + t + NT * j] = cd(a[s][j].x, a[s][j].y);
     });
