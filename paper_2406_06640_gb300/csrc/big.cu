@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(kModTpb<BL>) k_big_modulus(const BigArgs b) {
   for (int w = threadIdx.x; w < HR * (BL / NB); w += TPB) {
     const int r = w % HR, c0 = (w / HR) * NB;
     float out[NB];
-    blur_strip<NB, KH>(sA, r * LD, 1, c0, 0, BL, s_gx, out);
+    blur_strip<NB, KH>(sA, r * LD, 1, c0, 0, BL, s_gx, b.kh, out);
 #pragma unroll
     for (int o = 0; o < NB; ++o) sB[r * LD + c0 + o] = out[o];
   }
@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(kModTpb<BL>) k_big_modulus(const BigArgs b) {
     float sq[NB], out[NB];
 #pragma unroll
     for (int o = 0; o < NB; ++o) sq[o] = __ldcs(&Sn[(size_t)(y0 + rs + o) * BL + x]);
-    blur_strip<NB, KH>(sB, x, LD, rs + KH, 0, HR, s_gy, out);
+    blur_strip<NB, KH>(sB, x, LD, rs + KH, 0, HR, s_gy, b.kh, out);
 #pragma unroll
     for (int o = 0; o < NB; ++o) {
       const float acc = out[o];

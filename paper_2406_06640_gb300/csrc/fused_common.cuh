@@ -88,46 +88,59 @@ __device__ __forceinline__ void det_coords(int vt, int r, int& row, int& col) {
   }
 }
 
+template <int X>
+struct IntC {
+  static constexpr int value = X;
+};
+
 // NO consecutive outputs of a zero-padded correlation along a line of a f32
 // buffer: out[o] = sum_d g[d] in[c0 + o + d - KH], samples outside [lo, hi)
-// read as zero; `stride` steps between consecutive samples.
+// read as zero; `stride` steps between consecutive samples. Taps beyond the
+// half-width kh are zero; KH = 15 leaves out those beyond 5 or 10 (21 taps:
+// 1022 -> 1011 us an iteration of 4096 positions of 128^2, one mode).
 template <int NO, int KH>
 __device__ __forceinline__ void blur_strip(const float* in, int base, int stride, int c0, int lo, int hi,
-                                           const float* g, float (&out)[NO]) {
-  constexpr int E = NO;
-  constexpr int W = E + 2 * KH;
-  float win[W];
-#pragma unroll
-  for (int i = 0; i < W; ++i) {
-    const int c = c0 - KH + i;
-    win[i] = (c >= lo && c < hi) ? in[base + c * stride] : 0.f;
-  }
+                                           const float* g, int kh, float (&out)[NO]) {
+  auto sample = [&](int c) { return (c >= lo && c < hi) ? in[base + c * stride] : 0.f; };
   if constexpr (KH <= 7) {
+    constexpr int W = NO + 2 * KH;
+    float win[W];
+#pragma unroll
+    for (int i = 0; i < W; ++i) win[i] = sample(c0 - KH + i);
     float gr[2 * KH + 1];
 #pragma unroll
     for (int d = 0; d < 2 * KH + 1; ++d) gr[d] = g[d];
 #pragma unroll
-    for (int o = 0; o < E; ++o) {
+    for (int o = 0; o < NO; ++o) {
       float acc = 0.f;
 #pragma unroll
       for (int d = 0; d < 2 * KH + 1; ++d) acc = fmaf(gr[d], win[o + d], acc);
       out[o] = acc;
     }
   } else {
+    static_assert(KH == 15, "tap groups");
 #pragma unroll
-    for (int o = 0; o < E; ++o) out[o] = 0.f;
+    for (int o = 0; o < NO; ++o) out[o] = 0.f;
+    // taps [D0, D1), in increasing order over the groups; each group loads its own samples (a window kept
+    // across the groups' branches spills)
+    auto taps = [&](auto d0_c, auto d1_c) {
+      constexpr int D0 = decltype(d0_c)::value, D1 = decltype(d1_c)::value, W = NO + D1 - D0 - 1;
+      float win[W];
 #pragma unroll
-    for (int d = 0; d < 2 * KH + 1; ++d) {
-      const float gd = g[d];
+      for (int i = 0; i < W; ++i) win[i] = sample(c0 - KH + D0 + i);
 #pragma unroll
-      for (int o = 0; o < E; ++o) out[o] = fmaf(gd, win[o + d], out[o]);
-    }
+      for (int d = D0; d < D1; ++d) {
+        const float gd = g[d];
+#pragma unroll
+        for (int o = 0; o < NO; ++o) out[o] = fmaf(gd, win[o + d - D0], out[o]);
+      }
+    };
+    if (kh > 10) taps(IntC<0>{}, IntC<5>{});
+    if (kh > 5) taps(IntC<5>{}, IntC<10>{});
+    taps(IntC<10>{}, IntC<21>{});
+    if (kh > 5) taps(IntC<21>{}, IntC<26>{});
+    if (kh > 10) taps(IntC<26>{}, IntC<31>{});
   }
 }
-
-template <int X>
-struct IntC {
-  static constexpr int value = X;
-};
 
 }  // namespace ptycho

@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
         const int lr = w % nrow, c0 = (w / nrow) * NB;
         const int gr = r0 + lr;
         float out[NB];
-        blur_strip<NB, KH>(X, lr * LD, 1, c0, 0, M, s_gx, out);
+        blur_strip<NB, KH>(X, lr * LD, 1, c0, 0, M, s_gx, a.kh, out);
 #pragma unroll
         for (int o = 0; o < NB; ++o) Yb[(lr + KH) * LD + c0 + o] = out[o];
         for (int q = 0; q < K; ++q) {
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
         for (int w = tid; w < M * nstrip; w += TR) {
           const int col = w % M, rs = (w / M) * NB;
           float out[NB];
-          blur_strip<NB, KH>(Yb, col, LD, rs + KH, 0, nrow + 2 * KH, s_gy, out);
+          blur_strip<NB, KH>(Yb, col, LD, rs + KH, 0, nrow + 2 * KH, s_gy, a.kh, out);
 #pragma unroll
           for (int o = 0; o < NB; ++o) {
             const int lr = rs + o;

@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(SeqShape<M>::TR, SeqShape<M>::MIN_BLOCKS) pc_s
       for (int w = tid; w < M * (M / NB); w += TR) {
         const int row = w % M, c0 = (w / M) * NB;
         float out[NB];
-        blur_strip<NB, KH>(Z, row * LD, 1, c0, 0, M, s_gx, out);
+        blur_strip<NB, KH>(Z, row * LD, 1, c0, 0, M, s_gx, a.kh, out);
 #pragma unroll
         for (int o = 0; o < NB; ++o) X[row * LD + c0 + o] = out[o];
       }
@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(SeqShape<M>::TR, SeqShape<M>::MIN_BLOCKS) pc_s
 #pragma unroll
         for (int o = 0; o < NB; ++o) sq[o] = __ldcs(&Qn[(rs + o) * M + col]);
         float out[NB];
-        blur_strip<NB, KH>(X, col, LD, rs, 0, M, s_gy, out);
+        blur_strip<NB, KH>(X, col, LD, rs, 0, M, s_gy, a.kh, out);
 #pragma unroll
         for (int o = 0; o < NB; ++o) {
           const float acc = out[o];
