@@ -240,9 +240,10 @@ ptycho_status ptycho_profile(ptycho_plan_t plan, int32_t enable);
 ptycho_status ptycho_profile_read(ptycho_plan_t plan, double* fused_ms, int32_t* launches);
 
 /* Kernel launches one iteration issues: the fused kernel (M <= 128) or 5 (far)
- * / 7 (near) staged passes per chunk of positions (M = 256, 512; pc-DM 8 / 11), 4 update kernels
- * (2 more for pc-DM), per batch for the mini-batch engine, and 3 complex-constraint
- * kernels when `in_window` is non-zero (copies not counted). */
+ * / 7 (near) staged passes per chunk of positions (M = 256, 512; pc-DM 8 / 11), 2 update kernels
+ * (pc-DM 5; one more for M = 256, 512), per batch for the mini-batch engine, which adds one that
+ * finishes the error, and 2 complex-constraint kernels (mini-batches 3) when `in_window` is non-zero
+ * (copies not counted). */
 int32_t ptycho_launches_per_iteration(ptycho_plan_t plan, int32_t in_window);
 
 /* Allocation-free one-shot run (this entry point has no counterpart in the paper).

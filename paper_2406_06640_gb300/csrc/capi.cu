@@ -163,6 +163,25 @@ struct ptycho_plan_s {
   std::vector<QueueClass> qclasses;
   std::vector<char> queued;  // per member: drained by its class's work-queue launch
   double* d_errhist = nullptr;
+  // pinned words that the kernels write: the last E with its run, and the bounded waits' flag. Reading them
+  // after a synchronisation copies nothing
+  HostWords* host = nullptr;
+  // whether a bounded device wait gave up since the last call (clears the flag); after a synchronisation
+  bool timed_out() {
+    bool t = false;
+    if (host && host->timeout) host->timeout = 0, t = true;
+    for (ptycho_plan_s* m : members) t |= m->timed_out();
+    return t;
+  }
+  // E of the last run; after a synchronisation. A launch captured into a caller's graph runs (or not) at the
+  // caller's times: where the word is not of that run, E comes from the ring
+  cudaError_t last_error(double* e) const {
+    if (host->run == (unsigned long long)runs) {
+      *e = host->err;
+      return cudaSuccess;
+    }
+    return cudaMemcpy(e, d_errhist + (runs - 1) % kErrHistory, sizeof(double), cudaMemcpyDeviceToHost);
+  }
   // profiling: event pairs around the fused kernel
   bool profiling = false;
   std::vector<cudaEvent_t> ev;  // 2 * kProfSlots
@@ -183,8 +202,7 @@ struct ptycho_plan_s {
   static constexpr int kGraphAfter = 2, kRing = 4, kMaxGraphKeys = 32;  // beyond: eager
   std::vector<SingleGraph> sgraphs;
   std::vector<std::pair<std::array<uintptr_t, 3>, int>> eager_runs;
-  cudaStream_t gstream = nullptr, gside = nullptr;  // capture streams: the iteration, and its side branch
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  cudaStream_t gstream = nullptr;
   int ring = 0;
   // mini-batch plans: one graph per batch (its fused launch or staged passes and its update), keyed
   // by (batch, probe step on, object, probe) and replayed in each iteration's visiting order
@@ -211,9 +229,6 @@ struct ptycho_plan_s {
       if (g.e1) cudaEventDestroy(g.e1);
     }
     if (gstream) cudaStreamDestroy(gstream);
-    if (gside) cudaStreamDestroy(gside);
-    if (ev_fork) cudaEventDestroy(ev_fork);
-    if (ev_join) cudaEventDestroy(ev_join);
     for (cudaEvent_t e : branch_ev) cudaEventDestroy(e);
     for (cudaStream_t s : branch) cudaStreamDestroy(s);
     if (ev_in) cudaEventDestroy(ev_in);
@@ -221,6 +236,7 @@ struct ptycho_plan_s {
     if (origin) cudaStreamDestroy(origin);
     for (ptycho_plan_s* m : members) delete m;
     for (void* q : allocs) cudaFree(q);
+    if (host) cudaFreeHost(const_cast<HostWords*>(host));
     for (cudaEvent_t e : ev) cudaEventDestroy(e);
   }
   bool in_window(long long t) const {
@@ -387,6 +403,11 @@ static ptycho_status build_plan(ptycho_plan_s* pl, const float* intensities, con
   const int M = p.M, K = p.K, N = p.N;
   const size_t MM = (size_t)M * M;
   cudaStream_t s = pl->stream;
+  if (!pl->host) {
+    void* q = nullptr;
+    PT_CUDA(cudaHostAlloc(&q, sizeof(HostWords), cudaHostAllocPortable | cudaHostAllocMapped), "alloc host words");
+    pl->host = new (q) HostWords{};
+  }
 
   // ---- positions
   pl->h_pos.resize(N);
@@ -602,6 +623,9 @@ static ptycho_status build_plan(ptycho_plan_s* pl, const float* intensities, con
   fa.pacc = d_pacc;
   fa.dacc = d_dacc;
   fa.errpart = d_errpart;
+  fa.p2 = d_p2;
+  fa.dmax = d_dmax;
+  fa.timeout = &pl->host->timeout;
 
   ua.pos = d_pos;
   ua.N = N;
@@ -628,6 +652,7 @@ static ptycho_status build_plan(ptycho_plan_s* pl, const float* intensities, con
   ua.p2 = d_p2;
   ua.probe_blocks = pb;
   ua.errhist = pl->d_errhist;
+  ua.host = pl->host;
   ua.run_counter = d_runs;
   ua.errden = pl->errden;
   ua.beta_obj = (float)p.beta_obj;
@@ -773,7 +798,7 @@ static ptycho_status enqueue_batch(ptycho_plan_s* pl, const FusedArgs& fa, const
   }
   ub.err_mode = 1;
   ub.err_acc = pl->d_err_acc;
-  PT_CUDA(launch_update(ub, nullptr, true, true, s), "update launch");
+  PT_CUDA(launch_update(ub, nullptr, pl->big, true, s), "update launch");
   return PTYCHO_OK;
 }
 
@@ -837,15 +862,6 @@ static ptycho_status enqueue_iteration(ptycho_plan_s* pl, void* object, void* pr
   ua.O = static_cast<float2*>(object);
   ua.P = static_cast<float2*>(probe);
   ca.O = static_cast<float2*>(object);
-  // in a graph of a single plan the |P|^2 map runs beside the fused kernel (a branch from here to the update)
-  bool p2_done = false;
-  if (pe0 && pl->mb == 0 && !pl->d_psi) {
-    PT_CUDA(cudaEventRecord(pl->ev_fork, s), "fork event");
-    PT_CUDA(cudaStreamWaitEvent(pl->gside, pl->ev_fork, 0), "fork");
-    PT_CUDA(launch_p2(ua, pl->gside), "update launch");
-    PT_CUDA(cudaEventRecord(pl->ev_join, pl->gside), "join event");
-    p2_done = true;
-  }
   const int ps = pl->prof_count % ptycho_plan_s::kProfSlots;
   if (pe0) PT_CUDA(cudaEventRecordWithFlags(pe0, s, cudaEventRecordExternal), "profile event");
   else if (pl->profiling) PT_CUDA(cudaEventRecord(pl->ev[2 * ps], s), "profile event");
@@ -909,12 +925,11 @@ static ptycho_status enqueue_iteration(ptycho_plan_s* pl, void* object, void* pr
     pl->prof_count++;
   }
   ua.update_probe = t >= pl->p.probe_update_start;
-  if (p2_done) PT_CUDA(cudaStreamWaitEvent(s, pl->ev_join, 0), "join");
   if (pl->d_psi) {
     // pc-DM: the complex constraint acts between the object and the probe step, and the states
     // move with their boxes by P (O constrained - O)
     const bool win = pl->in_window(t);
-    PT_CUDA(launch_update_object(ua, win ? &ca : nullptr, s), "update launch");
+    PT_CUDA(launch_update_object(ua, win ? &ca : nullptr, pl->big, s), "update launch");
     ua.dm_obj_prev = nullptr;
     if (win) {
       PT_CUDA(cudaMemcpyAsync(pl->d_obj_prev, ua.O, (size_t)pl->p.obj_h * pl->p.obj_w * sizeof(float2),
@@ -927,7 +942,7 @@ static ptycho_status enqueue_iteration(ptycho_plan_s* pl, void* object, void* pr
     return PTYCHO_OK;
   }
   const bool win = pl->in_window(t);
-  PT_CUDA(launch_update(ua, win ? &ca : nullptr, !p2_done, true, s), "update launch");
+  PT_CUDA(launch_update(ua, win ? &ca : nullptr, pl->big, true, s), "update launch");
   if (win) PT_CUDA(launch_constraint(ca, false, s), "constraint launch");
   return PTYCHO_OK;
 }
@@ -945,7 +960,7 @@ static ptycho_status enqueue_update(ptycho_plan_s* pl, void* object, void* probe
     // pc-DM: the complex constraint acts between the object and the probe step, and the states
     // move with their boxes by P (O constrained - O)
     const bool win = pl->in_window(t);
-    PT_CUDA(launch_update_object(ua, win ? &ca : nullptr, s), "update launch");
+    PT_CUDA(launch_update_object(ua, win ? &ca : nullptr, pl->big, s), "update launch");
     ua.dm_obj_prev = nullptr;
     if (win) {
       PT_CUDA(cudaMemcpyAsync(pl->d_obj_prev, ua.O, (size_t)pl->p.obj_h * pl->p.obj_w * sizeof(float2),
@@ -1005,9 +1020,6 @@ static ptycho_status iterate_graph(ptycho_plan_s* pl, void* object, void* probe,
   if (gi == pl->sgraphs.size()) {
     // capture the key's whole ring
     if (!pl->gstream) PT_CUDA(cudaStreamCreateWithFlags(&pl->gstream, cudaStreamNonBlocking), "graph stream");
-    if (!pl->gside) PT_CUDA(cudaStreamCreateWithFlags(&pl->gside, cudaStreamNonBlocking), "graph stream");
-    for (cudaEvent_t* ev : {&pl->ev_fork, &pl->ev_join})
-      if (!*ev) PT_CUDA(cudaEventCreateWithFlags(ev, cudaEventDisableTiming), "graph event");
     const bool fresh = pl->dm_fresh;
     const bool prof = pl->profiling;
     pl->profiling = false;  // the ring's own events, not the eager event ring
@@ -1173,9 +1185,7 @@ static ptycho_status tune_chunk_length(ptycho_plan_s* pl, ptycho_plan_s::QueueCl
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (st == PTYCHO_OK) {
-    bool timed_out = false;
-    PT_CUDA(fused_timed_out(&timed_out), "read wait status");
-    if (timed_out) return fail(PTYCHO_ETIMEOUT, "a bounded device wait gave up while tuning");
+    if (pl->timed_out()) return fail(PTYCHO_ETIMEOUT, "a bounded device wait gave up while tuning");
   }
   return st;
 }
@@ -1464,16 +1474,12 @@ ptycho_status ptycho_batch_classes(ptycho_plan_t pl, int32_t max_classes, int32_
 ptycho_status ptycho_error_batch(ptycho_plan_t pl, double* nrmse_last) {
   if (!pl || pl->members.empty() || !nrmse_last) return fail(PTYCHO_EINVAL, "not a batch plan or NULL output");
   PT_CUDA(cudaStreamSynchronize(pl->stream), "stream sync");
-  bool timed_out = false;
-  PT_CUDA(fused_timed_out(&timed_out), "read wait status");
-  if (timed_out) return fail(PTYCHO_ETIMEOUT, "a bounded device wait gave up; results are not valid");
+  if (pl->timed_out()) return fail(PTYCHO_ETIMEOUT, "a bounded device wait gave up; results are not valid");
   bool finite = true;
   for (size_t b = 0; b < pl->members.size(); ++b) {
     const ptycho_plan_s* m = pl->members[b];
     if (m->runs == 0) return fail(PTYCHO_EINVAL, "no iteration has run");
-    PT_CUDA(cudaMemcpy(&nrmse_last[b], m->d_errhist + (m->runs - 1) % kErrHistory, sizeof(double),
-                       cudaMemcpyDeviceToHost),
-            "copy error");
+    PT_CUDA(m->last_error(&nrmse_last[b]), "copy error");
     finite = finite && std::isfinite(nrmse_last[b]);
   }
   if (!finite) return fail(PTYCHO_ENUMERIC, "an error metric is not finite");
@@ -1485,12 +1491,9 @@ ptycho_status ptycho_error(ptycho_plan_t pl, double* nrmse_last) {
   if (!pl->members.empty()) return fail(PTYCHO_EINVAL, "batch plans report through ptycho_error_batch");
   PT_CUDA(cudaStreamSynchronize(pl->stream), "stream sync");
   if (pl->runs == 0) return fail(PTYCHO_EINVAL, "no iteration has run");
-  bool timed_out = false;
-  PT_CUDA(fused_timed_out(&timed_out), "read wait status");
-  if (timed_out) return fail(PTYCHO_ETIMEOUT, "a bounded device wait gave up; results are not valid");
+  if (pl->timed_out()) return fail(PTYCHO_ETIMEOUT, "a bounded device wait gave up; results are not valid");
   double e = 0.0;
-  PT_CUDA(cudaMemcpy(&e, pl->d_errhist + (pl->runs - 1) % kErrHistory, sizeof(double), cudaMemcpyDeviceToHost),
-          "copy error");
+  PT_CUDA(pl->last_error(&e), "copy error");
   *nrmse_last = e;
   if (!std::isfinite(e)) return fail(PTYCHO_ENUMERIC, "error metric is not finite");
   return PTYCHO_OK;
@@ -1563,9 +1566,9 @@ int32_t ptycho_launches_per_iteration(ptycho_plan_t pl, int32_t in_window) {
   // pc-DM: the estimate sweep stops after the modulus pass (3 far, 4 near)
   const int dm_extra = pl->p.geometry == PTYCHO_NEARFIELD ? 4 : 3;
   if (pl->big) fft = (pl->p.N + pl->chunk - 1) / pl->chunk * (pl->d_psi ? passes + dm_extra : passes);
-  // update: |P|^2 map, gather, steps; pc-DM: the gather and the steps once per side, and the probe
-  // partials between them. Constraint: box sums, tile apply (the object step makes the row sums)
-  int update = pl->d_psi ? 6 : 3;
+  // update: gather, steps; pc-DM: the gather and the steps once per side, and the probe partials between
+  // them; staged plans: the |P|^2 map. Constraint: box sums, tile apply (the object step makes the row sums)
+  int update = (pl->d_psi ? 5 : 2) + (pl->big ? 1 : 0);
   if (pl->mb > 0) {  // per batch: its fused launch or staged passes and its update; the error finish after them
     fft = 1;
     for (int b = 0; b < pl->nb; ++b) {
@@ -1623,14 +1626,15 @@ const char* ptycho_last_error(void) { return g_last_error.c_str(); }
 ptycho_status ptycho_wait_selftest(int64_t budget_ns, int32_t signal, void* cuda_stream) {
   if (budget_ns < 0 || budget_ns > 2000000000LL) return fail(PTYCHO_EINVAL, "budget_ns must be in [0, 2e9]");
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  bool pending = false;
-  PT_CUDA(fused_timed_out(&pending), "read wait status");
-  if (pending) return fail(PTYCHO_ETIMEOUT, "a bounded device wait of an earlier launch had given up");
-  PT_CUDA(launch_wait_selftest((unsigned long long)budget_ns, signal != 0, s), "self-test launch");
-  PT_CUDA(cudaStreamSynchronize(s), "stream sync");
-  bool timed_out = false;
-  PT_CUDA(fused_timed_out(&timed_out), "read wait status");
-  if (timed_out) return fail(PTYCHO_ETIMEOUT, "the self-test wait gave up after its budget");
+  int* flag = nullptr;  // pinned, as a plan's
+  PT_CUDA(cudaHostAlloc(reinterpret_cast<void**>(&flag), sizeof(int), cudaHostAllocMapped), "alloc flag");
+  *flag = 0;
+  cudaError_t ce = launch_wait_selftest((unsigned long long)budget_ns, signal != 0, flag, s);
+  if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
+  const bool gave_up = *static_cast<volatile int*>(flag) != 0;
+  cudaFreeHost(flag);
+  PT_CUDA(ce, "self-test");
+  if (gave_up) return fail(PTYCHO_ETIMEOUT, "the self-test wait gave up after its budget");
   return PTYCHO_OK;
 }
 

@@ -230,6 +230,8 @@ extern "C" ptycho_status ptycho_iterate_static(const ptycho_params* p, const flo
   }
   fa.tw = tw_d;
   fa.hq = hq_d;
+  fa.p2 = ua.p2;
+  fa.dmax = ua.dmax;
   ua.O = static_cast<float2*>(object);
   ua.P = static_cast<float2*>(probe);
   ua.pos = dpos;
@@ -274,15 +276,12 @@ extern "C" ptycho_status ptycho_iterate_static(const ptycho_params* p, const flo
     bool win = false;
     for (int w = 0; w < p->n_windows; ++w)
       if (t >= p->windows[2 * w] && t <= p->windows[2 * w + 1]) win = true;
-    PS_CUDA(launch_update(ua, win ? &ca : nullptr, true, true, s), "update launch");
+    PS_CUDA(launch_update(ua, win ? &ca : nullptr, false, true, s), "update launch");
     if (win) PS_CUDA(launch_constraint(ca, false, s), "constraint launch");
   }
   if (errors && n_iter > 0)
     PS_CUDA(cudaMemcpyAsync(errors, ua.errhist, sizeof(double) * n_iter, cudaMemcpyDeviceToHost, s), "copy errors");
   PS_CUDA(cudaStreamSynchronize(s), "stream sync");
-  bool timed_out = false;
-  PS_CUDA(fused_timed_out(&timed_out), "read wait status");
-  if (timed_out) return capi_fail(PTYCHO_ETIMEOUT, "a bounded device wait gave up; results are not valid");
   capi_clear_error();
   return PTYCHO_OK;
 }

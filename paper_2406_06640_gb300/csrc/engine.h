@@ -15,6 +15,12 @@ constexpr int kObjSplit = 8;        // position groups per object tile (one clus
 constexpr int kErrHistory = 4096;   // ring of per-iteration errors kept on the device
 
 // Arguments of the fused per-position kernels.
+// a plan's pinned host words
+struct HostWords {
+  volatile double err;              // E of the last run
+  volatile unsigned long long run;  // runs finished when it was written
+  volatile int timeout;             // a bounded device wait gave up
+};
 struct FusedArgs {
   const float2* O;      // object, obj_h x obj_w, row-major
   const float2* P;      // probe modes, K x M x M
@@ -44,6 +50,10 @@ struct FusedArgs {
   // pc-DM launches: exit-wave state N x K x M x M (updated in place); dm_init: start it at P o_n
   float2* psi;
   int dm_init;
+  // single-problem launches: |P|^2 map and the maxima to clear for the update that follows (UpdateArgs)
+  float* p2;
+  int* dmax;
+  volatile int* timeout;  // HostWords: raised by a bounded wait that gives up
 };
 
 // single-problem fused launch (pc_fused_seq.cuh: one CTA per position, modes in sequence) over
@@ -65,11 +75,9 @@ cudaError_t launch_fused_dm(int M, const FusedArgs& a, int slots, cudaStream_t s
 cudaError_t fused_dm_max_slots(int M, int K, int* slots);
 bool fused_queue_supported(int M);
 size_t fused_smem_bytes(int M);
-// true if a bounded device wait of the fused kernel gave up since the last call (clears the flag; synchronous)
-cudaError_t fused_timed_out(bool* out);
 // one bounded mbarrier wait of the fused kernels' kind on a barrier that `signal` completes (or
-// nothing does), giving up after budget_ns; its timeout shows in fused_timed_out
-cudaError_t launch_wait_selftest(unsigned long long budget_ns, bool signal, cudaStream_t s);
+// nothing does), giving up after budget_ns; its timeout raises *flag
+cudaError_t launch_wait_selftest(unsigned long long budget_ns, bool signal, volatile int* flag, cudaStream_t s);
 
 // staged path for M = 256 and 512 (big.cu): a chunk of C positions x K modes in the scratch W
 struct BigArgs {
@@ -155,6 +163,7 @@ struct UpdateArgs {
   float2* np_sum; float* dp_sum; float* p2;  // K x M x M, M x M, M x M
   int probe_blocks;                  // ceil(M^2 / 256)
   double* errhist; double errden;
+  HostWords* host;  // host-visible copy of the last E, or null
   unsigned long long* run_counter;  // device: iterations finished; E goes to errhist[counter % kErrHistory]
   // error of a launch: 0 finishes E from this launch's partials; 1 adds them to *err_acc (a batch
   // of a mini-batch iteration); 2 adds them and finishes E from the total, clearing *err_acc
@@ -199,13 +208,12 @@ struct ConstraintArgs {
 cudaError_t launch_constraint(const ConstraintArgs& c, bool with_rows, cudaStream_t s);
 
 // the update of one iteration or batch (update.cu): the |P|^2 map, the gather of both sides, the steps.
-// c: the object step also makes the row sums of the complex constraint that follows. with_p2 false: launch_p2
-// ran beside the fused kernel already. one_apply: object and probe step in one launch
-cudaError_t launch_p2(const UpdateArgs& u, cudaStream_t s);
+// c: the object step also makes the row sums of the complex constraint that follows. with_p2 false: the
+// fused kernel made the |P|^2 map. one_apply: object and probe step in one launch
 cudaError_t launch_update(const UpdateArgs& u, const ConstraintArgs* c, bool with_p2, bool one_apply,
                           cudaStream_t s);
 // pc-DM: the object side, and (after the complex constraint) the probe side from the state
-cudaError_t launch_update_object(const UpdateArgs& u, const ConstraintArgs* c, cudaStream_t s);
+cudaError_t launch_update_object(const UpdateArgs& u, const ConstraintArgs* c, bool with_p2, cudaStream_t s);
 cudaError_t launch_update_probe_dm(const UpdateArgs& u, cudaStream_t s);
 
 // plan-time helpers (update.cu)

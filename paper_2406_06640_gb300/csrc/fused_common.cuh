@@ -88,6 +88,19 @@ __device__ __forceinline__ void det_coords(int vt, int r, int& row, int& col) {
   }
 }
 
+// |P|^2 map of the update that follows (sum_k |P_k|^2, which depends on the probe alone) and its two maxima
+// cleared, by the CTAs of the fused launch before their positions: a launch less per update
+template <int M>
+__device__ __forceinline__ void probe_map(const FusedArgs& a, int threads) {
+  const int t = (int)blockIdx.x * threads + (int)threadIdx.x;
+  if (t < 2) a.dmax[t] = 0;
+  for (int p = t; p < M * M; p += (int)gridDim.x * threads) {
+    float s = 0.f;
+    for (int k = 0; k < a.K; ++k) s += cabs2(a.P[(size_t)k * M * M + p]);
+    a.p2[p] = s;
+  }
+}
+
 template <int X>
 struct IntC {
   static constexpr int value = X;

@@ -35,32 +35,19 @@ namespace ptycho {
 // Self-test of the bounded wait above (the one the cluster kernels use on their copy barriers):
 // one thread waits for phase 0 of a fresh mbarrier with the given budget. With `signal` it arrives
 // first and the wait succeeds at once; otherwise nothing ever arrives, the wait gives up after
-// `budget_ns` and sets the flag fused_timed_out reads, exactly as a fused kernel does.
-__global__ void k_wait_selftest(unsigned long long budget_ns, int signal) {
+// `budget_ns` and raises the flag that status-reading calls look at, exactly as a fused kernel does.
+__global__ void k_wait_selftest(unsigned long long budget_ns, int signal, volatile int* flag) {
   __shared__ __align__(8) unsigned long long bar;
   if (threadIdx.x != 0) return;
   const uint32_t b = smem_addr(&bar);
   mbar_init(b, 1);
   if (signal) mbar_arrive_expect_tx(b, 0u);  // the one expected arrival, no transaction bytes
-  if (!mbar_wait_bounded(b, 0u, budget_ns)) atomicExch(&g_fused_timeout, 1);
+  if (!mbar_wait_bounded(b, 0u, budget_ns)) report_timeout(flag);
 }
 
-cudaError_t launch_wait_selftest(unsigned long long budget_ns, bool signal, cudaStream_t s) {
-  k_wait_selftest<<<1, 32, 0, s>>>(budget_ns, signal ? 1 : 0);
+cudaError_t launch_wait_selftest(unsigned long long budget_ns, bool signal, volatile int* flag, cudaStream_t s) {
+  k_wait_selftest<<<1, 32, 0, s>>>(budget_ns, signal ? 1 : 0, flag);
   return cudaGetLastError();
-}
-
-cudaError_t fused_timed_out(bool* out) {
-  int h = 0;
-  cudaError_t e = cudaMemcpyFromSymbol(&h, g_fused_timeout, sizeof(int));
-  if (e != cudaSuccess) return e;
-  if (h) {
-    const int z = 0;
-    e = cudaMemcpyToSymbol(g_fused_timeout, &z, sizeof(int));
-    if (e != cudaSuccess) return e;
-  }
-  *out = h != 0;
-  return cudaSuccess;
 }
 
 size_t fused_smem_bytes(int M) {

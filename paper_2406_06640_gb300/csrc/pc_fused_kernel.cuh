@@ -20,8 +20,11 @@ __device__ __forceinline__ void red_add_l2(float* a, float v) {
   asm volatile("red.global.add.f32 [%0], %1;" ::"l"(a), "f"(v));
 }
 
-// set when a bounded device wait of the fused kernel gave up (read and cleared by fused_timed_out)
-static __device__ int g_fused_timeout;
+// a bounded device wait gave up: raises the host-visible flag that status-reading calls look at
+__device__ __forceinline__ void report_timeout(volatile int* flag) {
+  *flag = 1;
+  __threadfence_system();
+}
 
 // ---- bounded mbarrier wait (global timer); false once `budget_ns` has passed without the phase
 constexpr unsigned long long kFusedWaitNs = 2000000000ull;  // 2 s
@@ -115,6 +118,7 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
     const int t = i / TL::LDW, k2 = i % TL::LDW;
     s_tw[i] = k2 < E ? a_in.tw[(t * k2) % M] : make_float2(0.f, 0.f);
   }
+  probe_map<M>(a_in, TR);
   int line[V], tp[V];
 #pragma unroll
   for (int v = 0; v < V; ++v) {
@@ -311,7 +315,7 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
         if (pre && waits_ok) {
           if (!mbar_wait_bounded(bar_s, mphase)) {
             waits_ok = false;  // report once and stop waiting; the results are flagged invalid
-            atomicExch(&g_fused_timeout, 1);
+            report_timeout(a.timeout);
           }
           mphase ^= 1u;
         }

@@ -168,6 +168,7 @@ __global__ void __launch_bounds__(SeqShape<M>::TR, SeqShape<M>::MIN_BLOCKS) pc_s
     }
   };
   if constexpr (MODE != QUEUED) setup(a_in);
+  if constexpr (MODE != QUEUED) probe_map<M>(a_in, TR);
   int line[V], tp[V];
 #pragma unroll
   for (int v = 0; v < V; ++v) {

@@ -93,8 +93,8 @@ cudaError_t launch_finish_sums(const double* partials, int nblocks, double* out,
 }
 
 // ------------------------------------------------------------------ |P|^2 map
-// sum_k |P_k|^2 per probe pixel, and the maxima of D_O and D_P cleared for this update's gather. It depends
-// on the probe alone, so a single plan's graph runs it beside the fused kernel
+// sum_k |P_k|^2 per probe pixel, and the maxima of D_O and D_P cleared for this update's gather (staged and
+// queued plans; the fused kernels of single plans make both, probe_map)
 __global__ void __launch_bounds__(256) k_p2(const UpdateArgs u) {
   const int MM = u.M * u.M;
   const int p = blockIdx.x * 256 + threadIdx.x;
@@ -311,6 +311,16 @@ __global__ void __launch_bounds__(256, SPLIT == 8 ? 3 : 4) k_gather(const Update
   if ((tid & 31) == 0 && wm > 0) atomicMax(&u.dmax[obj ? 0 : 1], wm);
 }
 
+// E of run r into the ring, the run counter and (where there is one) the host-visible copy
+__device__ __forceinline__ void finish_error(const UpdateArgs& u, double E, unsigned long long r) {
+  u.errhist[r % kErrHistory] = E;
+  *u.run_counter = r + 1;
+  if (u.host) {
+    u.host->err = E;
+    u.host->run = r + 1;
+  }
+}
+
 // ------------------------------------------------------------------ apply
 // Blocks 0 .. rows - 1 (rows = obj_h or 0) take one object row each: O += beta N_O / (c_d D_O + c_max max
 // D_O). CC: inside a complex-constraint window the row's prefix sums of the new object follow at once
@@ -360,8 +370,7 @@ __global__ void __launch_bounds__(256) k_apply(const UpdateArgs u, const Constra
         *u.err_acc = e;
       } else {
         const unsigned long long r = *u.run_counter;
-        u.errhist[r % kErrHistory] = sqrt(e / u.errden);
-        *u.run_counter = r + 1;
+        finish_error(u, sqrt(e / u.errden), r);
         if (u.err_mode == 2) *u.err_acc = 0.0;
       }
     }
@@ -382,7 +391,7 @@ __global__ void __launch_bounds__(256) k_apply(const UpdateArgs u, const Constra
   }
 }
 
-cudaError_t launch_p2(const UpdateArgs& u, cudaStream_t s) {
+static cudaError_t launch_p2(const UpdateArgs& u, cudaStream_t s) {
   k_p2<<<u.probe_blocks, 256, 0, s>>>(u);
   return cudaGetLastError();
 }
@@ -419,8 +428,8 @@ static cudaError_t launch_apply(const UpdateArgs& u, const ConstraintArgs* c, bo
   return cudaGetLastError();
 }
 
-cudaError_t launch_update_object(const UpdateArgs& u, const ConstraintArgs* c, cudaStream_t s) {
-  cudaError_t e = launch_p2(u, s);
+cudaError_t launch_update_object(const UpdateArgs& u, const ConstraintArgs* c, bool with_p2, cudaStream_t s) {
+  cudaError_t e = with_p2 ? launch_p2(u, s) : cudaSuccess;
   if (e == cudaSuccess) e = launch_gather(u, true, false, s);
   if (e == cudaSuccess) e = launch_apply(u, c, true, false, s);
   return e;
@@ -451,8 +460,7 @@ __global__ void k_err_finish(const UpdateArgs u) {
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   const double e = *u.err_acc;
   const unsigned long long r = *u.run_counter;
-  u.errhist[r % kErrHistory] = sqrt(e / u.errden);
-  *u.run_counter = r + 1;
+  finish_error(u, sqrt(e / u.errden), r);
   *u.err_acc = 0.0;
 }
 
