@@ -42,6 +42,16 @@ struct Tile3 {
   __device__ __forceinline__ static int freq_col(int tid) { return tid % M; }
 };
 
+// exchange buffer of a fused kernel's 2-D transform: this file's for M = 64 and 128, fft.cuh's below
+template <int M, bool F3 = (M >= 64)>
+struct ExchangeBytes {
+  static constexpr size_t value = (size_t)Tile<M>::SMEM * 8;
+};
+template <int M>
+struct ExchangeBytes<M, true> {
+  static constexpr size_t value = (size_t)Tile3<M>::SMEM * 8;
+};
+
 // tw[t * 17 + k2] = W_M^(t k2), tw2 the table described at Tile3::TW2.
 // The shared buffer must be free on entry; it is free again on return.
 template <int M>

@@ -6,6 +6,7 @@
 #include "engine.h"
 #include "cluster.cuh"
 #include "fft.cuh"
+#include "fft3.cuh"
 #include "fused_common.cuh"
 
 namespace ptycho {
@@ -57,7 +58,7 @@ constexpr int max_slot_rows(int M) {
 template <int M, int KH>
 struct FusedSmem {
   static constexpr int LD = M + 1;  // padded row stride of the f32 detector buffers
-  static constexpr size_t kX = (size_t)Tile<M>::SMEM * 8;  // FFT exchange buffer
+  static constexpr size_t kX = ExchangeBytes<M>::value;  // FFT exchange buffer
   // modulus phase (aliases the exchange buffer): R (M rows) + own x-blurred rows with halos
   static constexpr size_t kF = (size_t)(M + M + 2 * KH) * LD * 4;
   // contributions received from every rank for the own rows
@@ -68,7 +69,8 @@ struct FusedSmem {
   static constexpr size_t TWT = ((size_t)Tile<M>::G * Tile<M>::LDW * 8 + 15) / 16 * 16;  // twiddle table
   static constexpr size_t HQ = (size_t)M * 8;                                             // Fresnel factors
   static constexpr size_t TAPS = 2 * kMaxTaps * 4 + 8 + 16;  // taps, TMEM address, mbarrier (16-byte aligned)
-  static constexpr size_t BYTES = CBUF + IBUF + TWT + HQ + TAPS;
+  static constexpr size_t TW2 = (M >= 64 ? M : 0) * 8;  // second twiddles of fft3.cuh (Tile3::TW2)
+  static constexpr size_t BYTES = CBUF + IBUF + TWT + TW2 + HQ + TAPS;
   static_assert(BYTES <= 232448, "shared memory budget of one CTA");
 };
 
@@ -102,8 +104,9 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
   float2* recv = cbuf;                        // contributions for the own rows, one slot per source rank
   float* ibuf = reinterpret_cast<float*>(smem + SM::CBUF);  // |Psi|^2 for the own rows, one slot per rank
   float2* s_tw = reinterpret_cast<float2*>(smem + SM::CBUF + SM::IBUF);
-  float2* s_h = reinterpret_cast<float2*>(smem + SM::CBUF + SM::IBUF + SM::TWT);
-  float* s_gx = reinterpret_cast<float*>(smem + SM::CBUF + SM::IBUF + SM::TWT + SM::HQ);
+  float2* s_tw2 = reinterpret_cast<float2*>(smem + SM::CBUF + SM::IBUF + SM::TWT);
+  float2* s_h = s_tw2 + SM::TW2 / 8;
+  float* s_gx = reinterpret_cast<float*>(s_h + M);
   float* s_gy = s_gx + kMaxTaps;
 
   const int tid = threadIdx.x;
@@ -118,6 +121,10 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
     const int t = i / TL::LDW, k2 = i % TL::LDW;
     s_tw[i] = k2 < E ? a_in.tw[(t * k2) % M] : make_float2(0.f, 0.f);
   }
+  // M >= 64: the three-pass transform (fft3.cuh)
+  constexpr bool F3 = M >= 64;
+  if constexpr (F3)
+    for (int i = tid; i < Tile3<M>::TW2; i += TR) s_tw2[i] = a_in.tw[Tile3<M>::tw2_exp(i)];
   probe_map<M>(a_in, TR);
   int line[V], tp[V];
 #pragma unroll
@@ -194,6 +201,30 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
     const float2* On = a.O + (size_t)pn.x * a.obj_w + pn.y;
     float2 v[V][E];
 
+    // ---- 2-D transforms between the ROW layout and the frequency layout (row, col) = freq(q, r); detector
+    // pixel of a register (the near field ends in the ROW layout, the far field in frequencies)
+    auto transform = [&](auto inv_c) {
+      constexpr bool INV = decltype(inv_c)::value != 0;
+      if constexpr (F3) {
+        if constexpr (INV) fft3_inverse<M>(v, cbuf, s_tw, s_tw2, tid);
+        else fft3_forward<M>(v, cbuf, s_tw, s_tw2, tid);
+      } else {
+        if constexpr (INV) fft2_inverse<M, V>(v, cbuf, s_tw, tid);
+        else fft2_forward<M, V>(v, cbuf, s_tw, tid);
+      }
+    };
+    auto freq = [&](int q, int r, int& row, int& col) {
+      if constexpr (F3) {
+        row = Tile3<M>::freq_row(tid, q, r);
+        col = Tile3<M>::freq_col(tid);
+      } else {
+        det_coords<M, false>(tid + q * TR, r, row, col);
+      }
+    };
+    auto pixel = [&](int q, int r, int& row, int& col) {
+      if constexpr (NEAR) det_coords<M, true>(tid + q * TR, r, row, col);
+      else freq(q, r, row, col);
+    };
     // ---- exit wave P o_n in ROW layout; far field: times (-1)^(y + x), which centres the transform
     auto exit_wave = [&]() {
       if constexpr (TM) {
@@ -236,16 +267,17 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
     // whole tile)
     auto detector = [&]() {
       // ---- forward propagation
-      fft2_forward<M, V>(v, cbuf, s_tw, tid);  // COL layout
+      transform(IntC<0>{});
       if constexpr (NEAR) {
 #pragma unroll
         for (int q = 0; q < V; ++q)
 #pragma unroll
           for (int r = 0; r < E; ++r) {
-            const int vt = tid + q * TR;
-            v[q][r] = cmul(v[q][r], cmul(s_h[col_freq<M>(vt % G, r)], s_h[vt / G]));
+            int fu, fv;
+            freq(q, r, fu, fv);
+            v[q][r] = cmul(v[q][r], cmul(s_h[fu], s_h[fv]));
           }
-        fft2_inverse<M, V>(v, cbuf, s_tw, tid);  // ROW layout, times M^2
+        transform(IntC<1>{});  // ROW layout, times M^2
 #pragma unroll
         for (int q = 0; q < V; ++q)
 #pragma unroll
@@ -268,7 +300,7 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
 #pragma unroll
         for (int r = 0; r < E; ++r) {
           int row, col;
-          det_coords<M, NEAR>(tid + q * TR, r, row, col);
+          pixel(q, r, row, col);
           const int ow = row / RPO;
           const int lr = row - ow * RPO;
           st_cluster_f32(map_rank(ibuf_s + (uint32_t)(((rank * RPO + lr) * LD + col) * 4), (unsigned)ow),
@@ -359,22 +391,23 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
 #pragma unroll
       for (int r = 0; r < E; ++r) {
         int row, col;
-        det_coords<M, NEAR>(tid + q * TR, r, row, col);
+        pixel(q, r, row, col);
         v[q][r] = cscale(v[q][r], Z[row * LD + col]);
       }
     __syncthreads();  // Z aliases the exchange buffer
     // ---- (6) back-propagation to ROW layout
     if constexpr (NEAR) {
-      fft2_forward<M, V>(v, cbuf, s_tw, tid);
+      transform(IntC<0>{});
 #pragma unroll
       for (int q = 0; q < V; ++q)
 #pragma unroll
         for (int r = 0; r < E; ++r) {
-          const int vt = tid + q * TR;
-          v[q][r] = cmulc(v[q][r], cmul(s_h[col_freq<M>(vt % G, r)], s_h[vt / G]));
+          int fu, fv;
+          freq(q, r, fu, fv);
+          v[q][r] = cmulc(v[q][r], cmul(s_h[fu], s_h[fv]));
         }
     }
-    fft2_inverse<M, V>(v, cbuf, s_tw, tid);
+    transform(IntC<1>{});
     cluster_sync_all();  // every rank is done with its exchange buffer, which now receives contributions
     // ---- (7) dpsi; probe partials; conj(P) dpsi pushed to the row owner
 #pragma unroll

@@ -92,20 +92,10 @@ struct SeqShape {
   static constexpr int MIN_BLOCKS = M == 64 ? 2 : 1;
 };
 
-// exchange buffer of the 2-D transform: fft3.cuh for M = 64 and 128, fft.cuh below
-template <int M, bool F3 = (M >= 64)>
-struct SeqExchange {
-  static constexpr size_t BYTES = (size_t)Tile<M>::SMEM * 8;
-};
-template <int M>
-struct SeqExchange<M, true> {
-  static constexpr size_t BYTES = (size_t)Tile3<M>::SMEM * 8;
-};
-
 template <int M>
 struct SeqSmem {
   static constexpr int LD = M + 1;  // padded row stride of the f32 detector buffers
-  static constexpr size_t kX = SeqExchange<M>::BYTES;
+  static constexpr size_t kX = ExchangeBytes<M>::value;  // FFT exchange buffer
   static constexpr size_t kB = (size_t)M * LD * 4;         // one f32 detector buffer
   static constexpr size_t CBUF = ((kX > kB ? kX : kB) + 15) / 16 * 16;
   static constexpr size_t ZBUF = (kB + 15) / 16 * 16;      // S, then R
