@@ -14,9 +14,10 @@
 //                  t -> k1. The twiddle of line yl = yb + 16 ya for bit s is split: W_8^(ya s) in front of
 //                  the DFT-4 (no table; s is uniform over a warp), W_M^(yb s) together with W_64^(yb ka)
 //                  behind it: one multiplication fewer per value than W_M^(yl s) in pass A. The DFT-4 comes
-//                  first for the rounding: a model whose dark pixels amplify the transform's rounding (200 counts per pattern, flat
+//                  first for the rounding: a model whose dark pixels amplify it (200 counts per pattern, flat
 //                  start, 12 global phases of the probe) deviates from FP64 by 6.9e-5 in the median and
-//                  8.8e-5 at most, against 8.9e-5 and 1.3e-4 with the DFT-NT in front (7.0e-5 and 1.1e-4 for the row / transpose / column form).
+//                  8.8e-5 at most, against 8.9e-5 and 1.3e-4 with the DFT-NT in front (7.0e-5 and 1.1e-4 for
+//                  the row / transpose / column form).
 //   exchange 2     slot col + M (ka + 4 yb + 64 s), col = k2 + 16 k1: both sides run along col
 //   pass C         thread (col, ka) = (tid % M, tid / M): DFT-16 over yb -> kb
 //   FREQ layout    register a[s][kb] holds frequency row s + S (ka + 4 kb), column col
