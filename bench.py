@@ -282,7 +282,8 @@ def traffic_record(kernel_tag, name="fused_kernel_traffic.json", workload="far12
     return rec.get("dram_bytes_per_launch_full_size")
 
 
-def kernel_source_hash(files=("cluster.cuh", "fft.cuh", "fused_common.cuh", "pc_fused_seq.cu"), struct="FusedArgs"):
+def kernel_source_hash(files=("cluster.cuh", "fft.cuh", "fft3.cuh", "fused_common.cuh", "pc_fused_seq.cuh",
+                              "pc_fused_seq.cu"), struct="FusedArgs"):
     """Hash of what a kernel is compiled from: its sources and its argument struct."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2406_06640_gb300", "csrc")
@@ -301,7 +302,7 @@ def kernel_label(prob, params):
     if params.get("minibatch", 0):
         return f"pc_seq_kernel<{prob.M}, {geo}> per batch with its update kernels (events around the batch loop)"
     if params.get("engine") == "dm":
-        return f"pc_fused_kernel<{prob.M}, {geo}, DM>"
+        return f"pc_seq_kernel<{prob.M}, {geo}, DM>"
     return f"pc_seq_kernel<{prob.M}, {geo}>"
 
 
