@@ -489,7 +489,7 @@ def run_ours_mono(args):
                            "parallelism": f"replicas{ws}" if ws > 1 else "single GPU"},
                 "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                              "frac": achieved / peak, "traffic": traffic,
-                             "kernel": "k_mono_cgls_band (M=256, clusters of 4)" if M == 256 else f"k_mono_cgls<{M}>",
+                             "kernel": f"k_mono_walk<{M}>" if M >= 64 else f"k_mono_cgls<{M}>",
                              "peak_basis": "152 SMs x 128 FP32 lanes x 2 FLOP x 2070 MHz (FMA pipe, max clock)",
                              "flops_per_launch": flops, "avg_launch_ms": avg_s * 1e3},
                 "cpu_baseline": cpu,
