@@ -393,14 +393,14 @@ __global__ void k_weights_bf16(const float* w, bf16* wb, bf16* wr, int Cp, int C
   }
 }
 
-// out (Mo, 16) fp32, first 2 channels used; target (Mo, 2). d_out bf16 (Mo, 16), one pixel per thread
+// out (Mo, 16) fp32, first 2 channels used; target (Mo, 2), the caller's: aligned to its floats, no more, so
+// read one by one. d_out bf16 (Mo, 16), one pixel per thread
 __global__ void k_loss_grad(const float* out, const float* target, bf16* d_out, int Mo) {
   const float inv = 1.0f / (2.0f * Mo);
   uint4* d4 = reinterpret_cast<uint4*>(d_out);
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < Mo; p += gridDim.x * blockDim.x) {
     const float2 o = *reinterpret_cast<const float2*>(out + (size_t)p * 16);
-    const float2 t = reinterpret_cast<const float2*>(target)[p];
-    const float d0 = o.x - t.x, d1 = o.y - t.y;
+    const float d0 = o.x - target[2 * (size_t)p], d1 = o.y - target[2 * (size_t)p + 1];
     float g[8] = {2.f * d0 * inv, 2.f * d1 * inv, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     d4[2 * (size_t)p] = f_to_bf8(g);
     d4[2 * (size_t)p + 1] = make_uint4(0u, 0u, 0u, 0u);
