@@ -204,15 +204,16 @@ __global__ void __launch_bounds__(256, SPLIT == 8 ? 3 : 4) k_gather(const Update
   const int Y0 = tile / u.tiles_x * kObjTile + unit % BANDS * (kObjTile / BANDS);
   const int pu = (MM + VALUES - 1) / VALUES, k = obj ? 0 : (unit - units_o) / pu;  // k == K: D_P
   const int P0 = obj ? 0 : (unit - units_o) % pu * VALUES;
-  // output of value t of the unit (object: row-major in the tile part), -1: outside
-  auto output = [&](int t) {
+  // output of value t of the unit (object: row-major in the tile part; 64 bits, an object may hold 2^31 pixels
+  // and more), -1: outside
+  auto output = [&](int t) -> long long {
     if (!obj) return P0 + t < MM ? P0 + t : -1;
     const int X = X0 + t % kObjTile, Y = Y0 + t / kObjTile;
-    return X < u.obj_w && Y < u.obj_h ? Y * u.obj_w + X : -1;
+    return X < u.obj_w && Y < u.obj_h ? (long long)Y * u.obj_w + X : -1;
   };
   float m = 0.f;
   auto store = [&](int t, float2 a, float d) {
-    const int at = output(t);
+    const long long at = output(t);
     if (at < 0) return;
     if (obj) {
       u.no_part[at] = a;
