@@ -255,12 +255,19 @@ __global__ void __launch_bounds__(kModTpb<BL>) k_big_modulus(const BigArgs b) {
   // blur along y (rows, sigma_2) for the own rows, ratio, error
   const float eps = b.eps;
   float es = 0.f, ec = 0.f;
+  // the ratio takes sqrt(I), the error the counts I as they were given (their rounded roots squared are off by
+  // more than an ulp); pc-DM: each sweep needs one of the two
   const float* Sn = b.sqrtI + (size_t)n * MM;
+  const float* In = b.I + (size_t)n * MM;
+  const bool ratio = b.dm_pass != 1, error = b.dm_pass != 2;
   for (int w = threadIdx.x; w < BL * (RB / NB); w += TPB) {
     const int x = w % BL, rs = (w / BL) * NB;
-    float sq[NB], out[NB];
+    float sq[NB], im[NB], out[NB];
 #pragma unroll
-    for (int o = 0; o < NB; ++o) sq[o] = __ldcs(&Sn[(size_t)(y0 + rs + o) * BL + x]);
+    for (int o = 0; o < NB; ++o) {
+      sq[o] = ratio ? __ldcs(&Sn[(size_t)(y0 + rs + o) * BL + x]) : 0.f;
+      im[o] = error ? __ldcs(&In[(size_t)(y0 + rs + o) * BL + x]) : 0.f;
+    }
     blur_strip<NB, KH>(sB, x, LD, rs + KH, 0, HR, s_gy, b.kh, out);
 #pragma unroll
     for (int o = 0; o < NB; ++o) {
@@ -273,15 +280,15 @@ __global__ void __launch_bounds__(kModTpb<BL>) k_big_modulus(const BigArgs b) {
         ihat = acc * acc;
         R = __fdividef(sq[o], acc + eps);
       }
-      const float dd = ihat - sq[o] * sq[o];
+      const float dd = ihat - im[o];
       const float yv = fmaf(dd, dd, -ec);
       const float tt = es + yv;
       ec = (tt - es) - yv;
       es = tt;
-      if (b.dm_pass != 1) b.R[(size_t)c * MM + (size_t)(y0 + rs + o) * BL + x] = R;  // pc-DM: R of chi only
+      if (ratio) b.R[(size_t)c * MM + (size_t)(y0 + rs + o) * BL + x] = R;
     }
   }
-  if (b.dm_pass == 2) return;  // pc-DM: the error is the estimate's (first sweep); uniform per block
+  if (!error) return;  // pc-DM: the error is the estimate's (first sweep); uniform per block
   s_red[threadIdx.x] = (double)es - (double)ec;
   __syncthreads();
   for (int w = TPB / 2; w > 0; w >>= 1) {

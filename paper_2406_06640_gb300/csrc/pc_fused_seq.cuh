@@ -13,7 +13,7 @@
 //   A^G     = sqrt(S) (x) g   (Eq. 6)  or  I_m = S (x) g  (Eq. 2), g of Eq. 7 normalised,
 //             separable, zero padded
 //   R       = sqrt(I_n) / (A^G + eps)  or  sqrt(I_n) / sqrt(I_m + eps^2)     (Fig. 1 box 1)
-//   error  += sum (Ihat - I_n)^2 with I_n = (sqrt I_n)^2, Ihat = (A^G)^2 or I_m
+//   error  += sum (Ihat - I_n)^2 with Ihat = (A^G)^2 or I_m; SINGLE: I_n = (sqrt I_n)^2, of one read
 //   pass 2, k = K-1, 0, 1, .. K-2 (mode K-1 from TMEM, the others propagated again):
 //     Psi'_k = R Psi_k;  psi'_k = inverse propagation;  dpsi_k = psi'_k - P_k o_n
 //     c_n   += conj(P_k) dpsi_k                 (TMEM; written once per position)
@@ -190,8 +190,10 @@ __global__ void __launch_bounds__(SeqShape<M>::TR, SeqShape<M>::MIN_BLOCKS) pc_s
     const int2 pn = a.pos[n];
     const float2* On = a.O + (size_t)pn.x * a.obj_w + pn.y;
     const float* Qn = a.sqrtI + (size_t)n * M * M;
-    // sqrt(I_n) is read once, by the modulus step: start moving it into L2 now
+    const float* In = a.I + (size_t)n * M * M;  // QUEUED, DM: the counts themselves, for the error
+    // sqrt(I_n) is read once, by the modulus step (and I_n, by the error): start moving it into L2 now
     if (tid == 0) prefetch_l2(Qn, (uint32_t)(M * M * 4), stream);
+    if (MODE != SINGLE && tid == 0) prefetch_l2(In, (uint32_t)(M * M * 4), stream);
     float2 v[V][E];
 
     // ---- the object box in ROW layout into TMEM (every load in flight at once)
@@ -344,16 +346,22 @@ __global__ void __launch_bounds__(SeqShape<M>::TR, SeqShape<M>::MIN_BLOCKS) pc_s
       __syncthreads();
       for (int w = tid; w < M * (M / NB); w += TR) {
         const int col = w % M, rs = (w / M) * NB;
-        float sq[NB];
+        constexpr bool ROOT = MODE == SINGLE || (PS & 2) != 0, COUNTS = MODE != SINGLE && (PS & 1) != 0;
+        float sq[NB], in[NB];
 #pragma unroll
-        for (int o = 0; o < NB; ++o) sq[o] = __ldcs(&Qn[(rs + o) * M + col]);
+        for (int o = 0; o < NB; ++o) {
+          if constexpr (ROOT) sq[o] = __ldcs(&Qn[(rs + o) * M + col]);
+          if constexpr (COUNTS) in[o] = __ldcs(&In[(rs + o) * M + col]);
+        }
         float out[NB];
         blur_strip<NB, KH>(X, col, LD, rs, 0, M, s_gy, a.kh, out);
 #pragma unroll
         for (int o = 0; o < NB; ++o) {
           const float acc = out[o];
           if constexpr ((PS & 1) != 0) {
-            const float im = sq[o] * sq[o];
+            float im;
+            if constexpr (COUNTS) im = in[o];
+            else im = sq[o] * sq[o];
             const float ihat = a.blur_intensity ? acc : acc * acc;
             const float d = ihat - im;
             const float y = fmaf(d, d, -err_c);
