@@ -106,6 +106,21 @@ static std::vector<int> philox_permutation(int n, uint64_t seed, uint32_t stream
 // M = 128 while their partials (32 K M^2 complex) stay small beside the state they are summed from
 constexpr int kDmParts = 32;
 
+// Whether n positions run faster as clusters of K CTAs than with one CTA each: waves of a launch times the cost
+// of a position, about (K + 1/2) mode passes one after the other against a cluster's fixed cost in the same
+// unit. The smaller the tile, the more of that are barriers: 2.2 at 128^2, 2.7, 3.8, 4.4, 6 at 8^2. Iterations
+// of the difference map, clusters against CTAs, far field:
+//   128^2, 8 modes: 8 positions 83 / 271 us, 48 (3 waves of clusters) 295 / 323, 76 (4) 421 / 344
+//   128^2, 4 modes: 32 positions 89 / 160, 60 (2) 155 / 181, 76 (3) 232 / 190;  2 modes: 76 positions 101 / 106
+//   64^2, 4 modes: 32 positions 54 / 73, 48 (2) 77 / 76;  32^2, 8 modes: 76 (2) 82 / 84, 152 (3) 112 / 89
+//   16^2, 4 modes: 76 positions 49 / 52;  8^2, 6 modes: 8 positions 35 / 36, 200 (2) 61 / 52
+static bool cluster_form(int M, int K, int n, int cluster_slots, int slots) {
+  if (K < 2 || cluster_slots < 1) return false;
+  const double cost = M >= 128 ? 2.2 : M >= 64 ? 2.7 : M >= 32 ? 3.8 : M >= 16 ? 4.4 : 6.0;
+  const int waves = (n + cluster_slots - 1) / cluster_slots, one = (n + slots - 1) / slots;
+  return waves * cost < one * (K + 0.5);
+}
+
 struct ptycho_plan_s {
   ptycho_params p{};
   std::vector<int32_t> windows;
@@ -116,6 +131,7 @@ struct ptycho_plan_s {
   double errden = 0.0, eps = 0.0;
   int slots = 0;
   int cluster_slots = 0;  // mini-batch plans: co-resident clusters of the cluster form (small batches)
+  bool dm_clusters = false;  // pc-DM: the cluster form, `slots` clusters
   long long iter = 1;  // number of the next iteration
   long long runs = 0;  // iterations run so far
   FusedArgs fa{};
@@ -437,7 +453,7 @@ static ptycho_status build_plan(ptycho_plan_s* pl, const float* intensities, con
     pl->h_pos = perm;
   }
 
-  // ---- slots: co-resident clusters of the fused kernel (M <= 128), or the position chunk of
+  // ---- slots: co-resident CTAs (or clusters) of the fused kernel (M <= 128), or the position chunk of
   // the staged path (M = 256, 512), whose per-slot partials are summed in slot order
   pl->big = M > 128;
   if (pl->big) {
@@ -448,6 +464,10 @@ static ptycho_status build_plan(ptycho_plan_s* pl, const float* intensities, con
     if (p.engine == PTYCHO_ENGINE_DM) {
       PT_CUDA(fused_dm_max_slots(M, K, &max_slots), "occupancy of the pc-DM kernel");
       if (max_slots < 1) return fail(PTYCHO_EUNSUPPORTED, "the pc-DM kernel does not fit on this device");
+      int clusters = 0;
+      PT_CUDA(fused_dm_cluster_max_slots(M, K, &clusters), "occupancy of the pc-DM cluster form");
+      pl->dm_clusters = cluster_form(M, K, N, clusters, max_slots);
+      if (pl->dm_clusters) max_slots = clusters;
     } else {
       PT_CUDA(fused_max_slots(M, K, &max_slots), "occupancy of the fused kernel");
       if (max_slots < 1) return fail(PTYCHO_EUNSUPPORTED, "the fused kernel does not fit on this device");
@@ -913,7 +933,8 @@ static ptycho_status enqueue_iteration(ptycho_plan_s* pl, void* object, void* pr
   } else if (pl->d_psi) {
     fa.psi = pl->d_psi;
     fa.dm_init = pl->dm_fresh ? 1 : 0;
-    PT_CUDA(launch_fused_dm(pl->p.M, fa, pl->slots, s), "pc-DM kernel launch");
+    if (pl->dm_clusters) PT_CUDA(launch_fused_dm_cluster(pl->p.M, fa, pl->slots, s), "pc-DM kernel launch");
+    else PT_CUDA(launch_fused_dm(pl->p.M, fa, pl->slots, s), "pc-DM kernel launch");
     pl->dm_fresh = false;
   } else {
     PT_CUDA(launch_fused(pl->p.M, fa, pl->slots, s), "fused kernel launch");

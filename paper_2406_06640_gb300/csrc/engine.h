@@ -70,9 +70,11 @@ cudaError_t fused_cluster_max_slots(int M, int K, int* slots);
 cudaError_t launch_fused_queue(int M, const FusedArgs& a, int slots, cudaStream_t s);
 cudaError_t fused_queue_max_slots(int M, int K, int* slots);
 // pc-DM launch (single problem, M <= 128): as launch_fused with the exit-wave state a.psi and no probe
-// partials
+// partials; and as launch_fused_cluster
 cudaError_t launch_fused_dm(int M, const FusedArgs& a, int slots, cudaStream_t s);
 cudaError_t fused_dm_max_slots(int M, int K, int* slots);
+cudaError_t launch_fused_dm_cluster(int M, const FusedArgs& a, int slots, cudaStream_t s);
+cudaError_t fused_dm_cluster_max_slots(int M, int K, int* slots);
 bool fused_queue_supported(int M);
 size_t fused_smem_bytes(int M);
 // one bounded mbarrier wait of the fused kernels' kind on a barrier that `signal` completes (or

@@ -101,6 +101,10 @@ __device__ __forceinline__ void probe_map(const FusedArgs& a, int threads) {
   }
 }
 
+// what a fused launch runs: SINGLE one problem; QUEUED the chunks of several problems of one shape, taken from a
+// device counter, each chunk with its own partials; DM the difference map on one problem
+enum FusedMode { SINGLE = 0, QUEUED = 1, DM = 2 };
+
 template <int X>
 struct IntC {
   static constexpr int value = X;

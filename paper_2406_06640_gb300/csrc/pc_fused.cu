@@ -1,6 +1,6 @@
-// Fused per-position pc-engine kernel in its cluster form, used by mini-batches too small to fill the
-// GPU with one CTA per position (every other launch runs the one-CTA-per-position kernel of
-// pc_fused_seq.cuh): one cluster of K CTAs per scan position,
+// Fused per-position pc-engine kernel in its cluster form, used by mini-batches and difference-map scans too
+// small to fill the GPU with one CTA per position (every other launch runs the one-CTA-per-position kernel
+// of pc_fused_seq.cuh): one cluster of K CTAs per scan position,
 // CTA rank k owns probe mode k and rows [k R, (k + 1) R) of the detector
 // (R = ceil(M / K)). Everything between the object gather and the per-position
 // contributions stays on chip:
@@ -61,75 +61,9 @@ size_t fused_smem_bytes(int M) {
   }
 }
 
-template <int M, int KH>
-static cudaLaunchConfig_t fused_config(const FusedArgs& a, int slots, cudaStream_t s, cudaLaunchAttribute* attr) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(slots * a.K));
-  cfg.blockDim = dim3(FusedShape<M>::TR);
-  cfg.dynamicSmemBytes = FusedSmem<M, KH>::BYTES;
-  cfg.stream = s;
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)a.K;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cfg;
-}
-
-template <int M, bool NEAR, int KH>
-static cudaError_t launch_kh(const FusedArgs& a, int slots, cudaStream_t s) {
-  auto kern = pc_fused_kernel<M, NEAR, KH>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FusedSmem<M, KH>::BYTES);
-  if (e != cudaSuccess) return e;
-  cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = fused_config<M, KH>(a, slots, s, attr);
-  return cudaLaunchKernelEx(&cfg, kern, a);
-}
-
-// ---- single-problem launches of the cluster form: the mini-batch engine takes them for batches
-// with fewer positions than the one-CTA form has slots (K CTAs per position then fill more SMs)
-template <int M, bool NEAR>
-static cudaError_t launch_cluster_t(const FusedArgs& a, int slots, cudaStream_t s) {
-  return a.kh == 5 ? launch_kh<M, NEAR, 5>(a, slots, s) : launch_kh<M, NEAR, 15>(a, slots, s);
-}
-
 cudaError_t launch_fused_cluster(int M, const FusedArgs& a, int slots, cudaStream_t s) {
-  const bool nf = a.near_field != 0;
-  switch (M) {
-    case 8: return nf ? launch_cluster_t<8, true>(a, slots, s) : launch_cluster_t<8, false>(a, slots, s);
-    case 16: return nf ? launch_cluster_t<16, true>(a, slots, s) : launch_cluster_t<16, false>(a, slots, s);
-    case 32: return nf ? launch_cluster_t<32, true>(a, slots, s) : launch_cluster_t<32, false>(a, slots, s);
-    case 64: return nf ? launch_cluster_t<64, true>(a, slots, s) : launch_cluster_t<64, false>(a, slots, s);
-    case 128: return nf ? launch_cluster_t<128, true>(a, slots, s) : launch_cluster_t<128, false>(a, slots, s);
-    default: return cudaErrorInvalidValue;
-  }
+  return launch_cluster<SINGLE>(M, a, slots, s);
 }
-
-template <int M>
-static cudaError_t cluster_slots_t(int K, int* slots) {
-  auto kern = pc_fused_kernel<M, false, 15>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FusedSmem<M, 15>::BYTES);
-  if (e != cudaSuccess) return e;
-  FusedArgs a = {};
-  a.K = K;
-  cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = fused_config<M, 15>(a, 1, 0, attr);
-  int n = 0;
-  e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
-  *slots = n;
-  return e;
-}
-
-cudaError_t fused_cluster_max_slots(int M, int K, int* slots) {
-  switch (M) {
-    case 8: return cluster_slots_t<8>(K, slots);
-    case 16: return cluster_slots_t<16>(K, slots);
-    case 32: return cluster_slots_t<32>(K, slots);
-    case 64: return cluster_slots_t<64>(K, slots);
-    case 128: return cluster_slots_t<128>(K, slots);
-    default: return cudaErrorInvalidValue;
-  }
-}
+cudaError_t fused_cluster_max_slots(int M, int K, int* slots) { return cluster_slots<SINGLE>(M, K, slots); }
 
 }  // namespace ptycho

@@ -5,7 +5,8 @@
 // global memory). The overlap projection alternates: the object step of the single-problem path with
 // dpsi = psi_n - P o_n, then (update.cu) the probe step from the new object and the state.
 // Bound like the other modes by the transforms (4K - 1 per position against the cluster form's 3K plus
-// eight cluster barriers): 900 positions of 128^2, four modes, 1.92 -> 1.33 ms an iteration.
+// eight cluster barriers): 900 positions of 128^2, four modes, 1.66 ms an iteration as clusters, 1.28 here.
+// Few positions run as clusters (pc_fused_dm_cluster.cu; cluster_form in capi.cu).
 #include "pc_fused_seq.cuh"
 
 namespace ptycho {

@@ -89,7 +89,8 @@ struct FusedShape {
                 "TMEM allocation must be a power of two in [32, 512] columns");
 };
 
-template <int M, bool NEAR, int KH>
+// MODE: SINGLE one problem (a mini-batch); DM the difference map on one problem (pc_fused_seq.cuh describes both)
+template <int M, bool NEAR, int KH, int MODE>
 __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const FusedArgs a_in) {
   using TL = Tile<M>;
   using SM = FusedSmem<M, KH>;
@@ -197,6 +198,9 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
   auto run_position = [&](const FusedArgs& a, int n, bool first, float2* pacc, float* dacc) {
     const float2* Pk = a.P + (size_t)rank * M * M;
     const float eps = a.eps;
+    // pc-DM: this position's exit-wave state of mode `rank` (P o_n itself when the state starts)
+    float2* Sn = MODE == DM ? a.psi + ((size_t)n * K + rank) * M * M : nullptr;
+    const bool dm_init = MODE == DM && a.dm_init;
     const int2 pn = a.pos[n];
     const float2* On = a.O + (size_t)pn.x * a.obj_w + pn.y;
     float2 v[V][E];
@@ -225,8 +229,10 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
       if constexpr (NEAR) det_coords<M, true>(tid + q * TR, r, row, col);
       else freq(q, r, row, col);
     };
-    // ---- exit wave P o_n in ROW layout; far field: times (-1)^(y + x), which centres the transform
-    auto exit_wave = [&]() {
+    // ---- exit wave in ROW layout: P o_n, or (pc-DM, CHI) the reflected wave 2 P o_n - psi_n;
+    // far field: times (-1)^(y + x), which centres the transform
+    auto exit_wave = [&](auto chi_c) {
+      constexpr bool CHI = decltype(chi_c)::value != 0;
       if constexpr (TM) {
         // every object load of this thread in flight at once (the TMEM waits below are compiler
         // barriers: loads issued after them would expose one L2 round trip per group)
@@ -245,6 +251,10 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
             for (int jj = 0; jj < 4; ++jj) {
               const int x = tp[q] + G * (4 * h + jj);
               float2 psi = cmul(make_float2(pr[2 * jj], pr[2 * jj + 1]), v[q][4 * h + jj]);
+              if constexpr (CHI) {
+                const float2 st = dm_init ? psi : Sn[line[q] * M + x];
+                psi = make_float2(2.f * psi.x - st.x, 2.f * psi.y - st.y);
+              }
               if (!NEAR && ((line[q] + x) & 1)) psi = make_float2(-psi.x, -psi.y);
               v[q][4 * h + jj] = psi;
             }
@@ -256,16 +266,21 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
           for (int j = 0; j < E; ++j) {
             const int x = tp[q] + G * j;
             float2 psi = cmul(Pk[line[q] * M + x], On[(size_t)line[q] * a.obj_w + x]);
+            if constexpr (CHI) {
+              const float2 st = dm_init ? psi : Sn[line[q] * M + x];
+              psi = make_float2(2.f * psi.x - st.x, 2.f * psi.y - st.y);
+            }
             if (!NEAR && ((line[q] + x) & 1)) psi = make_float2(-psi.x, -psi.y);
             v[q][j] = psi;
           }
       }
     };
 
-    // ---- propagation to the detector and the pc intensity model of Fig. 1 box 1 on the own rows: the
-    // error of the model intensity, and the modulus ratio R pushed to every rank (Z holds R for the
-    // whole tile)
-    auto detector = [&]() {
+    // ---- propagation to the detector and the pc intensity model of Fig. 1 box 1 on the own rows.
+    // PS bit 0: accumulate the error of the model intensity; bit 1: push the modulus ratio R to
+    // every rank (then Z holds R for the whole tile)
+    auto detector = [&](auto ps_c) {
+      constexpr int PS = decltype(ps_c)::value;
       // ---- forward propagation
       transform(IntC<0>{});
       if constexpr (NEAR) {
@@ -362,7 +377,7 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
             if (lr >= nrow) break;
             const int gr = r0 + lr;
             const float acc = out[o];
-            {
+            if constexpr ((PS & 1) != 0) {
               const float im = pre ? s_meas[(nrow + lr) * M + col] : In[gr * M + col];
               const float ihat = a.blur_intensity ? acc : acc * acc;
               const float d = ihat - im;
@@ -371,7 +386,7 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
               err_c = (tt - err_s) - y;
               err_s = tt;
             }
-            {
+            if constexpr ((PS & 2) != 0) {
               const float sq = pre ? s_meas[lr * M + col] : Qn[gr * M + col];
               const float R = a.blur_intensity ? sq * rsqrtf(acc + eps * eps) : __fdividef(sq, acc + eps);
               const uint32_t zoff = z_s + (uint32_t)((gr * LD + col) * 4);
@@ -380,11 +395,20 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
           }
         }
       }
-      cluster_sync_all();  // R arrives from every rank
+      // R arrives from every rank; without R only this CTA's shared memory was read
+      if constexpr ((PS & 2) != 0) cluster_sync_all();
+      else __syncthreads();
     };
 
-    exit_wave();
-    detector();
+    if constexpr (MODE == DM) {
+      exit_wave(IntC<0>{});  // the estimate P o_n: its model error is E
+      detector(IntC<1>{});
+      exit_wave(IntC<1>{});  // the reflected wave: its modulus ratio
+      detector(IntC<2>{});
+    } else {
+      exit_wave(IntC<0>{});
+      detector(IntC<3>{});
+    }
     // ---- (5) Psi' = R Psi
 #pragma unroll
     for (int q = 0; q < V; ++q)
@@ -425,7 +449,7 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
         for (int h = 0; h < E / 4; ++h) {
           float pr[8], ac[8];
           tmem_ld8(t_lane + colP + 2 * (q * E + 4 * h), pr);
-          if (!first) tmem_ld8(t_lane + colA + 2 * (q * E + 4 * h), ac);
+          if (MODE != DM && !first) tmem_ld8(t_lane + colA + 2 * (q * E + 4 * h), ac);
           tmem_wait_ld();
 #pragma unroll
           for (int jj = 0; jj < 4; ++jj) {
@@ -434,9 +458,15 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
             float2 psi_new = cscale(v[q][j], inv_m2);
             if (!NEAR && ((ln + x) & 1)) psi_new = make_float2(-psi_new.x, -psi_new.y);
             const float2 p = make_float2(pr[2 * jj], pr[2 * jj + 1]);
-            const float2 dpsi = csub(psi_new, cmul(p, o[j]));
+            const float2 ov = cmul(p, o[j]);
+            float2 dpsi = csub(psi_new, ov);
+            if constexpr (MODE == DM) {  // psi_n <- psi_n + Pi_F(chi) - P o_n; the overlap step takes psi_n - P o_n
+              const float2 st = cadd(dm_init ? ov : Sn[ln * M + x], dpsi);
+              Sn[ln * M + x] = st;
+              dpsi = csub(st, ov);
+            }
             st_cluster_f2(dst + 8u * x, cconjmul(p, dpsi));
-            {
+            if constexpr (MODE != DM) {  // pc-DM takes its probe step after the object step, from its state
               const float2 pc = cconjmul(o[j], dpsi);
               ac[2 * jj] = first ? pc.x : ac[2 * jj] + pc.x;
               ac[2 * jj + 1] = first ? pc.y : ac[2 * jj + 1] + pc.y;
@@ -446,9 +476,9 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
               }
             }
           }
-          tmem_st8(t_lane + colA + 2 * (q * E + 4 * h), ac);
+          if constexpr (MODE != DM) tmem_st8(t_lane + colA + 2 * (q * E + 4 * h), ac);
         }
-        tmem_wait_st();
+        if constexpr (MODE != DM) tmem_wait_st();
       } else {
 #pragma unroll
         for (int j = 0; j < E; ++j) {
@@ -457,9 +487,15 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
           if (!NEAR && ((ln + x) & 1)) psi_new = make_float2(-psi_new.x, -psi_new.y);
           const float2 p = Pk[ln * M + x];
           const float2 o = On[(size_t)ln * a.obj_w + x];
-          const float2 dpsi = csub(psi_new, cmul(p, o));
+          const float2 ov = cmul(p, o);
+          float2 dpsi = csub(psi_new, ov);
+          if constexpr (MODE == DM) {  // psi_n <- psi_n + Pi_F(chi) - P o_n; the overlap step takes psi_n - P o_n
+            const float2 st = cadd(dm_init ? ov : Sn[ln * M + x], dpsi);
+            Sn[ln * M + x] = st;
+            dpsi = csub(st, ov);
+          }
           st_cluster_f2(dst + 8u * x, cconjmul(p, dpsi));
-          {
+          if constexpr (MODE != DM) {
             const int qi = ln * M + x;
             const float2 pc = cconjmul(o, dpsi);
             if (first) pacc[qi] = pc;
@@ -489,7 +525,7 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
   // ---- end of a unit: probe-numerator partial from TMEM to global; per-CTA FP64 error
   // numerator (the compensated FP32 thread sums, added in thread order) into partial `part`
   auto finish_unit = [&](const FusedArgs& a, float2* pacc, int part) {
-    if constexpr (TM) {
+    if constexpr (TM && MODE != DM) {
 #pragma unroll
       for (int q = 0; q < V; ++q)
 #pragma unroll
@@ -518,8 +554,8 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
   // cluster `slot` takes positions slot, slot + slots, ... and owns partial `slot`
   setup_unit(a_in);
   __syncthreads();
-  float2* pacc = a_in.pacc + ((size_t)slot * K + rank) * M * M;
-  float* dacc = a_in.dacc + (size_t)slot * M * M;
+  float2* pacc = MODE == DM ? nullptr : a_in.pacc + ((size_t)slot * K + rank) * M * M;
+  float* dacc = MODE == DM ? nullptr : a_in.dacc + (size_t)slot * M * M;
   for (int n = slot; n < a_in.N; n += nslots) run_position(a_in, n, n == slot, pacc, dacc);
   finish_unit(a_in, pacc, slot);
   if constexpr (TM) {
@@ -527,6 +563,82 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
     __syncthreads();
     tmem_fence_after();
     if (tid / 32 == 0) tmem_dealloc(*s_tmem, FusedShape<M>::TMEM_COLS);
+  }
+}
+
+// ------------------------------------------------------------------ launches
+template <int M, int KH>
+static cudaLaunchConfig_t fused_config(const FusedArgs& a, int slots, cudaStream_t s, cudaLaunchAttribute* attr) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(slots * a.K));
+  cfg.blockDim = dim3(FusedShape<M>::TR);
+  cfg.dynamicSmemBytes = FusedSmem<M, KH>::BYTES;
+  cfg.stream = s;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)a.K;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+template <int M, bool NEAR, int KH, int MODE>
+static cudaError_t launch_cluster_kh(const FusedArgs& a, int slots, cudaStream_t s) {
+  auto kern = pc_fused_kernel<M, NEAR, KH, MODE>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FusedSmem<M, KH>::BYTES);
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute attr[1];
+  cudaLaunchConfig_t cfg = fused_config<M, KH>(a, slots, s, attr);
+  return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+template <int M, int MODE>
+static cudaError_t launch_cluster_t(const FusedArgs& a, int slots, cudaStream_t s) {
+  if (a.near_field)
+    return a.kh == 5 ? launch_cluster_kh<M, true, 5, MODE>(a, slots, s)
+                     : launch_cluster_kh<M, true, 15, MODE>(a, slots, s);
+  return a.kh == 5 ? launch_cluster_kh<M, false, 5, MODE>(a, slots, s)
+                   : launch_cluster_kh<M, false, 15, MODE>(a, slots, s);
+}
+
+template <int MODE>
+static cudaError_t launch_cluster(int M, const FusedArgs& a, int slots, cudaStream_t s) {
+  switch (M) {
+    case 8: return launch_cluster_t<8, MODE>(a, slots, s);
+    case 16: return launch_cluster_t<16, MODE>(a, slots, s);
+    case 32: return launch_cluster_t<32, MODE>(a, slots, s);
+    case 64: return launch_cluster_t<64, MODE>(a, slots, s);
+    case 128: return launch_cluster_t<128, MODE>(a, slots, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+// co-resident clusters of K CTAs, taken for the largest shared-memory variant
+template <int M, int MODE>
+static cudaError_t cluster_slots_t(int K, int* slots) {
+  auto kern = pc_fused_kernel<M, false, 15, MODE>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FusedSmem<M, 15>::BYTES);
+  if (e != cudaSuccess) return e;
+  FusedArgs a = {};
+  a.K = K;
+  cudaLaunchAttribute attr[1];
+  cudaLaunchConfig_t cfg = fused_config<M, 15>(a, 1, 0, attr);
+  int n = 0;
+  e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+  *slots = n;
+  return e;
+}
+
+template <int MODE>
+static cudaError_t cluster_slots(int M, int K, int* slots) {
+  switch (M) {
+    case 8: return cluster_slots_t<8, MODE>(K, slots);
+    case 16: return cluster_slots_t<16, MODE>(K, slots);
+    case 32: return cluster_slots_t<32, MODE>(K, slots);
+    case 64: return cluster_slots_t<64, MODE>(K, slots);
+    case 128: return cluster_slots_t<128, MODE>(K, slots);
+    default: return cudaErrorInvalidValue;
   }
 }
 

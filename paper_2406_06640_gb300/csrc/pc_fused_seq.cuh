@@ -111,10 +111,6 @@ struct SeqSmem {
   static_assert((size_t)SeqShape<M>::TR * 8 <= CBUF, "error reduction buffer");
 };
 
-// MODE: SINGLE runs one problem; QUEUED drains the chunks of several problems of one shape from a device
-// counter, each chunk with its own partials; DM runs the difference map on one problem
-enum SeqMode { SINGLE = 0, QUEUED = 1, DM = 2 };
-
 template <int M, bool NEAR, int KH, int MODE>
 __global__ void __launch_bounds__(SeqShape<M>::TR, SeqShape<M>::MIN_BLOCKS) pc_seq_kernel(const FusedArgs a_in) {
   using TL = Tile<M>;
