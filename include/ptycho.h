@@ -183,13 +183,13 @@ ptycho_status ptycho_error_batch(ptycho_plan_t plan, double* nrmse_last);
 
 /* Work-queue batching: problems with M in {8, 16, 32, 64, 128} sharing K, geometry and
  * kernel width class (11 x 11 or any other size) are drained by one persistent
- * launch per class. Each chunk of L consecutive positions is one work item, or, in a class
- * with fewer chunks than the GPU has CTA slots, up to eight items of consecutive positions;
- * every item keeps its own probe and error partials, summed in position order (results do not
- * depend on which CTA took an item). L is chosen per class by an autotuner the first time a batch
- * plan of that class is built on a device in the process: it times the class's
- * launch for L = 8, 16, 32, 64 on the device and keeps the fastest (cached per
- * device, M, K, geometry and kernel width class).
+ * launch per class. A chunk of L consecutive positions is one work item, or, where that would leave
+ * CTA slots of the GPU idle, a power of two of items of consecutive positions; every item keeps its own
+ * probe and error partials, summed in position order (results do not depend on which CTA took an
+ * item). A class of few positions and several modes runs a cluster of K CTAs per position instead.
+ * L is chosen by an autotuner where it matters (chunks of 8 fill the GPU): it times the class's
+ * launch for L = 8, 16, 32, 64 on the device and keeps the fastest for the process (cached per
+ * device, M, K, geometry, kernel width class and powers of two of positions per CTA slot).
  * ptycho_set_batch_chunk fixes L for every later ptycho_plan_batch (8, 16, 32 or
  * 64; 0 restores tuning), e.g. for bitwise-reproducible runs across processes:
  * different L give the same result up to the FP32 order of the partial sums. */
@@ -209,6 +209,9 @@ int32_t ptycho_staged_chunk(ptycho_plan_t plan);
  * members, chunk length, chunks, co-resident groups of CTAs that serve a chunk) into out; *count = the
  * number of classes. */
 ptycho_status ptycho_batch_classes(ptycho_plan_t plan, int32_t max_classes, int32_t* out, int32_t* count);
+/* The work items of those classes: for each, 4 int32 (positions per item, items, CTAs per item: 1, or K in
+ * the cluster form, and CTAs launched) into out; *count as above. */
+ptycho_status ptycho_batch_items(ptycho_plan_t plan, int32_t max_classes, int32_t* out, int32_t* count);
 
 /* Kernel launches of one iteration of a batch plan: the kernel nodes of the CUDA graph that the last
  * ptycho_iterate_batch replayed per iteration (0 before the first call). kernels: host. EINVAL if

@@ -24,7 +24,8 @@ ENGINE_PIE, ENGINE_DM = 0, 1
 EXPORTED = ("ptycho_plan", "ptycho_iterate", "ptycho_error", "ptycho_error_history", "ptycho_destroy",
             "ptycho_plan_batch", "ptycho_iterate_batch", "ptycho_error_batch",
             "ptycho_profile", "ptycho_profile_read", "ptycho_launches_per_iteration", "ptycho_last_error",
-            "ptycho_version", "ptycho_set_batch_chunk", "ptycho_batch_classes", "ptycho_batch_launches", "ptycho_set_staged_chunk", "ptycho_staged_chunk", "ptycho_permutation", "ptycho_unet_create", "ptycho_unet_param_count", "ptycho_unet_set_params",
+            "ptycho_version", "ptycho_set_batch_chunk", "ptycho_batch_classes", "ptycho_batch_items",
+            "ptycho_batch_launches", "ptycho_set_staged_chunk", "ptycho_staged_chunk", "ptycho_permutation", "ptycho_unet_create", "ptycho_unet_param_count", "ptycho_unet_set_params",
             "ptycho_unet_get_params", "ptycho_unet_forward", "ptycho_unet_gradients", "ptycho_unet_train_step",
             "ptycho_unet_destroy", "ptycho_generate", "ptycho_warmstart", "ptycho_monochromatise",
             "ptycho_measure_fp32_peak", "ptycho_wait_selftest")
@@ -128,6 +129,8 @@ def load(build_if_missing: bool = True) -> ctypes.CDLL:
     lib.ptycho_batch_classes.argtypes = [P, ctypes.c_int32, ctypes.POINTER(ctypes.c_int32),
                                          ctypes.POINTER(ctypes.c_int32)]
     lib.ptycho_batch_classes.restype = st
+    lib.ptycho_batch_items.argtypes = lib.ptycho_batch_classes.argtypes
+    lib.ptycho_batch_items.restype = st
     lib.ptycho_batch_launches.argtypes = [P, ctypes.POINTER(ctypes.c_int32)]
     lib.ptycho_batch_launches.restype = st
     lib.ptycho_last_error.argtypes = []
@@ -300,6 +303,15 @@ class BatchPlan:
         _check(load().ptycho_batch_classes(self._h, n.value, buf, ctypes.byref(n)))
         keys = ("M", "K", "near", "kh", "members", "chunk_len", "chunks", "slots")
         return [dict(zip(keys, buf[8 * c:8 * c + 8])) for c in range(n.value)]
+
+    def items(self) -> list:
+        """Work items of those classes: dicts with item_len, items, ctas_per_item, ctas."""
+        n = ctypes.c_int32()
+        _check(load().ptycho_batch_items(self._h, 0, None, ctypes.byref(n)))
+        buf = (ctypes.c_int32 * (4 * max(n.value, 1)))()
+        _check(load().ptycho_batch_items(self._h, n.value, buf, ctypes.byref(n)))
+        keys = ("item_len", "items", "ctas_per_item", "ctas")
+        return [dict(zip(keys, buf[4 * c:4 * c + 4])) for c in range(n.value)]
 
     def launches_per_iteration(self) -> int:
         """Kernel nodes of the graph the last iterate replayed per iteration."""

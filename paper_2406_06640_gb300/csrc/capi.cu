@@ -62,10 +62,10 @@ std::vector<double> taps_1d(double sigma, int h) {
 constexpr int kChunkCandidates[] = {8, 16, 32, 64};
 constexpr int kQueueChunkMin = 8;
 
-// autotuner cache: chunk length per (device, M, K, geometry, kernel width class), and an optional
-// caller-fixed chunk length (0: tune)
+// autotuner cache: chunk length per (device, M, K, geometry, kernel width class, fill: powers of two of positions
+// per CTA slot), and an optional caller-fixed chunk length (0: tune)
 std::mutex g_tune_mutex;
-std::map<std::tuple<int, int, int, int, int>, int> g_tune_cache;
+std::map<std::tuple<int, int, int, int, int, int>, int> g_tune_cache;
 int g_fixed_chunk = 0;
 // staged path (M = 256, 512): positions per chunk of the staged passes, same key, and its fixed value
 constexpr int kStagedCandidates[] = {4, 8, 16, 32};
@@ -165,16 +165,28 @@ struct ptycho_plan_s {
   struct QueueClass {
     int M = 0, K = 0, near = 0, kh = 0;
     std::vector<int> members;  // batch member indices, in order
+    std::vector<int> sizes;  // positions of each member
     int4* d_chunks = nullptr;
     int nchunks = 0;
     int* d_queue = nullptr;
     int slots = 0;
     int chunk_len = 0;
-    // CTAs per chunk: a class with fewer chunks than the GPU has CTA slots splits each of them into this many
-    // items of chunk_len / split positions, each with its own partials (22 chunks of 8 positions of 128^2, two
-    // modes, near field: 741 us on 22 CTAs)
-    int split = 1;
+    bool clusters = false;  // a cluster of K CTAs per work item (cluster_form): items of one position
+    int item_len = 0;       // positions per work item (item_length)
     int nitems = 0;
+    int items(int len) const {
+      int n = 0;
+      for (int N : sizes) n += (N + len - 1) / len;
+      return n;
+    }
+    // Positions per work item for chunk length L: L, halved while that leaves CTA slots without an item. Each item has
+    // its own partials. 22 chunks of 8 positions of 128^2, two modes, near field: 741 us on 22 CTAs; 8 positions
+    // of 128^2, eight modes: 1314 us as one item.
+    int item_length(int L, int max_slots) const {
+      int len = clusters ? 1 : L;
+      while (len > 1 && items(len) < max_slots) len /= 2;
+      return len;
+    }
   };
   std::vector<QueueClass> qclasses;
   std::vector<char> queued;  // per member: drained by its class's work-queue launch
@@ -1107,29 +1119,31 @@ ptycho_status ptycho_iterate(ptycho_plan_t pl, void* object, void* probe, int32_
   return PTYCHO_OK;
 }
 
-// Work items of a class for chunk length L: (member position in the class, first position, end,
-// partial index), members in order, qc.split items per chunk.
-static std::vector<int4> chunk_list(ptycho_plan_s* pl, ptycho_plan_s::QueueClass& qc, int L) {
-  std::vector<int4> chunks;
-  for (size_t j = 0; j < qc.members.size(); ++j) {
-    const ptycho_plan_s* m = pl->members[qc.members[j]];
-    const int len = L / qc.split, parts = (m->p.N + len - 1) / len;
-    for (int c = 0; c < parts; ++c) chunks.push_back(make_int4((int)j, c * len, std::min(m->p.N, (c + 1) * len), c));
-  }
-  return chunks;
+// Work items of a class, `len` positions each: (member position in the class, first position, end, partial
+// index), members in order.
+static std::vector<int4> item_list(const ptycho_plan_s::QueueClass& qc, int len) {
+  std::vector<int4> items;
+  for (size_t j = 0; j < qc.sizes.size(); ++j)
+    for (int c = 0; c * len < qc.sizes[j]; ++c)
+      items.push_back(make_int4((int)j, c * len, std::min(qc.sizes[j], (c + 1) * len), c));
+  return items;
+}
+
+static cudaError_t launch_queue(const ptycho_plan_s::QueueClass& qc, const FusedArgs& fa, int slots, cudaStream_t s) {
+  return qc.clusters ? launch_fused_queue_cluster(qc.M, fa, slots, s) : launch_fused_queue(qc.M, fa, slots, s);
 }
 
 static cudaError_t st_apply_chunk_length(ptycho_plan_s* pl, ptycho_plan_s::QueueClass& qc, int L, int max_slots) {
-  const std::vector<int4> chunks = chunk_list(pl, qc, L);
   qc.chunk_len = L;
-  qc.nitems = (int)chunks.size();
+  qc.nchunks = qc.items(L);
+  qc.item_len = qc.item_length(L, max_slots);
+  const std::vector<int4> items = item_list(qc, qc.item_len);
+  qc.nitems = (int)items.size();
   qc.slots = std::min(max_slots, qc.nitems);
-  qc.nchunks = 0;
-  const cudaError_t e = h2d(pl->stream, qc.d_chunks, chunks.data(), sizeof(int4) * chunks.size());
+  const cudaError_t e = h2d(pl->stream, qc.d_chunks, items.data(), sizeof(int4) * items.size());
   for (int b : qc.members) {
     ptycho_plan_s* m = pl->members[b];
-    qc.nchunks += (m->p.N + L - 1) / L;
-    m->parts = (m->p.N + L / qc.split - 1) / (L / qc.split);
+    m->parts = (m->p.N + qc.item_len - 1) / qc.item_len;
     m->slots = m->parts;
     m->ua.slots = m->parts;
     m->ua.nerr = m->parts * m->p.K;
@@ -1174,7 +1188,7 @@ static ptycho_status tune_chunk_length(ptycho_plan_s* pl, ptycho_plan_s::QueueCl
   *best = kChunkCandidates[0];
   ptycho_status st = PTYCHO_OK;
   for (int L : kChunkCandidates) {
-    const std::vector<int4> chunks = chunk_list(pl, qc, L);
+    const std::vector<int4> chunks = item_list(qc, qc.item_length(L, max_slots));
     cudaError_t ce = h2d(pl->stream, qc.d_chunks, chunks.data(), sizeof(int4) * chunks.size());
     FusedArgs fa = pl->members[qc.members[0]]->fa;
     fa.probs = d_desc;
@@ -1187,7 +1201,7 @@ static ptycho_status tune_chunk_length(ptycho_plan_s* pl, ptycho_plan_s::QueueCl
     for (int r = 0; r < 4 && ce == cudaSuccess; ++r) {
       ce = cudaMemsetAsync(qc.d_queue, 0, sizeof(int), s);
       if (ce == cudaSuccess) ce = cudaEventRecord(e0, s);
-      if (ce == cudaSuccess) ce = launch_fused_queue(qc.M, fa, slots, s);
+      if (ce == cudaSuccess) ce = launch_queue(qc, fa, slots, s);
       if (ce == cudaSuccess) ce = cudaEventRecord(e1, s);
       if (ce == cudaSuccess) ce = cudaEventSynchronize(e1);
       float ms = 0.f;
@@ -1252,22 +1266,25 @@ ptycho_status ptycho_plan_batch(int32_t B, const ptycho_params* const* params, c
       qc.K = q.K;
       qc.near = near;
       qc.kh = kh;
-      qc.chunk_len = kQueueChunkMin;
       pl->qclasses.push_back(qc);
       ci = (int)pl->qclasses.size() - 1;
     }
     pl->qclasses[ci].members.push_back(b);
+    pl->qclasses[ci].sizes.push_back(q.N);
     member_class[b] = ci;
   }
+  std::vector<int> class_slots;  // co-resident CTAs or clusters of each class's launch
   for (auto& qc : pl->qclasses) {
-    int max_slots = 0, chunks = 0;
-    const cudaError_t oe = fused_queue_max_slots(qc.M, qc.K, &max_slots);
-    if (oe != cudaSuccess) {
+    int ctas = 0, clusters = 0;
+    cudaError_t oe = fused_queue_max_slots(qc.M, qc.K, &ctas);
+    if (oe == cudaSuccess && qc.K > 1) oe = fused_queue_cluster_max_slots(qc.M, qc.K, &clusters);
+    if (oe != cudaSuccess || ctas < 1) {
       delete pl;
-      return cuda_fail(oe, "occupancy of the work-queue kernel");
+      return oe != cudaSuccess ? cuda_fail(oe, "occupancy of the work-queue kernel")
+                               : fail(PTYCHO_EUNSUPPORTED, "the work-queue kernel does not fit on this device");
     }
-    for (int b : qc.members) chunks += (params[b]->N + kQueueChunkMin - 1) / kQueueChunkMin;
-    while (qc.split < kQueueChunkMin && chunks * qc.split < max_slots) qc.split *= 2;
+    qc.clusters = cluster_form(qc.M, qc.K, qc.items(1), clusters, ctas);
+    class_slots.push_back(qc.clusters ? clusters : ctas);
   }
   pl->queued.assign(B, 0);
   for (int b = 0; b < B; ++b) {
@@ -1283,8 +1300,7 @@ ptycho_status ptycho_plan_batch(int32_t B, const ptycho_params* const* params, c
       m->iter = params[b]->start_iteration;
       m->device = pl->device;
       if (member_class[b] >= 0) {
-        const auto& qc = pl->qclasses[member_class[b]];
-        const int len = qc.chunk_len / qc.split;
+        const int c = member_class[b], len = pl->qclasses[c].item_length(kQueueChunkMin, class_slots[c]);
         m->parts = (m->p.N + len - 1) / len;
         pl->queued[b] = 1;
       }
@@ -1297,22 +1313,23 @@ ptycho_status ptycho_plan_batch(int32_t B, const ptycho_params* const* params, c
       return fail(st, msg);
     }
   }
-  // chunk lists, sized for the smallest chunk length (the most chunks); the autotuner then picks the
-  // length per class and the lists and partial counts are rebuilt for it
-  for (auto& qc : pl->qclasses) {
-    int max_chunks = 0;
-    for (int b : qc.members) max_chunks += pl->members[b]->parts;
-    int max_slots = 0;
-    PT_CUDA(pl->alloc(&qc.d_chunks, (size_t)max_chunks), "alloc chunk list");
+  // item lists, sized for the smallest chunk length (the most items); the autotuner then picks the
+  // length per class and the lists and partial counts are rebuilt for it. A class whose smallest chunks are split
+  // has the same items for every length: nothing to tune. Otherwise what is fastest depends on how many chunks
+  // a CTA takes, so classes share a length only within a factor of two of that.
+  for (size_t c = 0; c < pl->qclasses.size(); ++c) {
+    auto& qc = pl->qclasses[c];
+    const int max_slots = class_slots[c], smallest = qc.item_length(kQueueChunkMin, max_slots);
+    PT_CUDA(pl->alloc(&qc.d_chunks, (size_t)qc.items(smallest)), "alloc chunk list");
     PT_CUDA(pl->alloc(&qc.d_queue, 1), "alloc work counter");
-    PT_CUDA(fused_queue_max_slots(qc.M, qc.K, &max_slots), "occupancy of the work-queue kernel");
-    if (max_slots < 1) return fail(PTYCHO_EUNSUPPORTED, "a cluster of K CTAs does not fit on this device");
-    const std::tuple<int, int, int, int, int> key{pl->device, qc.M, qc.K, qc.near, qc.kh};
-    int L = 0;
+    int fill = 0;
+    while (fill < 16 && qc.items(1) >> (fill + 1) >= max_slots) ++fill;
+    const std::tuple<int, int, int, int, int, int> key{pl->device, qc.M, qc.K, qc.near, qc.kh, fill};
+    int L = smallest < kQueueChunkMin ? kQueueChunkMin : 0;
     {
       std::lock_guard<std::mutex> lock(g_tune_mutex);
       if (g_fixed_chunk > 0) L = g_fixed_chunk;
-      else if (g_tune_cache.count(key)) L = g_tune_cache[key];
+      else if (L == 0 && g_tune_cache.count(key)) L = g_tune_cache[key];
     }
     if (L == 0) {
       ptycho_status st = tune_chunk_length(pl, qc, max_slots, &L);
@@ -1394,7 +1411,7 @@ ptycho_status ptycho_iterate_batch(ptycho_plan_t pl, void* const* objects, void*
         fa.nchunks = qc.nitems;
         fa.queue = qc.d_queue;
         fa.kh = qc.kh;
-        if (ce == cudaSuccess) ce = launch_fused_queue(qc.M, fa, qc.slots, bs);
+        if (ce == cudaSuccess) ce = launch_queue(qc, fa, qc.slots, bs);
         for (size_t j = 0; j < qc.members.size() && ce == cudaSuccess && st == PTYCHO_OK; ++j) {
           const int b = qc.members[j];
           st = enqueue_update(pl->members[b], objects[b], probes[b], pl->members[b]->iter, bs);
@@ -1485,9 +1502,22 @@ ptycho_status ptycho_batch_classes(ptycho_plan_t pl, int32_t max_classes, int32_
   *count = (int32_t)pl->qclasses.size();
   for (int c = 0; c < std::min<int>(max_classes, *count); ++c) {
     const auto& qc = pl->qclasses[c];
+    const int per_chunk = qc.chunk_len / qc.item_len;  // items
     const int32_t v[8] = {qc.M, qc.K, qc.near, qc.kh, (int32_t)qc.members.size(), qc.chunk_len, qc.nchunks,
-                          (qc.slots + qc.split - 1) / qc.split};
+                          (qc.slots + per_chunk - 1) / per_chunk};
     std::memcpy(out + 8 * c, v, sizeof(v));
+  }
+  return PTYCHO_OK;
+}
+
+ptycho_status ptycho_batch_items(ptycho_plan_t pl, int32_t max_classes, int32_t* out, int32_t* count) {
+  if (!pl || pl->members.empty() || !count || max_classes < 0 || (max_classes > 0 && !out))
+    return fail(PTYCHO_EINVAL, "not a batch plan or bad output");
+  *count = (int32_t)pl->qclasses.size();
+  for (int c = 0; c < std::min<int>(max_classes, *count); ++c) {
+    const auto& qc = pl->qclasses[c];
+    const int32_t v[4] = {qc.item_len, qc.nitems, qc.clusters ? qc.K : 1, qc.slots * (qc.clusters ? qc.K : 1)};
+    std::memcpy(out + 4 * c, v, sizeof(v));
   }
   return PTYCHO_OK;
 }

@@ -65,10 +65,12 @@ cudaError_t fused_max_slots(int M, int K, int* slots);
 // as launch_fused (errpart slots x K, one entry per rank)
 cudaError_t launch_fused_cluster(int M, const FusedArgs& a, int slots, cudaStream_t s);
 cudaError_t fused_cluster_max_slots(int M, int K, int* slots);
-// work-queue launch: `slots` persistent CTAs drain a.chunks through a.queue;
+// work-queue launch: `slots` persistent CTAs (or clusters of K) drain a.chunks through a.queue;
 // a.K, a.near_field, a.kh (kernel width class) and a.tw are those of every problem in a.probs
 cudaError_t launch_fused_queue(int M, const FusedArgs& a, int slots, cudaStream_t s);
 cudaError_t fused_queue_max_slots(int M, int K, int* slots);
+cudaError_t launch_fused_queue_cluster(int M, const FusedArgs& a, int slots, cudaStream_t s);
+cudaError_t fused_queue_cluster_max_slots(int M, int K, int* slots);
 // pc-DM launch (single problem, M <= 128): as launch_fused with the exit-wave state a.psi and no probe
 // partials; and as launch_fused_cluster
 cudaError_t launch_fused_dm(int M, const FusedArgs& a, int slots, cudaStream_t s);

@@ -71,7 +71,10 @@ struct FusedSmem {
   static constexpr size_t TAPS = 2 * kMaxTaps * 4 + 8 + 16;  // taps, TMEM address, mbarrier (16-byte aligned)
   static constexpr size_t TW2 = (M >= 64 ? M : 0) * 8;  // second twiddles of fft3.cuh (Tile3::TW2)
   static constexpr size_t BYTES = CBUF + IBUF + TWT + TW2 + HQ + TAPS;
-  static_assert(BYTES <= 232448, "shared memory budget of one CTA");
+  // queued launches: the current problem's arguments and the item index handed out by rank 0
+  static constexpr size_t DESC = (sizeof(FusedArgs) + 15) / 16 * 16 + 16;
+  static constexpr size_t bytes(int mode) { return BYTES + (mode == QUEUED ? DESC : 0); }
+  static_assert(BYTES % 16 == 0 && BYTES + DESC <= 232448, "shared memory budget of one CTA");
 };
 
 // lines per thread: the 128 x 128 tile runs on 512 threads with two lines each
@@ -89,7 +92,7 @@ struct FusedShape {
                 "TMEM allocation must be a power of two in [32, 512] columns");
 };
 
-// MODE: SINGLE one problem (a mini-batch); DM the difference map on one problem (pc_fused_seq.cuh describes both)
+// MODE: SINGLE one problem (a mini-batch); QUEUED the work items of several; DM the difference map on one
 template <int M, bool NEAR, int KH, int MODE>
 __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const FusedArgs a_in) {
   using TL = Tile<M>;
@@ -126,7 +129,7 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
   constexpr bool F3 = M >= 64;
   if constexpr (F3)
     for (int i = tid; i < Tile3<M>::TW2; i += TR) s_tw2[i] = a_in.tw[Tile3<M>::tw2_exp(i)];
-  probe_map<M>(a_in, TR);
+  if constexpr (MODE != QUEUED) probe_map<M>(a_in, TR);
   int line[V], tp[V];
 #pragma unroll
   for (int v = 0; v < V; ++v) {
@@ -551,13 +554,39 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
     __syncthreads();  // red aliases the exchange buffer
   };
 
-  // cluster `slot` takes positions slot, slot + slots, ... and owns partial `slot`
-  setup_unit(a_in);
-  __syncthreads();
-  float2* pacc = MODE == DM ? nullptr : a_in.pacc + ((size_t)slot * K + rank) * M * M;
-  float* dacc = MODE == DM ? nullptr : a_in.dacc + (size_t)slot * M * M;
-  for (int n = slot; n < a_in.N; n += nslots) run_position(a_in, n, n == slot, pacc, dacc);
-  finish_unit(a_in, pacc, slot);
+  if constexpr (MODE == QUEUED) {
+    // work item (problem, first position, end, partial): rank 0 takes the next index and hands it to every rank
+    // (which read the last one before the cluster barriers of its positions)
+    FusedArgs* s_desc = reinterpret_cast<FusedArgs*>(smem + SM::BYTES);
+    int* s_item = reinterpret_cast<int*>(smem + SM::BYTES + SM::DESC - 16);
+    for (;;) {
+      if (rank == 0 && tid == 0) {
+        const int c = atomicAdd(a_in.queue, 1);
+        for (int q = 0; q < K; ++q) st_cluster_s32(map_rank(smem_addr(s_item), (unsigned)q), c);
+      }
+      cluster_sync_all();
+      const int c = *s_item;
+      if (c >= a_in.nchunks) break;
+      const int4 ch = a_in.chunks[c];
+      const int* src = reinterpret_cast<const int*>(a_in.probs + ch.x);
+      for (int i = tid; i < (int)(sizeof(FusedArgs) / 4); i += TR) reinterpret_cast<int*>(s_desc)[i] = src[i];
+      __syncthreads();
+      setup_unit(*s_desc);
+      __syncthreads();
+      float2* pacc = s_desc->pacc + ((size_t)ch.w * K + rank) * M * M;
+      float* dacc = s_desc->dacc + (size_t)ch.w * M * M;
+      for (int n = ch.y; n < ch.z; ++n) run_position(*s_desc, n, n == ch.y, pacc, dacc);
+      finish_unit(*s_desc, pacc, ch.w);
+    }
+  } else {
+    // cluster `slot` takes positions slot, slot + slots, ... and owns partial `slot`
+    setup_unit(a_in);
+    __syncthreads();
+    float2* pacc = MODE == DM ? nullptr : a_in.pacc + ((size_t)slot * K + rank) * M * M;
+    float* dacc = MODE == DM ? nullptr : a_in.dacc + (size_t)slot * M * M;
+    for (int n = slot; n < a_in.N; n += nslots) run_position(a_in, n, n == slot, pacc, dacc);
+    finish_unit(a_in, pacc, slot);
+  }
   if constexpr (TM) {
     tmem_fence_before();
     __syncthreads();
@@ -567,12 +596,12 @@ __global__ void __launch_bounds__(FusedShape<M>::TR, 1) pc_fused_kernel(const Fu
 }
 
 // ------------------------------------------------------------------ launches
-template <int M, int KH>
+template <int M, int KH, int MODE>
 static cudaLaunchConfig_t fused_config(const FusedArgs& a, int slots, cudaStream_t s, cudaLaunchAttribute* attr) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(slots * a.K));
   cfg.blockDim = dim3(FusedShape<M>::TR);
-  cfg.dynamicSmemBytes = FusedSmem<M, KH>::BYTES;
+  cfg.dynamicSmemBytes = FusedSmem<M, KH>::bytes(MODE);
   cfg.stream = s;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned)a.K;
@@ -586,10 +615,11 @@ static cudaLaunchConfig_t fused_config(const FusedArgs& a, int slots, cudaStream
 template <int M, bool NEAR, int KH, int MODE>
 static cudaError_t launch_cluster_kh(const FusedArgs& a, int slots, cudaStream_t s) {
   auto kern = pc_fused_kernel<M, NEAR, KH, MODE>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FusedSmem<M, KH>::BYTES);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)FusedSmem<M, KH>::bytes(MODE));
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = fused_config<M, KH>(a, slots, s, attr);
+  cudaLaunchConfig_t cfg = fused_config<M, KH, MODE>(a, slots, s, attr);
   return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
@@ -618,12 +648,13 @@ static cudaError_t launch_cluster(int M, const FusedArgs& a, int slots, cudaStre
 template <int M, int MODE>
 static cudaError_t cluster_slots_t(int K, int* slots) {
   auto kern = pc_fused_kernel<M, false, 15, MODE>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FusedSmem<M, 15>::BYTES);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)FusedSmem<M, 15>::bytes(MODE));
   if (e != cudaSuccess) return e;
   FusedArgs a = {};
   a.K = K;
   cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = fused_config<M, 15>(a, 1, 0, attr);
+  cudaLaunchConfig_t cfg = fused_config<M, 15, MODE>(a, 1, 0, attr);
   int n = 0;
   e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
   *slots = n;

@@ -106,7 +106,7 @@ struct SeqSmem {
   static constexpr size_t BYTES = CBUF + ZBUF + TWT + TW2 + HQ + TAPS;
   // queued launches: the current problem's arguments and the chunk index
   static constexpr size_t DESC = (sizeof(FusedArgs) + 15) / 16 * 16 + 16;
-  static constexpr size_t bytes(int mode) { return BYTES + (mode == 1 ? DESC : 0); }
+  static constexpr size_t bytes(int mode) { return BYTES + (mode == QUEUED ? DESC : 0); }
   static_assert(BYTES % 16 == 0 && BYTES + DESC <= 232448, "shared memory budget of one CTA");
   static_assert((size_t)SeqShape<M>::TR * 8 <= CBUF, "error reduction buffer");
 };
