@@ -150,11 +150,15 @@ ptycho_status ptycho_iterate(ptycho_plan_t plan, void* object, void* probe, int3
 
 /* Synchronise the plan's stream and return E of the last iteration run
  * (host double). PTYCHO_EINVAL if no iteration has run yet; PTYCHO_ENUMERIC
- * if E is not finite. */
+ * if E is not finite; PTYCHO_ETIMEOUT if a bounded device wait of the plan's
+ * launches gave up since the last such call (results are not valid; reported
+ * once, by whichever of ptycho_error, ptycho_error_history and
+ * ptycho_error_batch comes first). */
 ptycho_status ptycho_error(ptycho_plan_t plan, double* nrmse_last);
 
 /* Synchronise and copy the errors of the last min(n, runs, 4096) iterations,
- * oldest first, into out (host, n doubles); *count receives how many. */
+ * oldest first, into out (host, n doubles); *count receives how many.
+ * PTYCHO_ETIMEOUT as ptycho_error. */
 ptycho_status ptycho_error_history(ptycho_plan_t plan, double* out, int32_t n, int32_t* count);
 
 /* Release every device resource of the plan (synchronises its stream). */
@@ -397,12 +401,15 @@ ptycho_status ptycho_measure_fp32_peak(double* tflops, double* ms, void* cuda_st
  * mbarrier wait of the kind the cluster-form fused kernels use on their copy barriers, with a
  * budget of budget_ns nanoseconds (0 ... 2e9, the kernels' own budget being 2 s). With signal != 0
  * the barrier is completed before the wait, which then succeeds (PTYCHO_OK); with signal == 0
- * nothing ever completes it, the wait gives up after the budget and sets the device flag that
- * ptycho_error reads, and this call reports it: PTYCHO_ETIMEOUT, the flag cleared and the context
- * still usable. Synchronises the stream. A timeout left pending by an earlier launch is reported
- * (and cleared) before the test runs, as PTYCHO_ETIMEOUT. PTYCHO_EINVAL for a budget out of
- * range (checked before any device work), PTYCHO_ECUDA. */
+ * nothing ever completes it, the wait gives up after the budget and raises a host-visible flag of this
+ * call, which reports it: PTYCHO_ETIMEOUT, the context still usable. Synchronises the stream.
+ * PTYCHO_EINVAL for a budget out of range (checked before any device work), PTYCHO_ECUDA. */
 ptycho_status ptycho_wait_selftest(int64_t budget_ns, int32_t signal, void* cuda_stream);
+/* The same wait on the plan's stream with the plan's own flag (of `member` for a batch plan, 0 for a
+ * single one), without synchronising: if it gives up, the plan's next ptycho_error,
+ * ptycho_error_history or ptycho_error_batch reports PTYCHO_ETIMEOUT, as for a wait of the plan's
+ * kernels. PTYCHO_EINVAL for a NULL plan, no such member or a budget out of range, PTYCHO_ECUDA. */
+ptycho_status ptycho_plan_wait_selftest(ptycho_plan_t plan, int32_t member, int64_t budget_ns, int32_t signal);
 
 /* Message of the calling thread's last failed call ("" if none). */
 const char* ptycho_last_error(void);

@@ -28,7 +28,7 @@ EXPORTED = ("ptycho_plan", "ptycho_iterate", "ptycho_error", "ptycho_error_histo
             "ptycho_batch_launches", "ptycho_set_staged_chunk", "ptycho_staged_chunk", "ptycho_permutation", "ptycho_unet_create", "ptycho_unet_param_count", "ptycho_unet_set_params",
             "ptycho_unet_get_params", "ptycho_unet_forward", "ptycho_unet_gradients", "ptycho_unet_train_step",
             "ptycho_unet_destroy", "ptycho_generate", "ptycho_warmstart", "ptycho_monochromatise",
-            "ptycho_measure_fp32_peak", "ptycho_wait_selftest")
+            "ptycho_measure_fp32_peak", "ptycho_wait_selftest", "ptycho_plan_wait_selftest")
 
 
 class PtychoError(RuntimeError):
@@ -139,6 +139,8 @@ def load(build_if_missing: bool = True) -> ctypes.CDLL:
     lib.ptycho_version.restype = ctypes.c_char_p
     lib.ptycho_measure_fp32_peak.argtypes = [ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_double), P]
     lib.ptycho_measure_fp32_peak.restype = st
+    lib.ptycho_plan_wait_selftest.argtypes = [P, ctypes.c_int32, ctypes.c_int64, ctypes.c_int32]
+    lib.ptycho_plan_wait_selftest.restype = st
     lib.ptycho_wait_selftest.argtypes = [ctypes.c_int64, ctypes.c_int32, P]
     lib.ptycho_wait_selftest.restype = st
     F32 = ctypes.c_float

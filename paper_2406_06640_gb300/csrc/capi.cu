@@ -1554,6 +1554,7 @@ ptycho_status ptycho_error_history(ptycho_plan_t pl, double* out, int32_t n, int
   if (!pl || !out || !count || n < 0) return fail(PTYCHO_EINVAL, "bad argument");
   if (!pl->members.empty()) return fail(PTYCHO_EINVAL, "batch plans report through ptycho_error_batch");
   PT_CUDA(cudaStreamSynchronize(pl->stream), "stream sync");
+  if (pl->timed_out()) return fail(PTYCHO_ETIMEOUT, "a bounded device wait gave up; results are not valid");
   const long long c = std::min<long long>({(long long)n, pl->runs, (long long)kErrHistory});
   std::vector<double> ring(kErrHistory);
   PT_CUDA(cudaMemcpy(ring.data(), pl->d_errhist, sizeof(double) * kErrHistory, cudaMemcpyDeviceToHost),
@@ -1686,6 +1687,18 @@ ptycho_status ptycho_wait_selftest(int64_t budget_ns, int32_t signal, void* cuda
   cudaFreeHost(flag);
   PT_CUDA(ce, "self-test");
   if (gave_up) return fail(PTYCHO_ETIMEOUT, "the self-test wait gave up after its budget");
+  return PTYCHO_OK;
+}
+
+ptycho_status ptycho_plan_wait_selftest(ptycho_plan_t pl, int32_t member, int64_t budget_ns, int32_t signal) {
+  if (!pl) return fail(PTYCHO_EINVAL, "plan is NULL");
+  if (member < 0 || member >= (int32_t)std::max<size_t>(pl->members.size(), 1))
+    return fail(PTYCHO_EINVAL, "no such member");
+  if (budget_ns < 0 || budget_ns > 2000000000LL) return fail(PTYCHO_EINVAL, "budget_ns must be in [0, 2e9]");
+  PT_CUDA(cudaSetDevice(pl->device), "cudaSetDevice");
+  const ptycho_plan_s* m = pl->members.empty() ? pl : pl->members[member];
+  PT_CUDA(launch_wait_selftest((unsigned long long)budget_ns, signal != 0, m->fa.timeout, pl->stream),
+          "self-test launch");
   return PTYCHO_OK;
 }
 
