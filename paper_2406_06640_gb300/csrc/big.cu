@@ -310,8 +310,9 @@ __device__ __forceinline__ void red_add(float* a, float v) {
 
 // ---- final inverse row DFT of every mode, dpsi, contributions. A CTA owns FR rows of the tile and walks the
 // positions g, g + groups, ... of the chunk (g = blockIdx.y) and their modes.
-// ACC: the probe partial of (group, mode, rows) stays in shared memory, every element touched by one thread,
-// and is read and written once per launch. Otherwise (partials of K modes too large for three CTAs on an
+// ACC: the launch's probe sums of (group, mode, rows) stay in shared memory, every element touched by one thread,
+// and are added to the group's partial once per launch (a sum of sums: one chain over all chunks' positions
+// would be several times longer than the partials per position of a chunk that it replaces). Otherwise (partials of K modes too large for three CTAs on an
 // SM) one group per position and L2 reductions into its partial. pc-DM (b.psi) has no probe partials here.
 template <int BL>
 struct FinalShape {
@@ -340,10 +341,6 @@ __global__ void __launch_bounds__(FinalShape<BL>::TPB) k_big_final(const BigArgs
   const float s = 1.0f / (float)(BL * BL);
   float2* pacc = b.pacc + (size_t)g * K * MM + yo;
   float* dacc = b.dacc + (size_t)g * MM + yo;
-  if (ACC && !start)
-    for (int k = 0; k < K; ++k)
-#pragma unroll
-      for (int j = 0; j < E; ++j) s_p[(k * FR + li) * BL + t + 16 * j] = pacc[(size_t)k * MM + t + 16 * j];
   float dsum[E];
 #pragma unroll
   for (int j = 0; j < E; ++j) dsum[j] = 0.f;
@@ -356,7 +353,7 @@ __global__ void __launch_bounds__(FinalShape<BL>::TPB) k_big_final(const BigArgs
   if constexpr (AHEAD) line(g, 0, nx);
   for (int c = g; c < nc; c += G) {
     const int n = b.n0 + c;
-    const bool first = start && c == g;
+    const bool first = c == g && (ACC || start);
     const int2 pn = b.pos[n];
     const float2* On = b.O + (size_t)(pn.x + y) * b.obj_w + pn.y;
     float2 cacc[E], ov[AHEAD ? E : 1];
@@ -418,7 +415,11 @@ __global__ void __launch_bounds__(FinalShape<BL>::TPB) k_big_final(const BigArgs
   if constexpr (ACC)
     for (int k = 0; k < K; ++k)
 #pragma unroll
-      for (int j = 0; j < E; ++j) pacc[(size_t)k * MM + t + 16 * j] = s_p[(k * FR + li) * BL + t + 16 * j];
+      for (int j = 0; j < E; ++j) {
+        float2& q = pacc[(size_t)k * MM + t + 16 * j];
+        const float2 v = s_p[(k * FR + li) * BL + t + 16 * j];
+        q = start ? v : cadd(q, v);
+      }
 }
 
 template <int BL, int OP>

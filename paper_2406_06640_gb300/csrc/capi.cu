@@ -102,9 +102,12 @@ static std::vector<int> philox_permutation(int n, uint64_t seed, uint32_t stream
   return a;
 }
 
-// pc-DM: groups of positions the probe sums are split into. 32 groups of M^2 / 512 blocks fill the GPU at
-// M = 128 while their partials (32 K M^2 complex) stay small beside the state they are summed from
-constexpr int kDmParts = 32;
+// pc-DM: groups of positions the probe sums are split into. 32 groups of M^2 / 512 blocks fill the GPU at M = 128
+// while their partials stay small beside the state they are summed from (1 / 24 of it at most); longer scans take
+// more, so that no sum is longer than with a partial per cluster of the fused launch (900 positions, four modes: 24
+// terms, then 38 partials in eight sums). A group per resident CTA costs 400 positions of 128^2, one mode, 239 us
+// an iteration against 206.
+static int dm_groups(int N) { return std::min(N, std::max(32, (N + 23) / 24)); }
 
 // Whether n positions run faster as clusters of K CTAs than with one CTA each: waves of a launch times the cost
 // of a position, about (K + 1/2) mode passes one after the other against a cluster's fixed cost in the same
@@ -557,7 +560,7 @@ static ptycho_status build_plan(ptycho_plan_s* pl, const float* intensities, con
   PT_CUDA(pl->alloc(&d_cn, (size_t)N * MM), "alloc contributions");
   // probe partials: one per slot, or (pc-DM, whose probe sums are a pass of their own over the state)
   // one per group of positions
-  const int parts = p.engine == PTYCHO_ENGINE_DM ? std::min(N, kDmParts) : pl->slots;
+  const int parts = p.engine == PTYCHO_ENGINE_DM ? dm_groups(N) : pl->slots;
   PT_CUDA(pl->alloc(&d_pacc, (size_t)parts * K * MM), "alloc probe partials");
   PT_CUDA(pl->alloc(&d_dacc, (size_t)parts * MM), "alloc probe partials");
   const size_t nerr = pl->big ? (size_t)N * big_row_blocks(M) : (size_t)pl->slots * K;

@@ -11,7 +11,6 @@ namespace ptycho {
 constexpr int kMaxTaps = 31;        // largest odd Gaussian kernel side accepted (Eq. 7 support)
 constexpr int kObjTile = 32;        // object tile side of the gather kernels
 constexpr int kMaxModes = 8;        // probe modes K handled (one cluster rank per mode)
-constexpr int kObjSplit = 8;        // position groups per object tile (one cluster, fixed order)
 constexpr int kErrHistory = 4096;   // ring of per-iteration errors kept on the device
 
 // Arguments of the fused per-position kernels.

@@ -182,18 +182,26 @@ static void launch_dm_probe_partials(const UpdateArgs& u, cudaStream_t s) {
 //   SPLIT = 8: a unit is a whole tile (PX = 4) shared by a cluster of eight blocks. Block `rank` takes terms
 //     rank, rank + 8, ..., and the ranks' sums are added in rank order through distributed shared memory. For
 //     long lists: a tile in the middle of a dense scan holds hundreds of positions.
-//   SPLIT = 1: a unit is 8 rows of a tile (PX = 1) and one block. For short lists (mini-batches, small scans),
-//     where the blocks of a cluster would mostly start, meet and end.
-// Bound by the latency of the term loads: 4 / PX positions of PX pixels and their |P|^2 in flight per thread. The
-// line between the forms is 24 terms on average. (Clusters of 8-row bands: 104 us against 77 us for 900
-// positions of 128^2 on 640^2, most blocks of the border tiles being overhead.)
+//   SPLIT = 1: a unit is 8 rows of a tile (PX = 1) and one block, whose threads hold the eight sums themselves. For
+//     short lists (mini-batches, small scans), where the blocks of a cluster would mostly start, meet and end.
+// Both forms add the same terms in the same order, so their results are the same bits: eight sums of every eighth
+// term, then those in order (a chain of all terms loses three bits more on a scan of hundreds).
+// Bound by the latency of the term loads: four (SPLIT = 8) or eight positions of PX pixels and their |P|^2 in flight
+// per thread. The line between the forms is 24 terms on average, where small scans cross: iterations of one mode,
+// SPLIT = 8 against 1, 100 positions of 64^2: 31 / 33 us at 22 terms, 31 / 35 at 29, 31 / 37 at 49; of 128^2: 59 / 52
+// at 18, 57 / 55 at 25, 54 / 58 at 45; 400 of 32^2: 43 / 41 at 7, 38 / 39 at 30, 35 / 47 at 86. Scans of more tiles
+// than the GPU has blocks cross later (400 of 128^2: 159 / 131 at 12, 149 / 131 at 25, 133 / 133 at 65, 129 / 138
+// at 96; 256^2 near 100). The probe side follows the object's form; with many slots and few probe pixels the split
+// would be faster for short lists too (900 positions of 8^2: 38 / 46). (Clusters of 8-row bands: 104 us against 77 us
+// for 900 positions of 128^2 on 640^2, most blocks of the border tiles being overhead.)
 // The maxima of D_O and D_P are integer atomics on the float bits (non-negative: the order of the bits),
 // so they do not depend on the order either.
 template <int SPLIT>
-__global__ void __launch_bounds__(256, SPLIT == 8 ? 3 : 4) k_gather(const UpdateArgs u, int units_o) {
+__global__ void __launch_bounds__(256, 3) k_gather(const UpdateArgs u, int units_o) {
   static_assert(SPLIT == 1 || SPLIT == 8, "cluster size");
   constexpr int PX = SPLIT == 8 ? 4 : 1, VALUES = 256 * PX, BANDS = 4 / PX;  // units per tile
   constexpr int U = SPLIT == 8 ? 4 : 8;                                      // positions in flight
+  constexpr int SUMS = 8 / SPLIT;                                            // of this thread, per value
   __shared__ float2 s_acc[SPLIT > 1 ? VALUES : 1];
   __shared__ float s_den[SPLIT > 1 ? VALUES : 1];
   const int unit = blockIdx.x / SPLIT, rank = SPLIT > 1 ? (int)cluster_ctarank() : 0;
@@ -227,13 +235,15 @@ __global__ void __launch_bounds__(256, SPLIT == 8 ? 3 : 4) k_gather(const Update
     }
   };
   constexpr int RPR = VALUES / SPLIT;  // values a rank finishes
-  float2 acc[PX];
-  float den[PX];
+  float2 acc[SUMS][PX];
+  float den[SUMS][PX];
 #pragma unroll
-  for (int i = 0; i < PX; ++i) {
-    acc[i] = make_float2(0.f, 0.f);
-    den[i] = 0.f;
-  }
+  for (int r = 0; r < SUMS; ++r)
+#pragma unroll
+    for (int i = 0; i < PX; ++i) {
+      acc[r][i] = make_float2(0.f, 0.f);
+      den[r][i] = 0.f;
+    }
   if (obj) {
     const int s0 = u.tile_start[tile], s1 = u.tile_start[tile + 1];
     if (s0 == s1) {  // no position (the same in every rank)
@@ -263,35 +273,59 @@ __global__ void __launch_bounds__(256, SPLIT == 8 ? 3 : 4) k_gather(const Update
       for (int r = 0; r < U; ++r)
 #pragma unroll
         for (int i = 0; i < PX; ++i) {
-          acc[i] = cadd(acc[i], cv[r][i]);
-          den[i] += dv[r][i];
+          acc[r % SUMS][i] = cadd(acc[r % SUMS][i], cv[r][i]);
+          den[r % SUMS][i] += dv[r][i];
         }
     }
   } else if (k < u.K) {
     const float2* part[PX];  // (past the last pixel: that pixel again, not stored)
 #pragma unroll
     for (int i = 0; i < PX; ++i) part[i] = u.pacc + (size_t)k * MM + min(P0 + tid + 256 * i, MM - 1);
-#pragma unroll 8 / PX * 2
-    for (int s = rank; s < u.slots; s += SPLIT)
+    // rounds of eight partials, sixteen loads in flight: no branch between the loads of a round
+    int s = 0;
+#pragma unroll SPLIT == 1 ? 2 : 4
+    for (; s + 8 <= u.slots; s += 8)
 #pragma unroll
-      for (int i = 0; i < PX; ++i) acc[i] = cadd(acc[i], part[i][(size_t)s * u.K * MM]);
+      for (int r = 0; r < SUMS; ++r)
+#pragma unroll
+        for (int i = 0; i < PX; ++i) acc[r][i] = cadd(acc[r][i], part[i][(size_t)(s + rank + r) * u.K * MM]);
+#pragma unroll
+    for (int r = 0; r < SUMS; ++r)
+      if (s + rank + r < u.slots)
+#pragma unroll
+        for (int i = 0; i < PX; ++i) acc[r][i] = cadd(acc[r][i], part[i][(size_t)(s + rank + r) * u.K * MM]);
   } else {
     const float* part[PX];
 #pragma unroll
     for (int i = 0; i < PX; ++i) part[i] = u.dacc + min(P0 + tid + 256 * i, MM - 1);
-#pragma unroll 8 / PX * 2
-    for (int s = rank; s < u.slots; s += SPLIT)
+    int s = 0;
+#pragma unroll SPLIT == 1 ? 2 : 4
+    for (; s + 8 <= u.slots; s += 8)
 #pragma unroll
-      for (int i = 0; i < PX; ++i) den[i] += part[i][(size_t)s * MM];
+      for (int r = 0; r < SUMS; ++r)
+#pragma unroll
+        for (int i = 0; i < PX; ++i) den[r][i] += part[i][(size_t)(s + rank + r) * MM];
+#pragma unroll
+    for (int r = 0; r < SUMS; ++r)
+      if (s + rank + r < u.slots)
+#pragma unroll
+        for (int i = 0; i < PX; ++i) den[r][i] += part[i][(size_t)(s + rank + r) * MM];
   }
   // (thread tid's values are tid, tid + 256, ...: rows tid / 32 + 8 i of a tile)
   if constexpr (SPLIT == 1) {
-    store(tid, acc[0], den[0]);
+    float2 a = make_float2(0.f, 0.f);
+    float d = 0.f;
+#pragma unroll
+    for (int r = 0; r < SUMS; ++r) {
+      a = cadd(a, acc[r][0]);
+      d += den[r][0];
+    }
+    store(tid, a, d);
   } else {
 #pragma unroll
     for (int i = 0; i < PX; ++i) {
-      s_acc[tid + 256 * i] = acc[i];
-      s_den[tid + 256 * i] = den[i];
+      s_acc[tid + 256 * i] = acc[0][i];
+      s_den[tid + 256 * i] = den[0][i];
     }
     cluster_sync_all();  // every rank's sums are complete
     if (tid < RPR) {
