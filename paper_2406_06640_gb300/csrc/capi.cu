@@ -67,9 +67,10 @@ constexpr int kQueueChunkMin = 8;
 std::mutex g_tune_mutex;
 std::map<std::tuple<int, int, int, int, int, int>, int> g_tune_cache;
 int g_fixed_chunk = 0;
-// staged path (M = 256, 512): positions per chunk of the staged passes, same key, and its fixed value
+// staged path (M = 256, 512): positions per chunk of the staged passes, per (device, M, K, geometry, kernel width
+// class, engine), and its fixed value
 constexpr int kStagedCandidates[] = {4, 8, 16, 32};
-std::map<std::tuple<int, int, int, int, int>, int> g_tune_staged;
+std::map<std::tuple<int, int, int, int, int, int>, int> g_tune_staged;
 int g_fixed_staged = 0;
 
 // Philox4x32-10 on the host (Salmon et al., SC'11) and the Fisher-Yates permutation of 0..n-1 that
@@ -343,10 +344,6 @@ static bool is_device_pointer(const void* ptr) {
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
-// Autotuner of the staged path (M = 256, 512): positions per chunk of the staged passes, timed on the
-// device for each candidate over one pass of all positions (object and probe from scratch buffers
-// of ones -- the passes only read them; they write the scratch, contributions and partials, which
-// the first real iteration overwrites), best of two after a warm-up.
 // Host vector -> plan buffer: ordered on the plan's stream and complete when it returns (a blocking
 // copy on the legacy stream is not ordered against a non-blocking caller stream).
 static cudaError_t h2d(cudaStream_t s, void* dst, const void* src, size_t bytes) {
@@ -354,6 +351,11 @@ static cudaError_t h2d(cudaStream_t s, void* dst, const void* src, size_t bytes)
   return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
 }
 
+// Autotuner of the staged path (M = 256, 512): positions per chunk of the staged passes, timed on the
+// device for each candidate over one pass of all positions (object and probe from scratch buffers
+// of ones -- the passes only read them; they write the scratch, contributions and partials, or the exit-wave
+// state of pc-DM as its first iteration does, which the first real iteration overwrites), best of two
+// after a warm-up.
 static ptycho_status tune_staged_chunk(ptycho_plan_s* pl, int* best) {
   cudaStream_t s = pl->stream;
   const ptycho_params& p = pl->p;
@@ -369,6 +371,8 @@ static ptycho_status tune_staged_chunk(ptycho_plan_s* pl, int* best) {
   BigArgs ba = pl->ba;
   ba.O = d_o;
   ba.P = d_p;
+  ba.psi = pl->d_psi;  // (null unless pc-DM)
+  ba.dm_init = 1;
   cudaEvent_t e0, e1;
   PT_CUDA(cudaEventCreate(&e0), "event");
   PT_CUDA(cudaEventCreate(&e1), "event");
@@ -379,12 +383,12 @@ static ptycho_status tune_staged_chunk(ptycho_plan_s* pl, int* best) {
     const int c = std::min(cand, pl->chunk);
     if (cand > kStagedCandidates[0] && c != cand) break;  // larger candidates than N add nothing
     float t_best = 1e30f;
+    ce = big_groups(p.M, p.K, ba.psi != nullptr, c, &ba.groups);
     for (int r = 0; r < 3 && ce == cudaSuccess; ++r) {
       ce = cudaEventRecord(e0, s);
-      ce = big_groups(p.M, p.K, p.engine == PTYCHO_ENGINE_DM, c, &ba.groups);
       for (int n0 = 0; n0 < p.N && ce == cudaSuccess; n0 += c) {
         ba.n0 = n0;
-        ce = launch_big_chunk(ba, std::min(c, p.N - n0), s);
+        ce = ba.psi ? launch_big_chunk_dm(ba, std::min(c, p.N - n0), s) : launch_big_chunk(ba, std::min(c, p.N - n0), s);
       }
       if (ce == cudaSuccess) ce = cudaEventRecord(e1, s);
       if (ce == cudaSuccess) ce = cudaEventSynchronize(e1);
@@ -740,7 +744,7 @@ static ptycho_status build_plan(ptycho_plan_s* pl, const float* intensities, con
 
   PT_CUDA(cudaStreamSynchronize(s), "plan sync");
   if (pl->big) {
-    const std::tuple<int, int, int, int, int> key{pl->device, M, K, fa.near_field, kh == 5 ? 5 : 15};
+    const std::tuple<int, int, int, int, int, int> key{pl->device, M, K, fa.near_field, kh == 5 ? 5 : 15, p.engine};
     int c = 0;
     {
       std::lock_guard<std::mutex> lock(g_tune_mutex);
