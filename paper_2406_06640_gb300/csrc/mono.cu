@@ -389,7 +389,7 @@ struct WalkShape {
   static constexpr size_t bytes(int J, bool ft) { return FIXED + (size_t)J * (TAB + (ft ? TAB_F : 0)) + 16; }
   static constexpr size_t LIMIT = MIN_BLOCKS == 1 ? 232448 : 233472 / MIN_BLOCKS - 1024;  // of one CTA
   static_assert(TILE % 64 == 0 && TPB % 32 == 0 && TPB > TILE, "strips, a thread per halo element");
-  static_assert(bytes(kMonoMaxJ, false) <= 232448, "shared memory of one CTA");
+  static_assert(bytes(kMonoMaxJ, false) <= LIMIT, "the largest spectrum without fraction tables fits");
 };
 
 // a value that is the same in all lanes, marked so for the compiler (uniform registers and branches)
