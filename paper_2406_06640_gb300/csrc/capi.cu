@@ -125,6 +125,68 @@ static bool cluster_form(int M, int K, int n, int cluster_slots, int slots) {
   return waves * cost < one * (K + 0.5);
 }
 
+// Pinned words of the plans, 64 to a 4 KB block: pinning memory takes 140 us, as long as half of a small plan's other
+// preparation. A word is given back when its plan is destroyed (its stream synchronised), and a block once it is
+// empty, except for one that the process keeps. Blocks that a device reset has taken are not handed out again.
+class HostWordsPool {
+ public:
+  cudaError_t take(HostWords** out) {
+    std::lock_guard<std::mutex> lock(mutex_);
+    for (Block& b : blocks_)
+      if (b.used != ~0ull && pinned(b.words)) return *out = b.take(), cudaSuccess;
+    void* q = nullptr;
+    const cudaError_t e = cudaHostAlloc(&q, 64 * sizeof(Word), cudaHostAllocPortable | cudaHostAllocMapped);
+    if (e != cudaSuccess) return e;
+    blocks_.push_back(Block{static_cast<Word*>(q), 0});
+    *out = blocks_.back().take();
+    return cudaSuccess;
+  }
+  void give(HostWords* w) {
+    std::lock_guard<std::mutex> lock(mutex_);
+    const Word* at = reinterpret_cast<const Word*>(w);
+    bool spare = false;  // another block has a free word
+    for (size_t i = 0; i < blocks_.size(); ++i)
+      if (at < blocks_[i].words || at >= blocks_[i].words + 64) spare |= blocks_[i].used != ~0ull;
+    for (size_t i = 0; i < blocks_.size(); ++i) {
+      Block& b = blocks_[i];
+      if (at < b.words || at >= b.words + 64) continue;
+      b.used &= ~(1ull << (at - b.words));
+      if (b.used == 0 && spare) {
+        cudaFreeHost(b.words);
+        blocks_.erase(blocks_.begin() + (long)i);
+      }
+      return;
+    }
+  }
+
+ private:
+  struct alignas(64) Word {
+    HostWords w;
+  };
+  struct Block {
+    Word* words;
+    unsigned long long used;  // bit per word
+    HostWords* take() {
+      int i = 0;
+      while (used >> i & 1) ++i;
+      used |= 1ull << i;
+      return new (&words[i].w) HostWords{};
+    }
+  };
+  static bool pinned(const void* p) {
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) == cudaSuccess) return at.type == cudaMemoryTypeHost;
+    cudaGetLastError();
+    return false;
+  }
+  std::mutex mutex_;
+  std::vector<Block> blocks_;
+};
+static HostWordsPool& host_words() {
+  static HostWordsPool* pool = new HostWordsPool;  // outlives every plan
+  return *pool;
+}
+
 struct ptycho_plan_s {
   ptycho_params p{};
   std::vector<int32_t> windows;
@@ -268,7 +330,7 @@ struct ptycho_plan_s {
     if (origin) cudaStreamDestroy(origin);
     for (ptycho_plan_s* m : members) delete m;
     for (void* q : allocs) cudaFree(q);
-    if (host) cudaFreeHost(const_cast<HostWords*>(host));
+    if (host) host_words().give(host);
     for (cudaEvent_t e : ev) cudaEventDestroy(e);
   }
   bool in_window(long long t) const {
@@ -438,12 +500,6 @@ static ptycho_status build_plan(ptycho_plan_s* pl, const float* intensities, con
   const int M = p.M, K = p.K, N = p.N;
   const size_t MM = (size_t)M * M;
   cudaStream_t s = pl->stream;
-  if (!pl->host) {
-    void* q = nullptr;
-    PT_CUDA(cudaHostAlloc(&q, sizeof(HostWords), cudaHostAllocPortable | cudaHostAllocMapped), "alloc host words");
-    pl->host = new (q) HostWords{};
-  }
-
   // ---- positions
   pl->h_pos.resize(N);
   if (is_device_pointer(positions)) {
@@ -530,6 +586,8 @@ static ptycho_status build_plan(ptycho_plan_s* pl, const float* intensities, con
   double h_sums[3];
   PT_CUDA(cudaMemcpyAsync(h_sums, d_sums, sizeof(h_sums), cudaMemcpyDeviceToHost, s), "copy sums");
   PT_CUDA(cudaStreamSynchronize(s), "plan sync");
+  // (pinning may wait for the device: not before the allocations above, which run beside it)
+  PT_CUDA(host_words().take(&pl->host), "alloc host words");
   if (h_sums[2] >= 1e30) return fail(PTYCHO_ENUMERIC, "intensities contain non-finite values");
   if (h_sums[2] > 0) return fail(PTYCHO_EINVAL, "intensities contain negative values");
   if (!(h_sums[1] > 0)) return fail(PTYCHO_EINVAL, "intensities are all zero");
@@ -590,9 +648,10 @@ static ptycho_status build_plan(ptycho_plan_s* pl, const float* intensities, con
   int4* d_list;
   PT_CUDA(pl->alloc(&d_start, start.size()), "alloc tile lists");
   PT_CUDA(pl->alloc(&d_list, flat.size()), "alloc tile lists");
-  PT_CUDA(h2d(pl->stream, d_start, start.data(), sizeof(int) * start.size()), "copy tiles");
+  // (on the plan's stream; the lists live until the synchronisation at the end)
+  PT_CUDA(cudaMemcpyAsync(d_start, start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice, s), "copy tiles");
   if (!flat.empty())
-    PT_CUDA(h2d(pl->stream, d_list, flat.data(), sizeof(int4) * flat.size()), "copy tiles");
+    PT_CUDA(cudaMemcpyAsync(d_list, flat.data(), sizeof(int4) * flat.size(), cudaMemcpyHostToDevice, s), "copy tiles");
   pl->d_starts = d_start;
   if (p.engine == PTYCHO_ENGINE_DM) {
     PT_CUDA(pl->alloc(&pl->d_psi, (size_t)N * K * MM), "alloc exit-wave state");
