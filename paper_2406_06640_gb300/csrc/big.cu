@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(BigShape<BL>::LINES * BT, BL == 256 ? (OP < 2 
 // R to its own buffer; the next pass applies Psi' = R Psi as it loads W. Each blur keeps a window of samples
 // in registers for eight outputs (blur_strip), lanes along the other axis of an odd-stride buffer.
 template <int BL>
-constexpr int kModTpb = BL == 256 ? 256 : 512;  // two CTAs fit an SM at 512 columns, four at 256
+constexpr int kModTpb = BL == 256 ? 256 : 512;  // CTAs on an SM: KH = 5, four at 256 columns and two at 512; KH = 15, two and one
 
 template <int BL, int KH>
 __global__ void __launch_bounds__(kModTpb<BL>) k_big_modulus(const BigArgs b) {

@@ -1055,22 +1055,8 @@ static ptycho_status enqueue_update(ptycho_plan_s* pl, void* object, void* probe
   ua.P = static_cast<float2*>(probe);
   ca.O = static_cast<float2*>(object);
   ua.update_probe = t >= pl->p.probe_update_start;
-  if (pl->d_psi) {
-    // pc-DM: the complex constraint acts between the object and the probe step, and the states
-    // move with their boxes by P (O constrained - O)
-    const bool win = pl->in_window(t);
-    PT_CUDA(launch_update_object(ua, win ? &ca : nullptr, pl->big, s), "update launch");
-    ua.dm_obj_prev = nullptr;
-    if (win) {
-      PT_CUDA(cudaMemcpyAsync(pl->d_obj_prev, ua.O, (size_t)pl->p.obj_h * pl->p.obj_w * sizeof(float2),
-                              cudaMemcpyDeviceToDevice, s),
-              "object copy");
-      PT_CUDA(launch_constraint(ca, false, s), "constraint launch");
-      ua.dm_obj_prev = pl->d_obj_prev;
-    }
-    PT_CUDA(launch_update_probe_dm(ua, s), "update launch");
-    return PTYCHO_OK;
-  }
+  // (pc-DM members are not queued.) Object and probe steps are a launch each: callers count on 1 + 4 launches a
+  // member in ptycho_batch_launches
   const bool win = pl->in_window(t);
   PT_CUDA(launch_update(ua, win ? &ca : nullptr, true, false, s), "update launch");
   if (win) PT_CUDA(launch_constraint(ca, false, s), "constraint launch");

@@ -6,8 +6,8 @@
 // Krylov subspace of Eq. 13.
 //
 // All k steps run on chip: the search direction p (with a one-pixel zero border, so samples outside
-// the grid read zeros) and the residual r live in shared memory, x and the step's product vector in
-// registers. C^T r runs separably per wavelength, r S_j then S_j^T (.), with the coordinate formula of
+// the grid read zeros) and the residual r live in shared memory, the step's product vector in registers,
+// x in registers or (k_mono_walk) tensor memory. C^T r runs separably per wavelength, r S_j then S_j^T (.), with the coordinate formula of
 // C, so the GPU's C^T is exactly the transpose of its C. Step sizes and norms are FP64 block
 // reductions in a fixed order (bitwise reproducible). Two forms:
 //   k_mono_walk  M = 64, 128 (one CTA per pattern) and 256 (a cluster of four): threads walk strips of

@@ -27,7 +27,7 @@
 // slot + slots, ... and owns partial `slot`, so every sum is taken in a fixed order and the
 // iteration is bitwise reproducible.
 //
-// Storage per CTA (M = 128): the FFT exchange buffer (146 KB of shared memory; the blur's
+// Storage per CTA (M = 128): the FFT exchange buffer (132 KB of shared memory; the blur's
 // intermediate aliases it), S and then R (66 KB), twiddles and taps; in tensor memory, per
 // thread, its 32 object-box values and its 32 contribution accumulators (512 columns). Probe
 // modes and partials are read from L2.
