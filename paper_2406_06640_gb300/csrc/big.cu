@@ -213,10 +213,14 @@ __global__ void __launch_bounds__(BigShape<BL>::LINES * BT, BL == 256 ? (OP < 2 
 // R to its own buffer; the next pass applies Psi' = R Psi as it loads W. Each blur keeps a window of samples
 // in registers for eight outputs (blur_strip), lanes along the other axis of an odd-stride buffer.
 template <int BL>
-constexpr int kModTpb = BL == 256 ? 256 : 512;  // CTAs on an SM: KH = 5, four at 256 columns and two at 512; KH = 15, two and one
+constexpr int kModTpb = BL == 256 ? 256 : 512;
+// CTAs that the shared memory lets on an SM, asked for in registers as well (KH = 5 at 512 columns with 79 registers
+// and one CTA instead of 64 and two: 49 positions of 512^2, two modes, 886 against 812 us an iteration)
+template <int BL, int KH>
+constexpr int kModCtas = (BL == 256 ? 2 : 1) * (KH == 5 ? 2 : 1);
 
 template <int BL, int KH>
-__global__ void __launch_bounds__(kModTpb<BL>) k_big_modulus(const BigArgs b) {
+__global__ void __launch_bounds__(kModTpb<BL>, kModCtas<BL, KH>) k_big_modulus(const BigArgs b) {
   constexpr int TPB = kModTpb<BL>;
   constexpr int HR = RB + 2 * KH;  // rows held
   constexpr int LD = BL + 1, NB = 8;
